@@ -259,7 +259,7 @@ def prepare(case, seed):
 
 
 def _replay_locus(L):
-    return (3 * (L - 1)) // 4 if L > 4 else L - 1
+    return (5 * (L - 1)) // 8  # between the snapshots at 1/2 and 3/4 of the region
 
 
 def run(s):
@@ -276,17 +276,17 @@ def run(s):
         ls.ls_table_read(s.fwd, s.alpha, s.logf)
         ls.ls_table_read(s.bck, s.beta, s.logg)
         ls.ls_distance(s.ctx, s.fwd, s.bck, s.d)
-        return s.alpha, s.logf, s.beta, s.logg, s.d
+        return s.alpha, s.logf.float(), s.beta, s.logg.float(), s.d  # log scales: sums of FP32 logarithms
     if kind == "ckpt":
         ls.ls_table_reset(s.fwd)
         ck = ls.ls_checkpoints(s.ctx, s.fwd, 0, case["L"] - 1, ls.LS_CKPT_F16 if case["f16"] else ls.LS_CKPT_F32)
         ls.ls_ckpt_replay(s.ctx, ck, s.fwd, _replay_locus(case["L"]))
         ls.ls_table_read(s.fwd, s.alpha, s.logf)
         ls.ls_ckpt_destroy(ck)
-        return s.alpha, s.logf
+        return s.alpha, s.logf.float()
     if kind == "grad":
         rc, pac, dmu, drho = ls.ls_pac_grad(s.ctx, s.groups, case["K"])
-        return pac, dmu, drho
+        return pac, dmu, drho.astype(np.float32)  # expectations under the FP32 recursions
     if kind == "propose":
         ls.ls_propose(s.ctx, case["C"], case["K"], s.net, s.idx)
         return s.idx
