@@ -1,9 +1,23 @@
 // ls_mlp.cuh -- training kernels of the donor-proposal MLP (FP32 master weights).
 //
 // Network: 8 inputs (7 window match fractions, one zero slot) -> 256 -> 256 -> 1, ReLU between
-// layers.  Loss: half mean squared error between the score and the label.  The kernels are plain
-// FP32: a tiled GEMM with optional transposes and accumulation, bias/activation epilogues, column
-// sums and the Adam update.  Inference uses the BF16 MMA kernel of ls_propose.cuh.
+// layers.  Loss: half mean squared error between the score and the label.  FP32 throughout; the
+// column sums behind the bias gradients, the loss and the sums over blocks are double or
+// two-float sums.
+//
+// One gradient is three launches:
+//   mlp_rows_kernel    tiles of 64 rows: both layers forward, the loss, dZ2, dH1 = dZ2 W2^T and the
+//                      gradients of W1, b1, b2, w3, b3 (one partial per CTA); only H1 and dZ2 go to memory
+//   mlp_dw2_kernel     H1^T dZ2 in 128 x 128 tiles, split over the rows
+//   mlp_update_kernel  the partials' sums in a fixed order, and the Adam update or the gradient itself
+// What bounds them is the FP32 pipe (3 x 2 x 65536 FLOP per row): packed FFMA2 on an 8 x 8 tile of
+// outputs per thread, both operands from shared memory.  64 rows per CTA (96 KB, two CTAs per SM) keep
+// every SM busy from 9728 rows on and hold a whole row of the hidden layers, so nothing but H1 and dZ2
+// is written between the layers.
+// Twenty training steps of 16384 rows: 195.7 -> 4.2 ms (before: naive 16 x 16 GEMM tiles, one thread
+// per column sum, twelve launches, seven allocations and a synchronisation a step).
+//
+// Inference uses the BF16 MMA kernel of ls_mlp_tc.cuh.
 #pragma once
 
 #include <cstdint>
@@ -22,108 +36,426 @@ constexpr int kOffW3 = kOffB2 + 256;
 constexpr int kOffB3 = kOffW3 + 256;
 constexpr int kMlpParams = kOffB3 + 1;
 
-// C[M][N] = beta * C + sum_k A(m, k) B(k, n), A(m, k) = ta ? A[k*lda + m] : A[m*lda + k],
-// B(k, n) = tb ? B[n*ldb + k] : B[k*ldb + n].  16 x 16 tiles, 256 threads.
-__global__ void gemm_f32_kernel(int M, int N, int K, const float* __restrict__ A, int lda, int ta,
-                                const float* __restrict__ B, int ldb, int tb, float* __restrict__ Cm, int ldc,
-                                float beta) {
-  __shared__ float As[16][17], Bs[16][17];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int m = blockIdx.y * 16 + ty, n = blockIdx.x * 16 + tx;
-  float acc = 0.0f;
-  for (int k0 = 0; k0 < K; k0 += 16) {
-    {
-      const int mm = blockIdx.y * 16 + ty, kk = k0 + tx;
-      As[ty][tx] = (mm < M && kk < K) ? (ta ? A[(size_t)kk * lda + mm] : A[(size_t)mm * lda + kk]) : 0.0f;
-      const int kb = k0 + ty, nn = blockIdx.x * 16 + tx;
-      Bs[ty][tx] = (kb < K && nn < N) ? (tb ? B[(size_t)nn * ldb + kb] : B[(size_t)kb * ldb + nn]) : 0.0f;
+constexpr int kTrRows = 64;      // rows per tile of mlp_rows_kernel
+constexpr int kTrThreads = 256;  // 8 warps: warp w holds rows 8w..8w+7, lane q columns 4q.. and 128 + 4q..
+constexpr int kTrK = 16;         // weight rows per staged chunk
+// dynamic shared memory: hidden tile [64][256], two weight chunks [16][256]
+constexpr int kTrSmem = (kTrRows * 256 + 2 * kTrK * 256) * 4;
+// a CTA's partial: dW1 [8][256], then [256] each: db1 (sum, error), db2 (sum, error), dw3
+constexpr int kTrPart = 256 * (kMlpIn + 5);
+constexpr int kDwTile = 128, kDwStages = 3;  // mlp_dw2_kernel
+constexpr int kDwSmem = kDwStages * 2 * kTrK * kDwTile * 4;
+
+__host__ __device__ inline uint64_t splitmix_at(uint64_t seed, uint64_t k) {  // k-th output (k >= 1) of the stream
+  uint64_t z = seed + k * 0x9e3779b97f4a7c15ull;
+  z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ull;
+  z = (z ^ (z >> 27)) * 0x94d049bb133111ebull;
+  return z ^ (z >> 31);
+}
+
+struct MlpBatch {
+  const float* X;    // [n_src][8]
+  const float* y;    // [n_src]
+  long long n_src;
+  int B;             // rows of the batch
+  int drawn;         // 1: row r of the batch is splitmix_at(seed, first + r + 1) % n_src, 0: row r
+  uint64_t seed, first;
+  const float* p;    // parameters
+  const float* w2t;  // [256][256] W2 transposed
+  float* H1;         // [B][256]
+  float* dZ2;        // [B][256]
+  float* part;       // [grid][kTrPart]
+  double* partd;     // [grid][2]: sums of (s - y)^2 / 2 and of ds
+};
+
+__device__ __forceinline__ void mlp_cp16(void* dst, const void* src, bool valid) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
+               "r"(valid ? 16 : 0)
+               : "memory");
+}
+__device__ __forceinline__ void mlp_cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int K>
+__device__ __forceinline__ void mlp_cp_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(K) : "memory");
+}
+// (s, e) += v with the exact error of the addition kept in e
+__device__ __forceinline__ void two_sum(float& s, float& e, float v) {
+  const float t = __fadd_rn(s, v), b = __fsub_rn(t, s);
+  e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(v, b)));
+  s = t;
+}
+
+// acc[r][.] += A[8 warp + r][k] Bg[k][columns of the lane], k < 256: A in shared memory, Bg [256][256]
+// in global memory staged through the two chunks at Wc.  Starts and ends with a CTA barrier behind it.
+__device__ __forceinline__ void mlp_tile_gemm(const float* A, const float* __restrict__ Bg, float* Wc, float2 (&acc)[8][4]) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  auto stage = [&](int c) {
+    float* d = Wc + (c & 1) * kTrK * 256;
+#pragma unroll
+    for (int i = 0; i < kTrK * 64 / kTrThreads; ++i) {
+      const int e = 4 * (tid + i * kTrThreads);
+      mlp_cp16(d + e, Bg + (size_t)c * kTrK * 256 + e, true);
+    }
+    mlp_cp_commit();
+  };
+#pragma unroll
+  for (int r = 0; r < 8; ++r)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[r][j] = make_float2(0.f, 0.f);
+  stage(0);
+#pragma unroll 1
+  for (int c = 0; c < 256 / kTrK; ++c) {
+    mlp_cp_wait<0>();
+    __syncthreads();  // chunk c is complete, and everyone is done with the chunk the next copies overwrite
+    if (c + 1 < 256 / kTrK) stage(c + 1);
+    const float* b = Wc + (c & 1) * kTrK * 256 + 4 * lane;
+    const float* a = A + (8 * warp) * 256 + c * kTrK;
+#pragma unroll
+    for (int k = 0; k < kTrK; k += 2) {
+      float2 av[8];
+#pragma unroll
+      for (int r = 0; r < 8; ++r) av[r] = *reinterpret_cast<const float2*>(a + r * 256 + k);
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const float4 b0 = *reinterpret_cast<const float4*>(b + (k + q) * 256);
+        const float4 b1 = *reinterpret_cast<const float4*>(b + (k + q) * 256 + 128);
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+          const float v = q ? av[r].y : av[r].x;
+          const float2 vv = make_float2(v, v);
+          acc[r][0] = __ffma2_rn(vv, make_float2(b0.x, b0.y), acc[r][0]);
+          acc[r][1] = __ffma2_rn(vv, make_float2(b0.z, b0.w), acc[r][1]);
+          acc[r][2] = __ffma2_rn(vv, make_float2(b1.x, b1.y), acc[r][2]);
+          acc[r][3] = __ffma2_rn(vv, make_float2(b1.z, b1.w), acc[r][3]);
+        }
+      }
+    }
+  }
+  __syncthreads();
+}
+
+__global__ void __launch_bounds__(kTrThreads, 2) mlp_rows_kernel(const MlpBatch m) {
+  extern __shared__ __align__(16) float tr_smem[];
+  float* A = tr_smem;                  // [64][256]: H1, then dZ2
+  float* Wc = A + kTrRows * 256;       // weight chunks; between the products, scratch of the column sums
+  __shared__ float Xs[kTrRows][kMlpIn];
+  __shared__ float ys[kTrRows];
+  __shared__ double redd[8][2];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int row0 = 8 * warp;
+  auto col = [&](int j) { return (j >> 2) * 128 + 4 * lane + (j & 3); };  // j-th of the lane's 8 columns
+  const float* p = m.p;
+  float* part = m.part + (size_t)blockIdx.x * kTrPart;
+  double lsum = 0.0, dsum = 0.0;  // lanes < 8: row row0 + lane of every tile
+  bool first = true;
+  for (long long r0 = (long long)blockIdx.x * kTrRows; r0 < m.B; r0 += (long long)gridDim.x * kTrRows, first = false) {
+    const int rows = (int)min((long long)kTrRows, m.B - r0);
+    for (int e = tid; e < kTrRows * kMlpIn; e += kTrThreads) {
+      const int r = e / kMlpIn, k = e % kMlpIn;
+      long long src = r0 + r;
+      if (m.drawn) src = (long long)(splitmix_at(m.seed, m.first + (uint64_t)src + 1) % (uint64_t)m.n_src);
+      Xs[r][k] = r < rows ? m.X[src * kMlpIn + k] : 0.0f;
+      if (k == 0) ys[r] = r < rows ? m.y[src] : 0.0f;
     }
     __syncthreads();
+    {  // layer 1: thread = hidden unit
+      float w1[kMlpIn];
 #pragma unroll
-    for (int k = 0; k < 16; ++k) acc = fmaf(As[ty][k], Bs[k][tx], acc);
+      for (int k = 0; k < kMlpIn; ++k) w1[k] = p[kOffW1 + k * 256 + tid];
+      const float b1 = p[kOffB1 + tid];
+#pragma unroll 4
+      for (int r = 0; r < kTrRows; ++r) {
+        float z = 0.0f;
+#pragma unroll
+        for (int k = 0; k < kMlpIn; ++k) z = fmaf(Xs[r][k], w1[k], z);
+        const float h = fmaxf(z + b1, 0.0f);
+        A[r * 256 + tid] = h;
+        if (r < rows) m.H1[(size_t)(r0 + r) * 256 + tid] = h;
+      }
+    }
     __syncthreads();
+    uint32_t live[2] = {0u, 0u};  // H1 > 0 at this thread's outputs of the last product, bit 4 r + j
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const float4 v = *reinterpret_cast<const float4*>(A + (row0 + r) * 256 + 128 * h + 4 * lane);
+        live[h] |= ((v.x > 0.f ? 1u : 0u) | (v.y > 0.f ? 2u : 0u) | (v.z > 0.f ? 4u : 0u) | (v.w > 0.f ? 8u : 0u)) << (4 * r);
+      }
+    float2 acc[8][4];
+    mlp_tile_gemm(A, p + kOffW2, Wc, acc);  // Z2 before its bias
+    {
+      // score, loss and ds of the warp's rows, dZ2 into A; column sums of dZ2 (db2) and of ds H2 (dw3)
+      const float b3 = p[kOffB3];
+      float ds[8];
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        float s = 0.0f;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          float2& z2 = acc[r][j >> 1];
+          float& z = (j & 1) ? z2.y : z2.x;
+          z += p[kOffB2 + col(j)];
+          s = fmaf(fmaxf(z, 0.0f), p[kOffW3 + col(j)], s);
+        }
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+        const float d = (s + b3) - ys[row0 + r];
+        ds[r] = row0 + r < rows ? d / (float)m.B : 0.0f;
+        if (lane == r && row0 + r < rows) {
+          lsum += 0.5 * (double)d * (double)d;
+          dsum += (double)ds[r];
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const float w3 = p[kOffW3 + col(j)];
+        float g3 = 0.0f, gs = 0.0f, ge = 0.0f;
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+          float& z = (j & 1) ? acc[r][j >> 1].y : acc[r][j >> 1].x;
+          g3 = fmaf(ds[r], fmaxf(z, 0.0f), g3);
+          z = z > 0.0f ? ds[r] * w3 : 0.0f;
+          two_sum(gs, ge, z);
+        }
+        Wc[warp * 256 + col(j)] = g3;
+        Wc[(8 + warp) * 256 + col(j)] = gs;
+        Wc[(16 + warp) * 256 + col(j)] = ge;
+      }
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const float4 v = make_float4(acc[r][2 * h].x, acc[r][2 * h].y, acc[r][2 * h + 1].x, acc[r][2 * h + 1].y);
+          *reinterpret_cast<float4*>(A + (row0 + r) * 256 + 128 * h + 4 * lane) = v;
+          if (row0 + r < rows) *reinterpret_cast<float4*>(m.dZ2 + (size_t)(r0 + row0 + r) * 256 + 128 * h + 4 * lane) = v;
+        }
+      __syncthreads();
+      float* o = part + kMlpIn * 256 + tid;  // db1 (2 x 256), db2 (2 x 256), dw3 (256)
+      float g3 = first ? 0.0f : o[4 * 256], gs = first ? 0.0f : o[2 * 256], ge = first ? 0.0f : o[3 * 256];
+#pragma unroll
+      for (int w = 0; w < 8; ++w) {
+        g3 += Wc[w * 256 + tid];
+        two_sum(gs, ge, Wc[(8 + w) * 256 + tid]);
+        ge += Wc[(16 + w) * 256 + tid];
+      }
+      o[4 * 256] = g3;
+      o[2 * 256] = gs;
+      o[3 * 256] = ge;
+      __syncthreads();
+    }
+    mlp_tile_gemm(A, m.w2t, Wc, acc);  // dH1
+    {
+      // dZ1; its column sums (db1) and products with the inputs (dW1) meet over the warps in A and Wc
+      float* S = A;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        float gs = 0.0f, ge = 0.0f, gw[kMlpIn];
+#pragma unroll
+        for (int k = 0; k < kMlpIn; ++k) gw[k] = 0.0f;
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+          const float a = (j & 1) ? acc[r][j >> 1].y : acc[r][j >> 1].x;
+          const float z = (live[j >> 2] >> (4 * r + (j & 3))) & 1u ? a : 0.0f;
+          two_sum(gs, ge, z);
+#pragma unroll
+          for (int k = 0; k < kMlpIn; ++k) gw[k] = fmaf(Xs[row0 + r][k], z, gw[k]);
+        }
+#pragma unroll
+        for (int k = 0; k < kMlpIn; ++k) S[(8 * k + warp) * 256 + col(j)] = gw[k];
+        S[(64 + warp) * 256 + col(j)] = gs;
+        S[(72 + warp) * 256 + col(j)] = ge;
+      }
+      __syncthreads();
+      float* o = part + tid;
+#pragma unroll
+      for (int k = 0; k < kMlpIn; ++k) {
+        float g = first ? 0.0f : o[k * 256];
+#pragma unroll
+        for (int w = 0; w < 8; ++w) g += S[(8 * k + w) * 256 + tid];
+        o[k * 256] = g;
+      }
+      float gs = first ? 0.0f : o[kMlpIn * 256], ge = first ? 0.0f : o[(kMlpIn + 1) * 256];
+#pragma unroll
+      for (int w = 0; w < 8; ++w) {
+        two_sum(gs, ge, S[(64 + w) * 256 + tid]);
+        ge += S[(72 + w) * 256 + tid];
+      }
+      o[kMlpIn * 256] = gs;
+      o[(kMlpIn + 1) * 256] = ge;
+      __syncthreads();  // before the next tile overwrites Xs and A
+    }
   }
-  if (m < M && n < N) {
-    float* c = Cm + (size_t)m * ldc + n;
-    *c = beta == 0.0f ? acc : fmaf(beta, *c, acc);
+#pragma unroll
+  for (int off = 4; off > 0; off >>= 1) {
+    lsum += __shfl_xor_sync(0xffffffffu, lsum, off);
+    dsum += __shfl_xor_sync(0xffffffffu, dsum, off);
   }
-}
-
-// Z[r][c] += b[c]; H = relu(Z) (H may alias nothing; Z keeps the pre-activation)
-__global__ void bias_relu_kernel(float* __restrict__ Z, const float* __restrict__ b, int rows, int cols,
-                                 float* __restrict__ H) {
-  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= (long long)rows * cols) return;
-  const float z = Z[e] + b[e % cols];
-  Z[e] = z;
-  if (H) H[e] = fmaxf(z, 0.0f);
-}
-
-// dZ = dH * (Z > 0), in place on dH
-__global__ void relu_back_kernel(float* __restrict__ dH, const float* __restrict__ Z, long long n) {
-  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e < n && !(Z[e] > 0.0f)) dH[e] = 0.0f;
-}
-
-// s = H2 w3 + b3 per row; ds = (s - y) / n; loss terms (s - y)^2 / 2 summed into loss (FP64 atomics
-// are avoided: one partial per block)
-__global__ void head_kernel(const float* __restrict__ H2, const float* __restrict__ w3, const float* __restrict__ b3,
-                            const float* __restrict__ y, int n, float* __restrict__ ds, double* __restrict__ part) {
-  __shared__ double red[256];
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  double l = 0.0;
-  if (r < n) {
-    float s = b3[0];
-    for (int c = 0; c < 256; ++c) s = fmaf(H2[(size_t)r * 256 + c], w3[c], s);
-    const float d = s - y[r];
-    ds[r] = d / (float)n;
-    l = 0.5 * (double)d * (double)d;
+  if (lane == 0) {
+    redd[warp][0] = lsum;
+    redd[warp][1] = dsum;
   }
-  red[threadIdx.x] = l;
   __syncthreads();
-  for (int h = blockDim.x / 2; h > 0; h >>= 1) {
-    if ((int)threadIdx.x < h) red[threadIdx.x] += red[threadIdx.x + h];
+  if (tid < 2) {
+    double t = 0.0;
+    for (int w = 0; w < 8; ++w) t += redd[w][tid];
+    m.partd[2 * blockIdx.x + tid] = t;
+  }
+}
+
+// Partial dW2 of the rows [blockIdx.y rows, ..): out[blockIdx.y][k][n] = sum_r H1[r][k] dZ2[r][n], one
+// 128 x 128 quarter per blockIdx.x.  `rows` is a multiple of kTrK.
+__global__ void __launch_bounds__(256, 2) mlp_dw2_kernel(const float* __restrict__ H1, const float* __restrict__ dZ2, int B,
+                                                         int rows, float* __restrict__ out) {
+  extern __shared__ __align__(16) float dw_smem[];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int k0 = (blockIdx.x >> 1) * kDwTile, n0 = (blockIdx.x & 1) * kDwTile;
+  const int r_begin = blockIdx.y * rows, r_end = min(B, r_begin + rows);
+  const int nchunk = (r_end - r_begin + kTrK - 1) / kTrK;
+  auto stage = [&](int c) {
+    float* a = dw_smem + (c % kDwStages) * 2 * kTrK * kDwTile;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int e = tid + i * 256, r = e >> 5, x = 4 * (e & 31), gr = r_begin + c * kTrK + r;
+      const bool in = gr < r_end;
+      const size_t o = (size_t)(in ? gr : r_begin) * 256 + x;
+      mlp_cp16(a + r * kDwTile + x, H1 + o + k0, in);
+      mlp_cp16(a + (kTrK + r) * kDwTile + x, dZ2 + o + n0, in);
+    }
+  };
+  float2 acc[8][4];
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int c = 0; c < kDwStages - 1; ++c) {
+    if (c < nchunk) stage(c);
+    mlp_cp_commit();
+  }
+  const int ka = 32 * (warp & 3) + 4 * (lane >> 3), nb = 64 * (warp >> 2) + 4 * (lane & 7);
+#pragma unroll 1
+  for (int c = 0; c < nchunk; ++c) {
+    mlp_cp_wait<kDwStages - 2>();
+    __syncthreads();
+    if (c + kDwStages - 1 < nchunk) stage(c + kDwStages - 1);
+    mlp_cp_commit();
+    const float* a = dw_smem + (c % kDwStages) * 2 * kTrK * kDwTile;
+    const float* b = a + kTrK * kDwTile;
+#pragma unroll 4
+    for (int r = 0; r < kTrK; ++r) {
+      const float4 a0 = *reinterpret_cast<const float4*>(a + r * kDwTile + ka);
+      const float4 a1 = *reinterpret_cast<const float4*>(a + r * kDwTile + ka + 16);
+      const float4 b0 = *reinterpret_cast<const float4*>(b + r * kDwTile + nb);
+      const float4 b1 = *reinterpret_cast<const float4*>(b + r * kDwTile + nb + 32);
+      const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const float2 vv = make_float2(av[i], av[i]);
+        acc[i][0] = __ffma2_rn(vv, make_float2(b0.x, b0.y), acc[i][0]);
+        acc[i][1] = __ffma2_rn(vv, make_float2(b0.z, b0.w), acc[i][1]);
+        acc[i][2] = __ffma2_rn(vv, make_float2(b1.x, b1.y), acc[i][2]);
+        acc[i][3] = __ffma2_rn(vv, make_float2(b1.z, b1.w), acc[i][3]);
+      }
+    }
+  }
+  float* o = out + (size_t)blockIdx.y * 65536;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    float* oi = o + (size_t)(k0 + ka + (i & 3) + 16 * (i >> 2)) * 256 + n0 + nb;
+    *reinterpret_cast<float4*>(oi) = make_float4(acc[i][0].x, acc[i][0].y, acc[i][1].x, acc[i][1].y);
+    *reinterpret_cast<float4*>(oi + 32) = make_float4(acc[i][2].x, acc[i][2].y, acc[i][3].x, acc[i][3].y);
+  }
+}
+
+struct MlpUpdate {
+  const float* partw;   // [splits][65536]
+  int splits;
+  const float* part;    // [ctas][kTrPart]
+  const double* partd;  // [ctas][2]
+  int ctas;
+  float* g;             // gradient out (null: Adam update of p instead)
+  double* loss;         // loss sum out (may be null)
+  float *p, *m, *v, *w2t;
+  float lr, b1, b2, c1, c2, eps;
+};
+
+// The gradient of every parameter from the partials, in a fixed order, and its Adam update:
+// m = b1 m + (1-b1) g; v = b2 v + (1-b2) g^2; p -= lr * mhat / (sqrt(vhat) + eps).  Blocks 0..255: W2, a
+// thread per weight; 256..343: 32 parameters of W1, b1, b2 and w3 each (8 threads a parameter, sums in
+// double); the last block: b3 and the loss.
+constexpr int kUpdBlocks = 256 + 11 * 256 / 32 + 1;
+__global__ void __launch_bounds__(256) mlp_update_kernel(const MlpUpdate u) {
+  const int tid = threadIdx.x;
+  auto apply = [&](int e, float gi) {
+    if (u.g) {
+      u.g[e] = gi;
+      return;
+    }
+    const float mi = u.b1 * u.m[e] + (1.0f - u.b1) * gi;
+    const float vi = u.b2 * u.v[e] + (1.0f - u.b2) * gi * gi;
+    u.m[e] = mi;
+    u.v[e] = vi;
+    const float pn = u.p[e] - u.lr * (mi / u.c1) / (sqrtf(vi / u.c2) + u.eps);
+    u.p[e] = pn;
+    if (e >= kOffW2 && e < kOffB2) u.w2t[((e - kOffW2) & 255) * 256 + ((e - kOffW2) >> 8)] = pn;
+  };
+  if (blockIdx.x < 256) {
+    const int e = blockIdx.x * 256 + tid;
+    float g = 0.0f;
+#pragma unroll 8
+    for (int s = 0; s < u.splits; ++s) g += u.partw[(size_t)s * 65536 + e];
+    apply(kOffW2 + e, g);
+    return;
+  }
+  if (blockIdx.x + 1 < gridDim.x) {
+    __shared__ double red[8][33];
+    const int q = (blockIdx.x - 256) * 32 + (tid & 31), sec = q >> 8, c = q & 255;  // sec 0..7 W1, 8 b1, 9 b2, 10 w3
+    const int o0 = (sec < 9 ? sec : sec == 9 ? kMlpIn + 2 : kMlpIn + 4) * 256 + c;
+    const bool pair = sec == 8 || sec == 9;  // (sum, error)
+    double t = 0.0;
+    for (int b = tid >> 5; b < u.ctas; b += 8) {
+      const float* o = u.part + (size_t)b * kTrPart + o0;
+      t += (double)o[0];
+      if (pair) t += (double)o[256];
+    }
+    red[tid >> 5][tid & 31] = t;
+    __syncthreads();
+    if (tid < 32) {
+      t = 0.0;
+      for (int k = 0; k < 8; ++k) t += red[k][tid];
+      apply(sec < 8 ? kOffW1 + q : (sec == 8 ? kOffB1 : sec == 9 ? kOffB2 : kOffW3) + c, (float)t);
+    }
+    return;
+  }
+  __shared__ double rd[256][2];
+  double l = 0.0, d = 0.0;
+  for (int b = tid; b < u.ctas; b += 256) {
+    l += u.partd[2 * b];
+    d += u.partd[2 * b + 1];
+  }
+  rd[tid][0] = l;
+  rd[tid][1] = d;
+  __syncthreads();
+  for (int h = 128; h > 0; h >>= 1) {
+    if (tid < h) {
+      rd[tid][0] += rd[tid + h][0];
+      rd[tid][1] += rd[tid + h][1];
+    }
     __syncthreads();
   }
-  if (threadIdx.x == 0) part[blockIdx.x] = red[0];
+  if (tid == 0) {
+    if (u.loss) *u.loss = rd[0][0];
+    apply(kOffB3, (float)rd[0][1]);
+  }
 }
 
-// dH2[r][c] = ds[r] w3[c]
-__global__ void outer_kernel(const float* __restrict__ ds, const float* __restrict__ w3, int n, float* __restrict__ dH) {
-  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e < (long long)n * 256) dH[e] = ds[e / 256] * w3[e % 256];
-}
-
-// out[c] = sum_r X[r][c] (column sums, fixed order per column), one thread per column
-__global__ void colsum_kernel(const float* __restrict__ X, int rows, int cols, float* __restrict__ out) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= cols) return;
-  double s = 0.0;
-  for (int r = 0; r < rows; ++r) s += X[(size_t)r * cols + c];
-  out[c] = (float)s;
-}
-
-// Adam: m = b1 m + (1-b1) g; v = b2 v + (1-b2) g^2; p -= lr * mhat / (sqrt(vhat) + eps)
-__global__ void adam_kernel(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
-                            float* __restrict__ v, int n, float lr, float b1, float b2, float c1, float c2, float eps) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= n) return;
-  const float gi = g[e];
-  const float mi = b1 * m[e] + (1.0f - b1) * gi;
-  const float vi = b2 * v[e] + (1.0f - b2) * gi * gi;
-  m[e] = mi;
-  v[e] = vi;
-  p[e] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-}
-
-// gather a minibatch: rows sel[r] of X ([n][8]) and y
-__global__ void gather_rows_kernel(const float* __restrict__ X, const float* __restrict__ y, const int* __restrict__ sel,
-                                   int B, float* __restrict__ Xb, float* __restrict__ yb) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= B * kMlpIn) return;
-  const int r = e / kMlpIn, c = e % kMlpIn;
-  Xb[e] = X[(size_t)sel[r] * kMlpIn + c];
-  if (c == 0) yb[r] = y[sel[r]];
+// W2 transposed, for the first gradient of a call
+__global__ void mlp_transpose_kernel(const float* __restrict__ w2, float* __restrict__ w2t) {
+  __shared__ float t[32][33];
+  for (int k = threadIdx.y; k < 32; k += 8) t[k][threadIdx.x] = w2[(blockIdx.y * 32 + k) * 256 + blockIdx.x * 32 + threadIdx.x];
+  __syncthreads();
+  for (int k = threadIdx.y; k < 32; k += 8) w2t[(blockIdx.x * 32 + k) * 256 + blockIdx.y * 32 + threadIdx.x] = t[threadIdx.x][k];
 }
 
 }  // namespace lsk

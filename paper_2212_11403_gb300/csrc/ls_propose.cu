@@ -119,56 +119,50 @@ uint64_t splitmix(uint64_t& s) {
 
 unsigned blocks(long long n, int t = 256) { return (unsigned)((n + t - 1) / t); }
 
-void gemm(cudaStream_t s, int M, int N, int K, const float* A, int lda, int ta, const float* B, int ldb, int tb, float* C,
-          int ldc, float beta) {
-  lsk::gemm_f32_kernel<<<dim3((N + 15) / 16, (M + 15) / 16), 256, 0, s>>>(M, N, K, A, lda, ta, B, ldb, tb, C, ldc, beta);
-}
-
-// forward + backward of a batch (X [B][8], y [B]) into m->g; loss sum into *loss
-int batch_grad(ls_mlp* m, const float* X, const float* y, int B, cudaStream_t s, double* loss) {
-  Bufs b;
-  float *Z1, *H1, *Z2, *H2, *ds, *dH2, *dH1;
-  double* part;
-  const int nb = (int)blocks(B);
-  int rc;
-  if ((rc = b.get(&Z1, (size_t)B * 256)) || (rc = b.get(&H1, (size_t)B * 256)) || (rc = b.get(&Z2, (size_t)B * 256)) ||
-      (rc = b.get(&H2, (size_t)B * 256)) || (rc = b.get(&ds, B)) || (rc = b.get(&dH2, (size_t)B * 256)) ||
-      (rc = b.get(&dH1, (size_t)B * 256)) || (rc = b.get(&part, nb)))
-    return rc;
-  const float* p = m->p;
-  float* g = m->g;
-  const long long n256 = (long long)B * 256;
-  gemm(s, B, 256, lsk::kMlpIn, X, lsk::kMlpIn, 0, p + lsk::kOffW1, 256, 0, Z1, 256, 0.0f);
-  lsk::bias_relu_kernel<<<blocks(n256), 256, 0, s>>>(Z1, p + lsk::kOffB1, B, 256, H1);
-  gemm(s, B, 256, 256, H1, 256, 0, p + lsk::kOffW2, 256, 0, Z2, 256, 0.0f);
-  lsk::bias_relu_kernel<<<blocks(n256), 256, 0, s>>>(Z2, p + lsk::kOffB2, B, 256, H2);
-  lsk::head_kernel<<<nb, 256, 0, s>>>(H2, p + lsk::kOffW3, p + lsk::kOffB3, y, B, ds, part);
-  // output layer
-  gemm(s, 256, 1, B, H2, 256, 1, ds, 1, 0, g + lsk::kOffW3, 1, 0.0f);
-  lsk::colsum_kernel<<<1, 32, 0, s>>>(ds, B, 1, g + lsk::kOffB3);
-  // hidden layer 2
-  lsk::outer_kernel<<<blocks(n256), 256, 0, s>>>(ds, p + lsk::kOffW3, B, dH2);
-  lsk::relu_back_kernel<<<blocks(n256), 256, 0, s>>>(dH2, Z2, n256);
-  gemm(s, 256, 256, B, H1, 256, 1, dH2, 256, 0, g + lsk::kOffW2, 256, 0.0f);
-  lsk::colsum_kernel<<<1, 256, 0, s>>>(dH2, B, 256, g + lsk::kOffB2);
-  // hidden layer 1
-  gemm(s, B, 256, 256, dH2, 256, 0, p + lsk::kOffW2, 256, 1, dH1, 256, 0.0f);
-  lsk::relu_back_kernel<<<blocks(n256), 256, 0, s>>>(dH1, Z1, n256);
-  gemm(s, lsk::kMlpIn, 256, B, X, lsk::kMlpIn, 1, dH1, 256, 0, g + lsk::kOffW1, 256, 0.0f);
-  lsk::colsum_kernel<<<1, 256, 0, s>>>(dH1, B, 256, g + lsk::kOffB1);
-  TRY(cudaGetLastError());
-  if (loss) {
-    std::vector<double> h(nb);
-    TRY(cudaMemcpyAsync(h.data(), part, sizeof(double) * nb, cudaMemcpyDeviceToHost, s));
-    TRY(cudaStreamSynchronize(s));
-    double t = 0.0;
-    for (double v : h) t += v;
-    *loss = t;
-  } else {
-    TRY(cudaStreamSynchronize(s));  // the batch buffers are freed on return
+// Scratch of the gradient of up to B rows and its launches.
+struct GradWork {
+  int ctas = 0, splits = 0, split_rows = 0;
+  float *H1, *dZ2, *part, *partw, *w2t;
+  double *partd, *loss;
+  int setup(const ls_mlp* m, Bufs& b, int B, int nloss, cudaStream_t s) {
+    int nsm = 0, rc;
+    TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, m->device));
+    TRY(cudaFuncSetAttribute(lsk::mlp_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, lsk::kTrSmem));
+    ctas = std::min(2 * nsm, (int)((B + (long long)lsk::kTrRows - 1) / lsk::kTrRows));  // two CTAs per SM
+    // four quarter tiles of dW2 per split, two CTAs per SM, at least 128 rows a split
+    const int most = std::max(1, 2 * nsm / 4);
+    split_rows = std::max(128, (int)((B + (long long)most - 1) / most));
+    split_rows = (split_rows + lsk::kTrK - 1) / lsk::kTrK * lsk::kTrK;
+    splits = (int)((B + (long long)split_rows - 1) / split_rows);
+    if ((rc = b.get(&H1, (size_t)B * 256)) || (rc = b.get(&dZ2, (size_t)B * 256)) ||
+        (rc = b.get(&part, (size_t)ctas * lsk::kTrPart)) || (rc = b.get(&partw, (size_t)splits * 65536)) ||
+        (rc = b.get(&w2t, 65536)) || (rc = b.get(&partd, 2 * (size_t)ctas)) || (rc = b.get(&loss, nloss)))
+      return rc;
+    lsk::mlp_transpose_kernel<<<dim3(8, 8), dim3(32, 8), 0, s>>>(m->p + lsk::kOffW2, w2t);
+    TRY(cudaGetLastError());
+    return LS_OK;
   }
-  return LS_OK;
-}
+  // gradient of the batch (its rows and source in mb), then into u.g or, with u.g null, an Adam update
+  int run(const ls_mlp* m, lsk::MlpBatch mb, lsk::MlpUpdate u, cudaStream_t s) const {
+    mb.p = m->p;
+    mb.w2t = w2t;
+    mb.H1 = H1;
+    mb.dZ2 = dZ2;
+    mb.part = part;
+    mb.partd = partd;
+    lsk::mlp_rows_kernel<<<ctas, lsk::kTrThreads, lsk::kTrSmem, s>>>(mb);
+    lsk::mlp_dw2_kernel<<<dim3(4, splits), 256, lsk::kDwSmem, s>>>(H1, dZ2, mb.B, split_rows, partw);
+    u.partw = partw;
+    u.splits = splits;
+    u.part = part;
+    u.partd = partd;
+    u.ctas = ctas;
+    u.w2t = w2t;
+    lsk::mlp_update_kernel<<<lsk::kUpdBlocks, 256, 0, s>>>(u);
+    TRY(cudaGetLastError());
+    return LS_OK;
+  }
+};
 
 }  // namespace
 
@@ -262,9 +256,23 @@ int ls_mlp_forward(const ls_mlp* m, const float* X, int64_t n, float* scores, ls
 int ls_mlp_grad(ls_mlp* m, const float* X, const float* y, int32_t n, float* grad, double* loss, ls_stream_t stream) {
   if (!m || !X || !y || n < 1) return fail(LS_ERR_ARG, "bad arguments");
   cudaStream_t s = (cudaStream_t)stream;
-  int rc = batch_grad(m, X, y, n, s, loss);
+  Bufs b;
+  GradWork gw;
+  int rc = gw.setup(m, b, n, 1, s);
   if (rc) return rc;
-  if (loss) *loss /= n;
+  lsk::MlpBatch mb = {};
+  mb.X = X;
+  mb.y = y;
+  mb.n_src = n;
+  mb.B = n;
+  lsk::MlpUpdate u = {};
+  u.g = m->g;
+  u.loss = gw.loss;
+  if ((rc = gw.run(m, mb, u, s))) return rc;
+  double l = 0.0;
+  TRY(cudaMemcpyAsync(&l, gw.loss, sizeof(double), cudaMemcpyDeviceToHost, s));
+  TRY(cudaStreamSynchronize(s));
+  if (loss) *loss = l / n;
   if (grad) TRY(cudaMemcpy(grad, m->g, sizeof(float) * lsk::kMlpParams, cudaMemcpyDeviceToHost));
   return LS_OK;
 }
@@ -274,33 +282,40 @@ int ls_mlp_train(ls_mlp* m, const float* X, const float* y, int64_t n, int32_t s
   if (!m || !X || !y || n < 1 || steps < 0 || batch < 1) return fail(LS_ERR_ARG, "bad arguments");
   cudaStream_t s = (cudaStream_t)stream;
   Bufs b;
-  float *Xb, *yb;
-  int* sel;
-  int rc;
-  if ((rc = b.get(&Xb, (size_t)batch * lsk::kMlpIn)) || (rc = b.get(&yb, batch)) || (rc = b.get(&sel, batch))) return rc;
-  std::vector<int> hs(batch);
-  uint64_t st = seed;
-  double tail = 0.0;
-  int ntail = 0;
+  GradWork gw;
+  const int ntail = std::min(steps, std::max(1, steps / 10));  // the steps whose losses are averaged
+  int rc = gw.setup(m, b, batch, ntail, s);
+  if (rc) return rc;
+  lsk::MlpBatch mb = {};
+  mb.X = X;
+  mb.y = y;
+  mb.n_src = n;
+  mb.B = batch;
+  mb.drawn = 1;
+  mb.seed = seed;
   for (int it = 0; it < steps; ++it) {
-    for (int r = 0; r < batch; ++r) hs[r] = (int)(splitmix(st) % (uint64_t)n);
-    TRY(cudaMemcpyAsync(sel, hs.data(), sizeof(int) * batch, cudaMemcpyHostToDevice, s));
-    lsk::gather_rows_kernel<<<blocks((long long)batch * lsk::kMlpIn), 256, 0, s>>>(X, y, sel, batch, Xb, yb);
-    const bool want = it >= steps - std::max(1, steps / 10);
-    double l = 0.0;
-    if ((rc = batch_grad(m, Xb, yb, batch, s, want ? &l : nullptr))) return rc;
-    if (want) {
-      tail += l / batch;
-      ++ntail;
-    }
+    mb.first = (uint64_t)it * (uint64_t)batch;
     ++m->t;
-    const float c1 = 1.0f - std::pow(0.9f, (float)m->t), c2 = 1.0f - std::pow(0.999f, (float)m->t);
-    lsk::adam_kernel<<<blocks(lsk::kMlpParams), 256, 0, s>>>(m->p, m->g, m->m, m->v, lsk::kMlpParams, lr, 0.9f, 0.999f, c1,
-                                                              c2, 1e-8f);
-    TRY(cudaGetLastError());
+    lsk::MlpUpdate u = {};
+    const int k = it - (steps - ntail);
+    u.loss = k >= 0 ? gw.loss + k : nullptr;
+    u.p = m->p;
+    u.m = m->m;
+    u.v = m->v;
+    u.lr = lr;
+    u.b1 = 0.9f;
+    u.b2 = 0.999f;
+    u.c1 = 1.0f - std::pow(0.9f, (float)m->t);
+    u.c2 = 1.0f - std::pow(0.999f, (float)m->t);
+    u.eps = 1e-8f;
+    if ((rc = gw.run(m, mb, u, s))) return rc;
   }
+  std::vector<double> tail(std::max(ntail, 1), 0.0);
+  if (ntail) TRY(cudaMemcpyAsync(tail.data(), gw.loss, sizeof(double) * ntail, cudaMemcpyDeviceToHost, s));
   TRY(cudaStreamSynchronize(s));
-  if (loss_out) *loss_out = ntail ? tail / ntail : 0.0;
+  double t = 0.0;
+  for (int k = 0; k < ntail; ++k) t += tail[k] / batch;
+  if (loss_out) *loss_out = ntail ? t / ntail : 0.0;
   return refresh(m);
 }
 
