@@ -356,7 +356,7 @@ int ensure(PropWork& pw, int w, cudaStream_t s) {
   return LS_OK;
 }
 
-int stage1(PropWork& pw, int w, int C, int32_t* cand, long long cstride, __nv_bfloat16* feat, float* feat32,
+int stage1(PropWork& pw, int w, int C, int32_t* cand, size_t cstride, __nv_bfloat16* feat, float* feat32,
            cudaStream_t s) {
   for (int d = -3; d <= 3; ++d) {
     const int ww = std::min(std::max(w + d, 0), pw.Wn - 1);
@@ -372,8 +372,19 @@ int stage1(PropWork& pw, int w, int C, int32_t* cand, long long cstride, __nv_bf
   a.use[0] = w - 1 >= 0;
   a.use[1] = 1;
   a.use[2] = w + 1 < pw.Wn;
-  (void)cstride;
-  lsk::stage1_kernel<<<pw.N, 256, 0, s>>>(a, pw.N, pw.Np, C, cand, feat, feat32);
+  lsk::stage1_kernel<<<pw.N, 256, 0, s>>>(a, pw.N, pw.Np, C, cand, cstride, feat, feat32);
+  TRY(cudaGetLastError());
+  return LS_OK;
+}
+
+// the K best of C scored candidates per target: C / 32 keys a lane, rounded up to a power of two
+int topk(const int32_t* cand, const float* scores, int N, int C, int K, int Wn, int w, int32_t* idx, cudaStream_t s) {
+  const unsigned grid = blocks(N, 8);
+  if (C <= 128) lsk::topk_kernel<4><<<grid, 256, 0, s>>>(cand, scores, N, C, K, Wn, w, idx);
+  else if (C <= 256) lsk::topk_kernel<8><<<grid, 256, 0, s>>>(cand, scores, N, C, K, Wn, w, idx);
+  else if (C <= 512) lsk::topk_kernel<16><<<grid, 256, 0, s>>>(cand, scores, N, C, K, Wn, w, idx);
+  else if (C <= 1024) lsk::topk_kernel<32><<<grid, 256, 0, s>>>(cand, scores, N, C, K, Wn, w, idx);
+  else lsk::topk_kernel<64><<<grid, 256, 0, s>>>(cand, scores, N, C, K, Wn, w, idx);
   TRY(cudaGetLastError());
   return LS_OK;
 }
@@ -415,21 +426,20 @@ int ls_propose(ls_ctx* ctx, int32_t C, int32_t K, const ls_mlp* mlp, int32_t* id
   int rc = prop_setup(ctx, b, pw, s);
   if (rc) return rc;
   const int N = pw.N, Wn = pw.Wn;
-  const int Ce = mlp ? C : K;
-  int32_t* cand;
+  int32_t* cand = nullptr;
   __nv_bfloat16* feat = nullptr;
   float* scores = nullptr;
-  if ((rc = b.get(&cand, (size_t)N * Ce))) return rc;
-  if (mlp && ((rc = b.get(&feat, (size_t)N * Ce * lsk::kFeat)) || (rc = b.get(&scores, (size_t)N * Ce)))) return rc;
-  int P = 1;
-  while (P < Ce) P <<= 1;
-  // topk needs P * 8 <= 16 KB of dynamic shared memory, within the default limit
+  if (mlp && ((rc = b.get(&cand, (size_t)N * C)) || (rc = b.get(&feat, (size_t)N * C * lsk::kFeat)) ||
+              (rc = b.get(&scores, (size_t)N * C))))
+    return rc;
   for (int w = 0; w < Wn; ++w) {
-    if ((rc = stage1(pw, w, Ce, cand, Ce, feat, nullptr, s))) return rc;
-    if (mlp && (rc = launch_scores(mlp, feat, (long long)N * Ce, scores, ctx->num_sms, s))) return rc;
-    // the K best (by score, or by the stage-1 order when there is no network) in ascending id order
-    lsk::topk_kernel<<<N, 256, P * 8, s>>>(cand, mlp ? scores : nullptr, Ce, K, P, Wn, w, idx_out);
-    TRY(cudaGetLastError());
+    if (!mlp) {  // stage 1's K candidates are the set, already in ascending id order
+      if ((rc = stage1(pw, w, K, idx_out + (size_t)w * K, (size_t)Wn * K, nullptr, nullptr, s))) return rc;
+      continue;
+    }
+    if ((rc = stage1(pw, w, C, cand, C, feat, nullptr, s))) return rc;
+    if ((rc = launch_scores(mlp, feat, (long long)N * C, scores, ctx->num_sms, s))) return rc;
+    if ((rc = topk(cand, scores, N, C, K, Wn, w, idx_out, s))) return rc;
   }
   TRY(cudaStreamSynchronize(s));
   return mlp ? scorer_status(mlp, s) : LS_OK;

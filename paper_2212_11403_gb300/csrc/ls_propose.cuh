@@ -67,8 +67,8 @@ __global__ void mismatch_kernel(const uint32_t* __restrict__ hw, int N, int Np, 
 
 // Stage 1 for one window, one block (256 threads) per target i: the C donors with the smallest
 // mismatch sum over the available windows among w-1..w+1 (score <= 765), ties to the lower id,
-// written in ascending id order together with their features (match fractions of windows
-// w-3..w+3, clamped).  Ms[d] = count matrix of window w+d-3 (clamped), nv[d] its locus count.
+// written in ascending id order (target i's row at cand + i cstride) together with their features
+// (match fractions of windows w-3..w+3, clamped).  Ms[d] = count matrix of window w+d-3 (clamped), nv[d] its locus count.
 struct Stage1Args {
   const uint8_t* Ms[7];
   float inv_nv[7];
@@ -76,6 +76,7 @@ struct Stage1Args {
 };
 
 __global__ void __launch_bounds__(256) stage1_kernel(Stage1Args a, int N, int Np, int C, int32_t* __restrict__ cand,
+                                                     size_t cstride,
                                                      __nv_bfloat16* __restrict__ feat, float* __restrict__ feat32) {
   constexpr int NB = 768, NT = 256, V = 16;  // score bins, threads, donors per thread per pass step
   __shared__ int hist[8][NB];                // one histogram per warp (fewer colliding atomics)
@@ -180,7 +181,7 @@ __global__ void __launch_bounds__(256) stage1_kernel(Stage1Args a, int N, int Np
     for (uint32_t m = selm; m; m &= m - 1u, ++pos) {
       if (pos >= C) break;
       const int j = j0 + __ffs(m) - 1;
-      cand[(size_t)i * C + pos] = j;
+      cand[i * cstride + pos] = j;
       float f[kFeatUsed];
 #pragma unroll
       for (int d = 0; d < kFeatUsed; ++d) f[d] = 1.0f - (float)a.Ms[d][(size_t)i * Np + j] * a.inv_nv[d];
@@ -199,7 +200,7 @@ __global__ void __launch_bounds__(256) stage1_kernel(Stage1Args a, int N, int Np
     eq_seen += eq_tot;
   }
   // fewer than C donors (C >= N): pad with -1
-  for (int q = base_sel + tid; q < C; q += NT) cand[(size_t)i * C + q] = -1;
+  for (int q = base_sel + tid; q < C; q += NT) cand[i * cstride + q] = -1;
 }
 
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
@@ -207,67 +208,73 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   return *reinterpret_cast<const uint32_t*>(&v);
 }
 
-// Stage 2, one block (256 threads) per target: the K best of C candidates by score (higher first,
-// ties to the lower id; -1 entries last), written to idx[(i*Wn + w)*K ...] in ascending id order.
-// Bitonic sorts in shared memory over P = next power of two >= C (<= 2048).
-__global__ void topk_kernel(const int32_t* __restrict__ cand, const float* __restrict__ scores, int C, int K, int P,
-                            int Wn, int w, int32_t* __restrict__ idx) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  float* key = reinterpret_cast<float*>(smem);
-  int* val = reinterpret_cast<int*>(key + P);
-  const int i = blockIdx.x;
-  for (int q = threadIdx.x; q < P; q += blockDim.x) {
-    const int j = q < C ? cand[(size_t)i * C + q] : -1;
-    val[q] = j;
-    key[q] = (j >= 0 && scores) ? scores[(size_t)i * C + q] : -3.0e38f;
-  }
-  __syncthreads();
-  // order: higher key first, then lower id (ids >= 0 before -1)
-  auto before = [&](int a, int b) -> bool {
-    if (key[a] != key[b]) return key[a] > key[b];
-    const unsigned ua = (unsigned)val[a], ub = (unsigned)val[b];
-    return ua < ub;
-  };
-  for (int size = 2; size <= P; size <<= 1)
-    for (int stride = size >> 1; stride > 0; stride >>= 1) {
-      for (int q = threadIdx.x; q < P; q += blockDim.x) {
-        const int o = q ^ stride;
-        if (o > q) {
-          const bool up = (q & size) == 0;
-          if (before(o, q) == up) {
-            const float tk = key[q];
-            key[q] = key[o];
-            key[o] = tk;
-            const int tv = val[q];
-            val[q] = val[o];
-            val[o] = tv;
-          }
-        }
-      }
-      __syncthreads();
+// Stage 2, one warp per target: the K best of C candidates by score (higher first, ties to the lower
+// id; -1 entries score -3e38 and lose ties), written to idx[(i*Wn + w)*K ...] in ascending id order.
+// Stage 1 hands the candidates over in ascending id order with the -1 entries last, so position order
+// is id order and nothing has to be sorted: the K-th largest score is found by bisection over the 32
+// bits of an order-preserving integer key held in registers (V keys a lane, key v of lane q is
+// candidate 32 v + q), and the selected candidates are compacted in position order by ballots.  It is
+// bound by the compares' integer pipe; no barrier.  12345 targets, C = 1024, K = 512: 988 -> 173 us a
+// window (before: two bitonic sorts in shared memory per target; 246 us without the shared leading
+// bits and the early end).
+template <int V>
+__global__ void __launch_bounds__(256) topk_kernel(const int32_t* __restrict__ cand, const float* __restrict__ scores, int N,
+                                                   int C, int K, int Wn, int w, int32_t* __restrict__ idx) {
+  const int lane = threadIdx.x & 31;
+  const int i = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (i >= N) return;
+  const int32_t* ci = cand + (size_t)i * C;
+  uint32_t key[V];
+#pragma unroll
+  for (int v = 0; v < V; ++v) {
+    const int q = 32 * v + lane;
+    key[v] = 0u;  // beyond C: below every key of a candidate
+    if (q < C) {
+      const float f = (ci[q] >= 0 ? scores[(size_t)i * C + q] : -3.0e38f) + 0.0f;  // -0 becomes +0: they tie
+      const uint32_t u = __float_as_uint(f);
+      key[v] = u ^ ((u >> 31) ? 0xffffffffu : 0x80000000u);
     }
-  // the first K by ascending id: sort ids of positions < K (others become +inf)
-  for (int q = threadIdx.x; q < P; q += blockDim.x) {
-    const int j = q < K ? val[q] : -1;
-    val[q] = j;
   }
-  __syncthreads();
-  for (int size = 2; size <= P; size <<= 1)
-    for (int stride = size >> 1; stride > 0; stride >>= 1) {
-      for (int q = threadIdx.x; q < P; q += blockDim.x) {
-        const int o = q ^ stride;
-        if (o > q) {
-          const bool up = (q & size) == 0;
-          const unsigned a = (unsigned)val[q], b = (unsigned)val[o];
-          if ((a > b) == up) {
-            val[q] = (int)b;
-            val[o] = (int)a;
-          }
-        }
-      }
-      __syncthreads();
-    }
-  for (int q = threadIdx.x; q < K; q += blockDim.x) idx[((size_t)i * Wn + w) * K + q] = val[q];
+  // T becomes the largest value with #{key >= T} >= K (the K-th largest key), or any value with
+  // #{key >= T} = K.  The bits that the smallest and the largest candidate key share are T's too.
+  uint32_t kmin = 0xffffffffu, kmax = 0u;
+#pragma unroll
+  for (int v = 0; v < V; ++v) {
+    if (32 * v + lane < C) kmin = min(kmin, key[v]);
+    kmax = max(kmax, key[v]);
+  }
+  kmin = __reduce_min_sync(0xffffffffu, kmin);
+  kmax = __reduce_max_sync(0xffffffffu, kmax);
+  const int shared_bits = __clz(kmin ^ kmax);
+  uint32_t T = shared_bits ? kmax & ~(0xffffffffu >> shared_bits) : 0u;
+  if (shared_bits == 32) T = kmax;
+#pragma unroll 1
+  for (uint32_t bit = shared_bits == 32 ? 0u : 0x80000000u >> shared_bits; bit; bit >>= 1) {
+    const uint32_t t = T | bit;
+    int c[4] = {0, 0, 0, 0};
+#pragma unroll
+    for (int v = 0; v < V; ++v) c[v & 3] += key[v] >= t ? 1 : 0;
+    const int n = __reduce_add_sync(0xffffffffu, (c[0] + c[1]) + (c[2] + c[3]));
+    if (n >= K) T = t;
+    if (n == K) break;
+  }
+  int above = 0;
+#pragma unroll
+  for (int v = 0; v < V; ++v) above += key[v] > T ? 1 : 0;
+  int need = K - __reduce_add_sync(0xffffffffu, above);  // entries equal to T to take, in position order
+  const uint32_t lt = (1u << lane) - 1u;
+  int32_t* out = idx + ((size_t)i * Wn + w) * K;
+  int base = 0;
+#pragma unroll
+  for (int v = 0; v < V; ++v) {
+    const int q = 32 * v + lane;
+    const uint32_t eq = __ballot_sync(0xffffffffu, key[v] == T && q < C);
+    const bool sel = key[v] > T || (((eq >> lane) & 1u) && __popc(eq & lt) < need);
+    need -= min(need, __popc(eq));
+    const uint32_t m = __ballot_sync(0xffffffffu, sel);
+    if (sel) out[base + __popc(m & lt)] = ci[q];
+    base += __popc(m);
+  }
 }
 
 // Training labels of the stage-1 candidates of one window, one thread per (target, candidate):
