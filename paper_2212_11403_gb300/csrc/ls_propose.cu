@@ -372,7 +372,11 @@ int stage1(PropWork& pw, int w, int C, int32_t* cand, size_t cstride, __nv_bfloa
   a.use[0] = w - 1 >= 0;
   a.use[1] = 1;
   a.use[2] = w + 1 < pw.Wn;
-  lsk::stage1_kernel<<<pw.N, 256, 0, s>>>(a, pw.N, pw.Np, C, cand, cstride, feat, feat32);
+  // one block per target, 2048 donors a warp; the histogram kernel beyond the largest block's registers
+  const int threads = 32 * ((pw.N + 2047) / 2048);
+  if (threads <= 256) lsk::stage1_kernel<256><<<pw.N, threads, 0, s>>>(a, pw.N, pw.Np, C, cand, cstride, feat, feat32);
+  else if (threads <= 1024) lsk::stage1_kernel<1024><<<pw.N, threads, 0, s>>>(a, pw.N, pw.Np, C, cand, cstride, feat, feat32);
+  else lsk::stage1_hist_kernel<<<pw.N, 256, 0, s>>>(a, pw.N, pw.Np, C, cand, cstride, feat, feat32);
   TRY(cudaGetLastError());
   return LS_OK;
 }

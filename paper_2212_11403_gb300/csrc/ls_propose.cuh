@@ -11,6 +11,7 @@
 
 #include <cstdint>
 #include <cuda_bf16.h>
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 namespace lsk {
@@ -19,6 +20,11 @@ constexpr int kPropWS = 256;       // loci per window
 constexpr int kFeat = 16;          // feature slots per candidate (7 used, zero padded to one MMA k-step)
 constexpr int kFeatUsed = 7;
 constexpr int kHidden = 256;
+
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const uint32_t*>(&v);
+}
 
 // Haplotype-major window bits: hw[(w*N + i)*8 + k] bit b = allele of haplotype i at locus
 // w*256 + 32k + b (0 beyond L).  grid (ceil(N/32), 8, Wn), one warp: a 32 x 32 bit transpose by
@@ -75,7 +81,166 @@ struct Stage1Args {
   int use[3];  // whether windows w-1, w, w+1 exist
 };
 
-__global__ void __launch_bounds__(256) stage1_kernel(Stage1Args a, int N, int Np, int C, int32_t* __restrict__ cand,
+// Targets with N <= kS1MaxN donors: a thread keeps the scores of 4 x 16 donors in registers as
+// binary16 pairs 1024 + score (exact: scores are below 1024), finds the threshold by bisecting its ten
+// bits (two packed operations per pair and bit), and the block compacts the selected ids with two
+// scans; features are then read by position, consecutive threads on ascending ids.  The count rows are
+// read once for the scores and once for the features, in whole lines; what bounds it is that traffic and
+// the bisection's arithmetic.  N = 12345, C = 1024: 1330 -> 387 us a window (stage1_hist_kernel, whose
+// shared-memory histogram costs one atomic per donor and whose features are 7 scattered bytes per
+// selected donor).
+constexpr int kS1Iter = 4;                        // chunks of 16 donors per thread
+constexpr int kS1MaxN = 16 * kS1Iter * 1024;      // 1024 threads
+
+template <int NT>  // largest block size: warps = ceil(N / 2048) at the launch
+__global__ void __launch_bounds__(NT) stage1_kernel(Stage1Args a, int N, int Np, int C, int32_t* __restrict__ cand,
+                                                    size_t cstride, __nv_bfloat16* __restrict__ feat,
+                                                    float* __restrict__ feat32) {
+  __shared__ int cnt_s[2][32];
+  __shared__ uint2 scan_s[32];
+  const int i = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nt = blockDim.x, nw = nt >> 5;
+  const uint8_t* r0 = a.use[0] ? a.Ms[2] + (size_t)i * Np : nullptr;
+  const uint8_t* r1 = a.Ms[3] + (size_t)i * Np;
+  const uint8_t* r2 = a.use[2] ? a.Ms[4] + (size_t)i * Np : nullptr;
+  // sc[t][2m], sc[t][2m + 1]: donors (4m, 4m + 2) and (4m + 1, 4m + 3) of chunk t, low half first
+  uint32_t sc[kS1Iter][8];
+#pragma unroll
+  for (int t = 0; t < kS1Iter; ++t) {
+    const int j0 = 16 * (t * nt + tid);
+#pragma unroll
+    for (int m = 0; m < 8; ++m) sc[t][m] = 0x64006400u;
+    auto add = [&](const uint8_t* r) {
+      const uint4 v = *reinterpret_cast<const uint4*>(r + j0);  // rows are 16-byte multiples (Np a multiple of 64)
+      const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        sc[t][2 * m] += w[m] & 0x00ff00ffu;
+        sc[t][2 * m + 1] += (w[m] >> 8) & 0x00ff00ffu;
+      }
+    };
+    if (j0 < N) {
+      if (r0) add(r0);
+      add(r1);
+      if (r2) add(r2);
+    }
+    if (j0 + 16 > N || (unsigned)(i - j0) < 16u) {  // donors beyond N and the target: never below a threshold
+#pragma unroll
+      for (int k = 0; k < 16; ++k)
+        if (j0 + k >= N || j0 + k == i) sc[t][2 * (k >> 2) + (k & 1)] |= (k & 2) ? 0x67ff0000u : 0x67ffu;
+    }
+  }
+  // T: the largest t with #{score < t} < C; n_lt = #{score < T}.  A t with #{score < t} = C ends the
+  // search (nothing is taken at the threshold then).
+  int T = 0, n_lt = 0;
+  for (int bit = 512, ph = 0; bit; bit >>= 1, ph ^= 1) {
+    const int t = T | bit;
+    const uint32_t tt = (uint32_t)(0x6400 + t) * 0x10001u;
+    const __half2 th = *reinterpret_cast<const __half2*>(&tt);
+    __half2 c0 = __float2half2_rn(0.0f), c1 = c0;  // counts of at most 32 per half: exact
+#pragma unroll
+    for (int q = 0; q < kS1Iter; ++q)
+#pragma unroll
+      for (int m = 0; m < 8; m += 2) {
+        c0 = __hadd2(c0, __hlt2(*reinterpret_cast<const __half2*>(&sc[q][m]), th));
+        c1 = __hadd2(c1, __hlt2(*reinterpret_cast<const __half2*>(&sc[q][m + 1]), th));
+      }
+    c0 = __hadd2(c0, c1);
+    const int mine = (int)(__low2float(c0) + __high2float(c0));
+    const int wsum = __reduce_add_sync(0xffffffffu, mine);
+    if (lane == 0) cnt_s[ph][warp] = wsum;
+    __syncthreads();
+    const int n = __reduce_add_sync(0xffffffffu, lane < nw ? cnt_s[ph][lane] : 0);
+    if (n <= C) {
+      T = t;
+      n_lt = n;
+    }
+    if (n == C) break;
+  }
+  const int need_eq = C - n_lt;
+  // donors below / at the threshold, 16 bits per chunk
+  uint32_t ltm[kS1Iter], eqm[kS1Iter];
+#pragma unroll
+  for (int t = 0; t < kS1Iter; ++t) {
+    ltm[t] = eqm[t] = 0u;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+      const int s = (int)((sc[t][2 * (k >> 2) + (k & 1)] >> ((k & 2) ? 16 : 0)) & 0xffffu) - 0x6400;
+      ltm[t] |= (s < T ? 1u : 0u) << k;
+      eqm[t] |= (s == T && s < 1023 ? 1u : 0u) << k;
+    }
+  }
+  // exclusive prefixes over the block of four 16-bit counts per thread (chunk t of every thread comes
+  // before chunk t + 1 of any), and the block totals
+  auto scan = [&](const uint32_t (&m)[kS1Iter], int (&pre)[kS1Iter]) -> int {
+    const uint2 own = make_uint2(__popc(m[0]) | (__popc(m[1]) << 16), __popc(m[2]) | (__popc(m[3]) << 16));
+    uint2 x = own;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const uint32_t ya = __shfl_up_sync(0xffffffffu, x.x, off), yb = __shfl_up_sync(0xffffffffu, x.y, off);
+      if (lane >= off) {
+        x.x += ya;
+        x.y += yb;
+      }
+    }
+    __syncthreads();  // the previous scan's words have been read
+    if (lane == 31) scan_s[warp] = x;
+    __syncthreads();
+    const uint2 v = lane < nw ? scan_s[lane] : make_uint2(0u, 0u);
+    const uint32_t ta = __reduce_add_sync(0xffffffffu, v.x), tb = __reduce_add_sync(0xffffffffu, v.y);
+    const uint32_t wa = __reduce_add_sync(0xffffffffu, lane < warp ? v.x : 0u);
+    const uint32_t wb = __reduce_add_sync(0xffffffffu, lane < warp ? v.y : 0u);
+    const uint32_t pa = wa + x.x - own.x, pb = wb + x.y - own.y;
+    const int t0 = (int)(ta & 0xffffu), t1 = (int)(ta >> 16), t2 = (int)(tb & 0xffffu), t3 = (int)(tb >> 16);
+    pre[0] = (int)(pa & 0xffffu);
+    pre[1] = t0 + (int)(pa >> 16);
+    pre[2] = t0 + t1 + (int)(pb & 0xffffu);
+    pre[3] = t0 + t1 + t2 + (int)(pb >> 16);
+    return t0 + t1 + t2 + t3;
+  };
+  int pre[kS1Iter];
+  scan(eqm, pre);
+  uint32_t selm[kS1Iter];  // equal scores are taken in ascending id until need_eq of them are in
+#pragma unroll
+  for (int t = 0; t < kS1Iter; ++t) {
+    selm[t] = ltm[t];
+    for (uint32_t m = eqm[t]; m && pre[t] < need_eq; m &= m - 1u, ++pre[t]) selm[t] |= m & (~m + 1u);
+  }
+  const int nsel = min(scan(selm, pre), C);
+  int32_t* ci = cand + i * cstride;
+#pragma unroll
+  for (int t = 0; t < kS1Iter; ++t) {
+    int pos = pre[t];
+    for (uint32_t m = selm[t]; m; m &= m - 1u, ++pos) ci[pos] = 16 * (t * nt + tid) + __ffs(m) - 1;
+  }
+  for (int q = nsel + tid; q < C; q += nt) ci[q] = -1;  // fewer than C donors (C >= N)
+  if (!feat && !feat32) return;
+  __syncthreads();  // the block's ids are visible to all its threads
+  for (int q = tid; q < nsel; q += nt) {
+    const int j = ci[q];
+    float f[kFeatUsed];
+#pragma unroll
+    for (int d = 0; d < kFeatUsed; ++d) f[d] = 1.0f - (float)a.Ms[d][(size_t)i * Np + j] * a.inv_nv[d];
+    if (feat) {
+      uint4 lo;
+      lo.x = pack_bf16(f[0], f[1]);
+      lo.y = pack_bf16(f[2], f[3]);
+      lo.z = pack_bf16(f[4], f[5]);
+      lo.w = pack_bf16(f[6], 0.0f);
+      uint4* fo = reinterpret_cast<uint4*>(feat + ((size_t)i * C + q) * kFeat);
+      fo[0] = lo;
+      fo[1] = make_uint4(0u, 0u, 0u, 0u);
+    }
+    if (feat32) {
+      float* fo = feat32 + ((size_t)i * C + q) * 8;
+#pragma unroll
+      for (int d = 0; d < 8; ++d) fo[d] = d < kFeatUsed ? f[d] : 0.0f;
+    }
+  }
+}
+
+// The same for any N, with a histogram of the scores in shared memory: beyond kS1MaxN donors, which the
+// registers of one block cannot hold.
+__global__ void __launch_bounds__(256) stage1_hist_kernel(Stage1Args a, int N, int Np, int C, int32_t* __restrict__ cand,
                                                      size_t cstride,
                                                      __nv_bfloat16* __restrict__ feat, float* __restrict__ feat32) {
   constexpr int NB = 768, NT = 256, V = 16;  // score bins, threads, donors per thread per pass step
@@ -201,11 +366,6 @@ __global__ void __launch_bounds__(256) stage1_kernel(Stage1Args a, int N, int Np
   }
   // fewer than C donors (C >= N): pad with -1
   for (int q = base_sel + tid; q < C; q += NT) cand[i * cstride + q] = -1;
-}
-
-__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
-  const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-  return *reinterpret_cast<const uint32_t*>(&v);
 }
 
 // Stage 2, one warp per target: the K best of C candidates by score (higher first, ties to the lower
