@@ -20,7 +20,7 @@ struct ls_mlp {
   long long t = 0;          // Adam step count
   __nv_bfloat16* w1t = nullptr;  // [256][16]
   __nv_bfloat16* w2t = nullptr;  // [256][256]
-  float b3 = 0.0f;
+  std::vector<float> vec;        // host copy of b1, b2, w3, b3 (parameters of the scorer kernel)
   int* err = nullptr;            // device word: a scorer wait ran out of time
 };
 
@@ -65,35 +65,31 @@ __global__ void mlp_refresh_kernel(const float* __restrict__ p, __nv_bfloat16* _
   }
 }
 
-__global__ void to_bf16_feat_kernel(const float* __restrict__ X, long long n, __nv_bfloat16* __restrict__ Xb) {
-  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= n * lsk::kFeat) return;
-  const long long r = e / lsk::kFeat;
-  const int k = (int)(e % lsk::kFeat);
-  Xb[e] = __float2bfloat16_rn(k < lsk::kMlpIn ? X[r * lsk::kMlpIn + k] : 0.0f);
-}
-
 int refresh(ls_mlp* m) {
   mlp_refresh_kernel<<<256, 256>>>(m->p, m->w1t, m->w2t);
   TRY(cudaGetLastError());
-  TRY(cudaMemcpy(&m->b3, m->p + lsk::kOffB3, sizeof(float), cudaMemcpyDeviceToHost));
+  m->vec.resize(3 * 256 + 1);
+  TRY(cudaMemcpy(m->vec.data(), m->p + lsk::kOffB1, sizeof(float) * 256, cudaMemcpyDeviceToHost));
+  TRY(cudaMemcpy(m->vec.data() + 256, m->p + lsk::kOffB2, sizeof(float) * 513, cudaMemcpyDeviceToHost));
   return LS_OK;
 }
 
-// Scores of n BF16 feature rows on the tensor cores (persistent CTAs, one per SM).
-int launch_scores(const ls_mlp* m, const __nv_bfloat16* X, long long n, float* scores, int nsm, cudaStream_t s) {
-  TRY(cudaFuncSetAttribute(lsk::mlp_score_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, lsk::kTcSmem));
+// Scores of n feature rows (8 BF16 values, or 8 floats, each) on the tensor cores (persistent CTAs, one
+// per SM).
+template <class T>
+int launch_scores(const ls_mlp* m, const T* X, long long n, float* scores, int nsm, cudaStream_t s) {
+  TRY(cudaFuncSetAttribute(lsk::mlp_score_tc_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, lsk::kTcSmem));
   lsk::MlpTcDev d;
+  memcpy(d.b1, m->vec.data(), sizeof d.b1);
+  memcpy(d.b2, m->vec.data() + 256, sizeof d.b2);
+  memcpy(d.w3, m->vec.data() + 512, sizeof d.w3);
+  d.b3 = m->vec[768];
   d.w1t = m->w1t;
-  d.b1 = m->p + lsk::kOffB1;
   d.w2t = m->w2t;
-  d.b2 = m->p + lsk::kOffB2;
-  d.w3 = m->p + lsk::kOffW3;
-  d.b3 = m->b3;
   d.err = m->err;
   const long long tiles = (n + lsk::kTcRows - 1) / lsk::kTcRows;
   const int grid = (int)std::min<long long>(nsm, tiles);
-  lsk::mlp_score_tc_kernel<<<grid, lsk::kTcThreads, lsk::kTcSmem, s>>>(d, X, n, scores);
+  lsk::mlp_score_tc_kernel<T><<<grid, lsk::kTcThreads, lsk::kTcSmem, s>>>(d, X, n, scores);
   TRY(cudaGetLastError());
   return LS_OK;
 }
@@ -242,14 +238,9 @@ int ls_mlp_forward(const ls_mlp* m, const float* X, int64_t n, float* scores, ls
   if (!m || (n > 0 && (!X || !scores))) return fail(LS_ERR_ARG, "null argument");
   if (n <= 0) return LS_OK;
   cudaStream_t s = (cudaStream_t)stream;
-  Bufs b;
-  __nv_bfloat16* Xb;
-  int rc;
-  if ((rc = b.get(&Xb, (size_t)n * lsk::kFeat))) return rc;
-  to_bf16_feat_kernel<<<blocks(n * lsk::kFeat), 256, 0, s>>>(X, n, Xb);
-  int nsm = 0;
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, m->device);
-  if ((rc = launch_scores(m, Xb, n, scores, nsm, s))) return rc;
+  int nsm = 0, rc;
+  TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, m->device));
+  if ((rc = launch_scores(m, X, n, scores, nsm, s))) return rc;
   return scorer_status(m, s);
 }
 
@@ -433,7 +424,7 @@ int ls_propose(ls_ctx* ctx, int32_t C, int32_t K, const ls_mlp* mlp, int32_t* id
   int32_t* cand = nullptr;
   __nv_bfloat16* feat = nullptr;
   float* scores = nullptr;
-  if (mlp && ((rc = b.get(&cand, (size_t)N * C)) || (rc = b.get(&feat, (size_t)N * C * lsk::kFeat)) ||
+  if (mlp && ((rc = b.get(&cand, (size_t)N * C)) || (rc = b.get(&feat, (size_t)N * C * 8)) ||
               (rc = b.get(&scores, (size_t)N * C))))
     return rc;
   for (int w = 0; w < Wn; ++w) {

@@ -17,7 +17,7 @@
 namespace lsk {
 
 constexpr int kPropWS = 256;       // loci per window
-constexpr int kFeat = 16;          // feature slots per candidate (7 used, zero padded to one MMA k-step)
+constexpr int kFeat = 16;          // inputs of layer 1 on the tensor cores (one k-step; a feature row holds the first 8)
 constexpr int kFeatUsed = 7;
 constexpr int kHidden = 256;
 
@@ -226,9 +226,7 @@ __global__ void __launch_bounds__(NT) stage1_kernel(Stage1Args a, int N, int Np,
       lo.y = pack_bf16(f[2], f[3]);
       lo.z = pack_bf16(f[4], f[5]);
       lo.w = pack_bf16(f[6], 0.0f);
-      uint4* fo = reinterpret_cast<uint4*>(feat + ((size_t)i * C + q) * kFeat);
-      fo[0] = lo;
-      fo[1] = make_uint4(0u, 0u, 0u, 0u);
+      *reinterpret_cast<uint4*>(feat + ((size_t)i * C + q) * 8) = lo;
     }
     if (feat32) {
       float* fo = feat32 + ((size_t)i * C + q) * 8;
@@ -351,9 +349,9 @@ __global__ void __launch_bounds__(256) stage1_hist_kernel(Stage1Args a, int N, i
 #pragma unroll
       for (int d = 0; d < kFeatUsed; ++d) f[d] = 1.0f - (float)a.Ms[d][(size_t)i * Np + j] * a.inv_nv[d];
       if (feat) {
-        __nv_bfloat16* fo = feat + ((size_t)i * C + pos) * kFeat;
+        __nv_bfloat16* fo = feat + ((size_t)i * C + pos) * 8;
 #pragma unroll
-        for (int d = 0; d < kFeat; ++d) fo[d] = __float2bfloat16_rn(d < kFeatUsed ? f[d] : 0.0f);
+        for (int d = 0; d < 8; ++d) fo[d] = __float2bfloat16_rn(d < kFeatUsed ? f[d] : 0.0f);
       }
       if (feat32) {
         float* fo = feat32 + ((size_t)i * C + pos) * 8;

@@ -43,3 +43,29 @@ def test_topk_is_the_sorted_selection(ls, N, C, K, ties):
         best = np.full(K, -1)
         best[:len(order)] = np.sort(cand[i, :n][order])
         np.testing.assert_array_equal(idx[i], best)
+
+
+# one row, around one tile, more tiles than SMs by one row; rows on and off a 16-byte boundary
+@pytest.mark.parametrize("n", [1, 127, 128, 129, 152 * 128 + 1, 152 * 128 * 2 + 5])
+@pytest.mark.parametrize("offset", [0, 1])
+def test_scorer_row_counts_and_alignment(ls, n, offset):
+    import torch
+
+    import oracle.proposal as op
+    rng = np.random.default_rng(n)
+    p = (rng.normal(0, 1, op.N_PARAMS) * 0.15).astype(np.float32)
+    X = rng.random((n, 8)).astype(np.float32)
+    m = ls.ls_mlp_create(p)
+    try:
+        flat = torch.zeros(8 * n + offset, device="cuda")
+        Xd = flat[offset:].view(n, 8)
+        Xd.copy_(torch.from_numpy(X))
+        s = torch.full((n + 1,), 7.0, device="cuda")
+        ls.ls_mlp_forward(m, Xd, s[:n])
+        s = s.cpu().numpy().astype(np.float64)
+    finally:
+        ls.ls_mlp_destroy(m)
+    assert s[n] == 7.0
+    ref = op.mlp_forward_bf16(p.astype(np.float64), X.astype(np.float64))
+    # FP32 accumulation against exact sums, and a hidden unit on a BF16 rounding boundary
+    assert float(np.max(np.abs(s[:n] - ref))) <= 2e-3 * float(np.max(np.abs(ref)))
