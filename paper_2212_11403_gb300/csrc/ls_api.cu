@@ -12,6 +12,7 @@
 
 #include "ls.h"
 #include "ls_aux.cuh"
+#include "ls_row.cuh"
 #define LS_SPARSE_PARAMS_ONLY
 #include "ls_sparse.cuh"
 #include "ls_internal.h"
@@ -269,6 +270,42 @@ int run_launches(ls_ctx* c, lsk::PropParams p, int t_begin, int t_count, cudaStr
     if (e != cudaSuccess) return fail(LS_ERR_CUDA, "propagation launch (TPW=%d W=%d KQ=%d): %s", L.k->tpw, L.k->w, L.k->kq,
                                       cudaGetErrorString(e));
   }
+  return LS_OK;
+}
+
+// 16-byte accesses need rows of whole quads on 16-byte boundaries (stored rows are the caller's)
+bool row_quads(int N, const void* a, const void* b = nullptr) {
+  return N % 4 == 0 && ((reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b)) & 15) == 0;
+}
+
+// Table calls of few steps with the uniform prior go to the row kernel (one target per CTA, the row in
+// registers).  It costs less per call and more per step than the register-tile kernels: one / eight /
+// sixteen loci forward take 158 / 533 / 988 us against 658 / 762 / 875 us at N = 10000, 16 / 22 / 30
+// against 30 / 29 / 33 us at N = 1000 and 654 / 2264 / 4211 against 2412 / 2775 / 3214 us at N = 20000.
+// Rows off the 16-byte grid cost twice as much per step beyond N = 2048 (N = 4999, one / four / eight
+// loci: 83 / 177 / 311 against 160 / 169 / 182 us), so the line lies lower there.
+bool row_steps_serve(const ls_ctx* c, const lsk::PropParams& p) {
+  const int most = row_quads(p.N, p.state, p.store) || p.N <= 2048 ? 8 : 3;
+  return !c->Pi && p.N <= lsk::kRowMaxN && p.n_steps <= most;
+}
+
+template <int E4, int VEC>
+void launch_row_steps(const lsk::PropParams& p, cudaStream_t s) {
+  const int nt = 32 * ((p.N + 128 * E4 - 1) / (128 * E4));
+  if (p.dir == 0) lsk::row_steps_kernel<0, E4, VEC><<<p.t_count, nt, 0, s>>>(p);
+  else lsk::row_steps_kernel<1, E4, VEC><<<p.t_count, nt, 0, s>>>(p);
+}
+
+int run_row_steps(lsk::PropParams p, int t_begin, int t_count, cudaStream_t s) {
+  p.t_begin = t_begin;
+  p.t_count = t_count;
+  const bool vec = row_quads(p.N, p.state, p.store);
+  // 8, 20 or 40 elements a thread: at most 256 threads a CTA up to N = 10240
+  if (p.N <= 2048) vec ? launch_row_steps<2, 4>(p, s) : launch_row_steps<2, 1>(p, s);
+  else if (p.N <= 5120) vec ? launch_row_steps<5, 4>(p, s) : launch_row_steps<5, 1>(p, s);
+  else vec ? launch_row_steps<10, 4>(p, s) : launch_row_steps<10, 1>(p, s);
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return fail(LS_ERR_CUDA, "row step launch: %s", cudaGetErrorString(e));
   return LS_OK;
 }
 
@@ -713,7 +750,7 @@ static int propagate(ls_ctx* ctx, ls_table* tb, int dir, int32_t to, const int32
     }
     p.store = out;
     if (p.n_steps > 0) {
-      rc = run_launches(ctx, p, tb->t_from, T, s);
+      rc = row_steps_serve(ctx, p) ? run_row_steps(p, tb->t_from, T, s) : run_launches(ctx, p, tb->t_from, T, s);
       if (rc) return rc;
     }
     pos = seg_end;

@@ -1,0 +1,144 @@
+// ls_row.cuh -- kernels that take one table row per CTA and hold it in registers: single steps of a
+// table, and posteriors / half distances of a row.
+//
+// Both are bound by memory: a row is read once, stays in registers across its reductions and is
+// written once, with 16-byte accesses where rows are 16-byte multiples (VEC = 4) and 4-byte ones
+// otherwise (VEC = 1).  Thread t of nt holds 4 E4 elements: quads t, t + nt, .. (VEC = 4) or elements
+// t, t + nt, .. (VEC = 1), so a warp's accesses are contiguous either way.
+#pragma once
+
+#include <cstdint>
+#include <cuda_runtime.h>
+
+#include "ls_prop.cuh"
+
+namespace lsk {
+
+constexpr int kRowMaxThreads = 512;
+constexpr int kRowMaxN = 40 * kRowMaxThreads;  // E4 = 10
+
+// sum over the CTA, the same value in every thread; buf holds 32 floats and alternates between calls
+__device__ __forceinline__ float row_sum(float v, float* buf) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+  if (nw == 1) return v;
+  if (lane == 0) buf[warp] = v;
+  __syncthreads();
+  v = lane < nw ? buf[lane] : 0.0f;
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+  return v;
+}
+
+template <int E4, int VEC>
+struct RowPos {  // first position of the e-th access and the number of accesses
+  static constexpr int COUNT = VEC == 4 ? E4 : 4 * E4;
+  __device__ static int at(int e) { return VEC * ((int)threadIdx.x + e * (int)blockDim.x); }
+};
+
+template <int VEC>
+__device__ __forceinline__ void row_load(const float* p, float* v) {
+  if (VEC == 4) {
+    const float4 q = __ldcs(reinterpret_cast<const float4*>(p));
+    v[0] = q.x, v[1] = q.y, v[2] = q.z, v[3] = q.w;
+  } else {
+    v[0] = __ldcs(p);
+  }
+}
+template <int VEC>
+__device__ __forceinline__ void row_store(float* p, const float* v) {
+  if (VEC == 4) __stcs(reinterpret_cast<float4*>(p), make_float4(v[0], v[1], v[2], v[3]));
+  else __stcs(p, v[0]);
+}
+
+// A few steps of a table (uniform prior; PropParams as for ls_prop_kernel, without alpha_dec and
+// tlist), one target per CTA.  The register-tile kernel loads and saves its tile through shared memory
+// element by element; a table moved by one locus is all load and save, so this kernel takes calls of
+// few steps.  N = 10000, one locus forward / backward: 658 / 520 -> 158 / 186 us (0.8 GB moved, 75 / 63 % of
+// the measured copy rate); the two reductions between load and save are what keeps it from the rest.
+template <int DIR, int E4, int VEC>
+__global__ void __launch_bounds__(kRowMaxThreads) row_steps_kernel(const PropParams p) {
+  using P = RowPos<E4, VEC>;
+  __shared__ float buf[2][32];
+  const int N = p.N, i = p.t_begin + blockIdx.x, row = i - p.tab_t0;
+  float* state = p.state + (size_t)row * N;
+  float x[P::COUNT][VEC];
+  int ph = 0;
+  auto total = [&](float s) {
+    ph ^= 1;
+    return row_sum(s, buf[ph]);
+  };
+  float sig_prev = 1.0f;
+  {
+    float s = 0.0f;
+#pragma unroll
+    for (int e = 0; e < P::COUNT; ++e) {
+      const int pos = P::at(e);
+#pragma unroll
+      for (int k = 0; k < VEC; ++k) x[e][k] = 0.0f;
+      if (p.load_state && pos < N) row_load<VEC>(state + pos, x[e]);
+#pragma unroll
+      for (int k = 0; k < VEC; ++k) s += x[e][k];
+    }
+    if (p.load_state && DIR == 0) sig_prev = total(s);
+  }
+  double lg = 0.0;
+  uint32_t sts = 0u;
+  int store_next = 0;
+  for (int step = 0; step < p.n_steps; ++step) {
+    const int l = DIR == 0 ? p.l_first + step : p.l_first - step;
+    const bool last = step + 1 == p.n_steps;
+    float c, r, sg = 1.0f;
+    if (step == 0 && p.init) {
+      c = 0.0f;
+      r = DIR == 0 ? p.pi_u : 1.0f;  // alpha^0 = theta pi ; beta^{L-1} = 1
+    } else if (step == 0 && DIR == 1) {
+      c = 1.0f;  // backward resume: x = theta^l beta^l from the stored beta
+      r = 0.0f;
+    } else {
+      const int m = DIR == 0 ? l - 1 : l;
+      c = __fdividef(p.omr[m], sig_prev);
+      r = p.rr[m];
+      sg = sig_prev;
+    }
+    const bool store_here = store_next < p.n_store && p.store_loci[store_next] == l;
+    float* out = store_here ? p.store + ((size_t)p.store_slot[store_next] * p.state_rows + row) * N : nullptr;
+    store_next += store_here ? 1 : 0;
+    const uint32_t* bits = p.bits2 + (size_t)l * p.rw2;
+    const uint32_t inv = (bits[i >> 5] >> (i & 31)) & 1u ? 0u : 0xffffffffu;  // match = bit ^ inv
+    const float tm = p.thm[l], tx = p.thx[l];
+    float s = 0.0f;
+#pragma unroll
+    for (int e = 0; e < P::COUNT; ++e) {
+      const int pos = P::at(e);
+      if (pos < N) {
+        const uint32_t w = (bits[pos >> 5] ^ inv) >> (pos & 31);
+        float b[VEC];
+#pragma unroll
+        for (int k = 0; k < VEC; ++k) {
+          b[k] = pos + k == i ? 0.0f : fmaf(c, x[e][k], r);  // alpha before its emission, or beta
+          x[e][k] = ((w >> k) & 1u ? tm : tx) * b[k];
+          s += x[e][k];
+        }
+        const float* v = DIR == 0 ? x[e] : b;
+        if (out) row_store<VEC>(out + pos, v);
+        if (last && p.save_state) row_store<VEC>(state + pos, v);
+      }
+    }
+    if (DIR == 0 || !last) {
+      const float sig = total(s) * (DIR == 0 ? 1.0f : p.pi_u);
+      if (DIR == 0) sg = sig;
+      sig_prev = sig;
+    }
+    if (sg < 1.17549435e-38f) sts |= 1u;      // LS_STATUS_UNDERFLOW
+    if (!(sg <= 3.40282347e+38f)) sts |= 2u;  // LS_STATUS_OVERFLOW
+    lg += (double)logf(sg);
+  }
+  if (threadIdx.x == 0) {
+    if (p.logs) p.logs[row] = (p.init ? 0.0 : p.logs[row]) + lg;
+    if (p.status && sts) atomicOr(p.status + row, sts);
+  }
+}
+
+}  // namespace lsk
