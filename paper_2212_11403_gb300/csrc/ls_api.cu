@@ -309,6 +309,53 @@ int run_row_steps(lsk::PropParams p, int t_begin, int t_count, cudaStream_t s) {
   return LS_OK;
 }
 
+// Posterior rows: DEC 0 grid (rows), DEC 1 grid (N, D).  The row kernel takes rows of whole quads on
+// 16-byte boundaries: posteriors up to 64 elements a thread (N = 5000 / 10000 / 20000 / 26000: 100 / 442 /
+// 893 / 1170 -> 64 / 249 / 637 / 902 us), the decode in place up to 20 (N = 2500 / 5000: 25 / 74 -> 16 / 49
+// us; at N = 10000 both take 0.31 ms, bound by the logarithms).  Other rows are faster with the two-pass
+// kernels (N = 10001: 443 against 683 us with 4-byte accesses held in registers).
+template <int DEC, int E4>
+void launch_posterior(const lsk::PostArgs& a, dim3 grid, cudaStream_t s) {
+  const int nt = 32 * ((a.N + 128 * E4 - 1) / (128 * E4));
+  lsk::row_posterior_kernel<DEC, E4><<<grid, nt, 0, s>>>(a);
+}
+template <int DEC>
+int launch_posterior(const lsk::PostArgs& a, dim3 grid, cudaStream_t s) {
+  const bool quads = row_quads(a.N, a.out) && (DEC || row_quads(a.N, a.alpha, a.beta));
+  if (quads && a.N <= 2048) launch_posterior<DEC, 2>(a, grid, s);
+  else if (quads && a.N <= 5120) launch_posterior<DEC, 5>(a, grid, s);
+  else if (DEC) lsk::decode_kernel<<<grid, 256, 0, s>>>(a.out, a.N, a.bits, a.row_words, a.thm, a.thx, a.dl);
+  else if (quads && a.N <= 20480) launch_posterior<0, 10>(a, grid, s);
+  else if (quads && a.N <= lsk::kRowMaxPostN) launch_posterior<0, 16>(a, grid, s);
+  else lsk::posterior_kernel<<<grid, 256, 0, s>>>(a.alpha, a.beta, a.N, a.t0, a.mode, a.out);
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return fail(LS_ERR_CUDA, "posterior launch: %s", cudaGetErrorString(e));
+  return LS_OK;
+}
+// p (mode 0) or half distances (mode 1) of T targets from t0 on
+int posterior_rows(const float* alpha, const float* beta, int N, int t0, int T, int mode, float* out, cudaStream_t s) {
+  lsk::PostArgs a = {};
+  a.alpha = alpha;
+  a.beta = beta;
+  a.out = out;
+  a.N = N;
+  a.t0 = t0;
+  a.mode = mode;
+  return launch_posterior<0>(a, dim3(T), s);
+}
+// the backward's products at D decode loci into half distances, in place
+int decode_rows(const ls_ctx* c, const int32_t* loci, int D, float* d, cudaStream_t s) {
+  lsk::PostArgs a = {};
+  a.out = d;
+  a.N = c->N;
+  a.bits = c->bits;
+  a.row_words = c->row_words;
+  a.thm = c->thm;
+  a.thx = c->thx;
+  for (int k = 0; k < D; ++k) a.dl.l[k] = loci[k];
+  return launch_posterior<1>(a, dim3(c->N, D), s);
+}
+
 int check_ctx(const ls_ctx* c) {
   if (!c) return fail(LS_ERR_ARG, "null context");
   if (cudaSetDevice(c->device) != cudaSuccess) return fail(LS_ERR_CUDA, "cudaSetDevice(%d) failed", c->device);
@@ -915,9 +962,7 @@ int ls_posterior(ls_ctx* ctx, const ls_table* fwd, const ls_table* bck, float* p
   if (rc) return rc;
   if (!p_out) return fail(LS_ERR_ARG, "null output");
   const int T = fwd->t_to - fwd->t_from;
-  lsk::posterior_kernel<<<T, 256, 0, (cudaStream_t)stream>>>(fwd->state, bck->state, ctx->N, fwd->t_from, 0, p_out);
-  CUDA_TRY(cudaGetLastError());
-  return LS_OK;
+  return posterior_rows(fwd->state, bck->state, ctx->N, fwd->t_from, T, 0, p_out, (cudaStream_t)stream);
 }
 
 int ls_distance(ls_ctx* ctx, const ls_table* fwd, const ls_table* bck, float* d_out, ls_stream_t stream) {
@@ -927,8 +972,7 @@ int ls_distance(ls_ctx* ctx, const ls_table* fwd, const ls_table* bck, float* d_
   if (fwd->t_from != 0 || fwd->t_to != ctx->N) return fail(LS_ERR_RANGE, "the distance matrix needs tables over all N targets");
   const int N = ctx->N;
   cudaStream_t s = (cudaStream_t)stream;
-  lsk::posterior_kernel<<<N, 256, 0, s>>>(fwd->state, bck->state, N, 0, 1, d_out);
-  CUDA_TRY(cudaGetLastError());
+  if ((rc = posterior_rows(fwd->state, bck->state, N, 0, N, 1, d_out, s))) return rc;
   const int nt = (N + 31) / 32;
   lsk::symmetrize_kernel<<<dim3(nt, nt, 1), dim3(32, 8), 0, s>>>(d_out, N);
   CUDA_TRY(cudaGetLastError());
@@ -1002,10 +1046,7 @@ int ls_run_all(ls_ctx* ctx, const int32_t* decode_loci, int32_t D, float* d_out,
   if (prof) CUDA_TRY(cudaEventRecord(ctx->ev[2], s));
   ctx->launches[2] = ctx->launches[3] = 0;
   if (D > 0) {
-    lsk::DecodeLoci dl;
-    for (int k = 0; k < D; ++k) dl.l[k] = decode_loci[k];
-    lsk::decode_kernel<<<dim3(N, D), 256, 0, s>>>(dd, N, ctx->bits, ctx->row_words, ctx->thm, ctx->thx, dl);
-    CUDA_TRY(cudaGetLastError());
+    if ((rc = decode_rows(ctx, decode_loci, D, dd, s))) return rc;
     ctx->launches[2] = 1;
   }
   if (prof) CUDA_TRY(cudaEventRecord(ctx->ev[3], s));
@@ -1522,9 +1563,7 @@ int ls_posterior_rows(ls_ctx* ctx, const float* alpha, const float* beta, int32_
   int rc = check_ctx(ctx);
   if (rc) return rc;
   if (!alpha || !beta || !p_out || T < 1 || t_from < 0 || t_from + T > ctx->N) return fail(LS_ERR_ARG, "bad arguments");
-  lsk::posterior_kernel<<<T, 256, 0, (cudaStream_t)stream>>>(alpha, beta, ctx->N, t_from, 0, p_out);
-  CUDA_TRY(cudaGetLastError());
-  return LS_OK;
+  return posterior_rows(alpha, beta, ctx->N, t_from, T, 0, p_out, (cudaStream_t)stream);
 }
 
 int ls_set_profiling(ls_ctx* ctx, int32_t enable) {
@@ -1673,10 +1712,7 @@ extern "C" int ls_run_all_noalloc(ls_ctx* ctx, const int32_t* decode_loci, int32
     }
   }
   if (D > 0) {
-    lsk::DecodeLoci dl;
-    for (int k = 0; k < D; ++k) dl.l[k] = decode_loci[k];
-    lsk::decode_kernel<<<dim3(N, D), 256, 0, s>>>(d_out, N, ctx->bits, ctx->row_words, ctx->thm, ctx->thx, dl);
-    CUDA_TRY(cudaGetLastError());
+    if ((rc = decode_rows(ctx, decode_loci, D, d_out, s))) return rc;
     const int nt = (N + 31) / 32;
     lsk::symmetrize_kernel<<<dim3(nt, nt, D), dim3(32, 8), 0, s>>>(d_out, N);
     CUDA_TRY(cudaGetLastError());

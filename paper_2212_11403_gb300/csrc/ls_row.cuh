@@ -10,12 +10,13 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
-#include "ls_prop.cuh"
+#include "ls_aux.cuh"
 
 namespace lsk {
 
 constexpr int kRowMaxThreads = 512;
-constexpr int kRowMaxN = 40 * kRowMaxThreads;  // E4 = 10
+constexpr int kRowMaxN = 40 * kRowMaxThreads;  // single steps (E4 = 10)
+constexpr int kRowMaxPostN = 64 * kRowMaxThreads;  // posteriors (E4 = 16)
 
 // sum over the CTA, the same value in every thread; buf holds 32 floats and alternates between calls
 __device__ __forceinline__ float row_sum(float v, float* buf) {
@@ -138,6 +139,87 @@ __global__ void __launch_bounds__(kRowMaxThreads) row_steps_kernel(const PropPar
   if (threadIdx.x == 0) {
     if (p.logs) p.logs[row] = (p.init ? 0.0 : p.logs[row]) + lg;
     if (p.status && sts) atomicOr(p.status + row, sts);
+  }
+}
+
+// Eq. postprob of one row per CTA, the row's products held in registers between their sum and their use.
+// DEC = 0: products alpha (beta 2^100) of caller-held rows (target t0 + r), written as p (mode 0) or as
+// half distances -log(max(p, eps))/2 (mode 1).  DEC = 1: the products alpha t 2^100 that the backward
+// pass left in out at D decode loci ([D][N][N], row i = recipient i), t = theta beta, are divided by their
+// emission theta^l (1 - mu where the donor carries the target's allele at l, mu elsewhere; a zero theta
+// means alpha = 0 too, and the entry is 0) and replaced by half distances.  A zero normaliser gives p =
+// eps for every donor (Sec. 2.2); the target's own entry is 0.  Rows are whole quads
+// on 16-byte boundaries.  Bound by memory (posteriors at N = 10000: 249 us, 4.8 TB/s; before, with the
+// rows read twice, 442 us) and, with distances, by the logarithms too.
+struct PostArgs {
+  const float *alpha, *beta;  // DEC 0
+  float* out;
+  int N, t0, mode;
+  const uint32_t* bits;       // DEC 1: packed rows
+  int row_words;
+  const float *thm, *thx;
+  DecodeLoci dl;
+};
+
+template <int DEC, int E4>
+__global__ void __launch_bounds__(kRowMaxThreads) row_posterior_kernel(const __grid_constant__ PostArgs a) {
+  constexpr float eps = 2.220446049250313e-16f;
+  constexpr int VEC = 4;
+  using P = RowPos<E4, VEC>;
+  __shared__ float buf[32];
+  const int N = a.N, r = blockIdx.x, i = DEC ? r : a.t0 + r;
+  float* o = a.out + ((size_t)(DEC ? blockIdx.y : 0) * (DEC ? N : 0) + r) * N;
+  const uint32_t* bits = nullptr;
+  uint32_t inv = 0u;
+  float im = 0.0f, ix = 0.0f;
+  if (DEC) {
+    const int l = a.dl.l[blockIdx.y];
+    bits = a.bits + (size_t)l * a.row_words;
+    inv = (bits[i >> 5] >> (i & 31)) & 1u ? 0u : 0xffffffffu;
+    im = a.thm[l] > 0.0f ? 1.0f / a.thm[l] : 0.0f;
+    ix = a.thx[l] > 0.0f ? 1.0f / a.thx[l] : 0.0f;
+  }
+  float q[P::COUNT][VEC];
+  float s = 0.0f;
+#pragma unroll
+  for (int e = 0; e < P::COUNT; ++e) {
+    const int pos = P::at(e);
+#pragma unroll
+    for (int k = 0; k < VEC; ++k) q[e][k] = 0.0f;
+    if (pos < N) {
+      if (DEC) {
+        row_load<VEC>(o + pos, q[e]);
+        const uint32_t w = (bits[pos >> 5] ^ inv) >> (pos & 31);
+#pragma unroll
+        for (int k = 0; k < VEC; ++k) q[e][k] *= (w >> k) & 1u ? im : ix;
+      } else {
+        float b[VEC];
+        row_load<VEC>(a.alpha + (size_t)r * N + pos, q[e]);
+        row_load<VEC>(a.beta + (size_t)r * N + pos, b);
+#pragma unroll
+        for (int k = 0; k < VEC; ++k) q[e][k] *= b[k] * kProdScale;
+      }
+#pragma unroll
+      for (int k = 0; k < VEC; ++k) {
+        if (pos + k == i) q[e][k] = 0.0f;
+        s += q[e][k];
+      }
+    }
+  }
+  const float Z = row_sum(s, buf);
+  const float invZ = Z > 0.0f ? 1.0f / Z : 0.0f;
+#pragma unroll
+  for (int e = 0; e < P::COUNT; ++e) {
+    const int pos = P::at(e);
+    if (pos < N) {
+      float v[VEC];
+#pragma unroll
+      for (int k = 0; k < VEC; ++k) {
+        const float p = Z > 0.0f ? q[e][k] * invZ : eps;
+        v[k] = pos + k == i ? 0.0f : (DEC || a.mode == 1 ? -0.5f * logf(fmaxf(p, eps)) : p);
+      }
+      row_store<VEC>(o + pos, v);
+    }
   }
 }
 
