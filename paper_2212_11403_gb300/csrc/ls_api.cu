@@ -1439,8 +1439,23 @@ int ls_sparse_run_all(ls_ctx* ctx, const int32_t* idx, int32_t K, int32_t WS, in
     cudaError_t eh = ls_launch_hapmajor(ctx->bits, ctx->row_words, N, L, hw, s);
     if (eh != cudaSuccess) return fail(LS_ERR_CUDA, "haplotype-major words: %s", cudaGetErrorString(eh));
   }
+  float* emit;  // ratio of the emission values per locus
+  if ((rc = db.get(&emit, L))) return rc;
+  {
+    cudaError_t ee = ls_launch_emission(ctx->thm, ctx->thx, L, emit, s);
+    if (ee != cudaSuccess) return fail(LS_ERR_CUDA, "emission values: %s", cudaGetErrorString(ee));
+  }
   lsk::SparseParams sp;
   memset(&sp, 0, sizeof sp);
+  sp.ratio = emit;
+  for (int l = 0; l < L; ++l) {  // the chains run with emissions over the larger value (its FP32 rounding)
+    if (l > 0 && ctx->mu_h.size() == 1) {
+      sp.log_base *= L;
+      break;
+    }
+    const double m = ctx->mu_h[l];
+    sp.log_base += std::log((double)std::max((float)(1.0 - m), (float)m));
+  }
   sp.hw = hw;
   sp.N = N;
   sp.L = L;
@@ -1450,8 +1465,6 @@ int ls_sparse_run_all(ls_ctx* ctx, const int32_t* idx, int32_t K, int32_t WS, in
   sp.idx = sets;
   sp.omr = ctx->omr;
   sp.rho = ctx->rr_b;
-  sp.thm = ctx->thm;
-  sp.thx = ctx->thx;
   sp.t_begin = 0;
   sp.t_count = N;
   sp.store = P;

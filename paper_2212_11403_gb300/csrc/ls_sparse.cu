@@ -17,15 +17,19 @@ cudaError_t launch_ks(int dir, const lsk::SparseParams& p0, cudaStream_t s) {
 }
 }  // namespace
 
-// slots per lane: the smallest of 1, 2, 4, 8, 16, 32, 48 with 32 * KS >= K (K <= 1536)
+// slots per lane: the smallest of 2, 4, 8, 16, 32, 48 with 32 * KS >= K (K <= 1536)
 cudaError_t ls_launch_sparse(int dir, const lsk::SparseParams& p, cudaStream_t s) {
-  if (p.K <= 32) return launch_ks<1>(dir, p, s);
   if (p.K <= 64) return launch_ks<2>(dir, p, s);
   if (p.K <= 128) return launch_ks<4>(dir, p, s);
   if (p.K <= 256) return launch_ks<8>(dir, p, s);
   if (p.K <= 512) return launch_ks<16>(dir, p, s);
   if (p.K <= 1024) return launch_ks<32>(dir, p, s);
   return launch_ks<48>(dir, p, s);
+}
+
+cudaError_t ls_launch_emission(const float* thm, const float* thx, int L, float* ratio, cudaStream_t s) {
+  lsk::emission_kernel<<<(L + 255) / 256, 256, 0, s>>>(thm, thx, L, ratio);
+  return cudaGetLastError();
 }
 
 cudaError_t ls_launch_lookahead(const int32_t* idx, int N, int Wn, int K, int span, int32_t* U, cudaStream_t s) {

@@ -23,10 +23,21 @@
 // backward value of the outside donors, and each outside donor receives an equal share of the
 // pool's posterior mass (an estimate, reported apart from the set donors' values).
 //
-// One warp per target, slot s of lane q <-> set index 32 s + q (coalesced set loads and stores);
-// eight targets per CTA share the packed locus rows, staged up to eight rows at a time in shared
-// memory together with the rows' per-locus constants, double-buffered: the asynchronous copies
-// (cp.async) of the next block run while the current one is processed.
+// One warp per target, slot s of lane q <-> set index 32 s + q (coalesced set loads and stores).  Loci
+// run in blocks of 64.  At the start of a block (and at a window change) a lane loads the block's 64
+// bits of each of its donors from the haplotype-major words (8 bytes of a 32-byte sector), XORs them
+// with the target's and transposes them in registers to one word per locus and 32 slots, bit s = slot
+// s differs from the target; the words wait in shared memory.  A locus then needs its words, a packed
+// FFMA2 and FADD2 per pair of slots and one predicated multiply per slot: theta (c x + r) = f (c b x + r b)
+// with b = max(1-mu, mu) and f in {1, min/b}, the number of matching slots is a population count, and
+// the per-locus logarithms are taken 32 at a time.  Padding slots count as mismatches; they start at 0
+// when their window starts and so hold one common value xs, which the row sum subtracts.  The
+// per-locus constants of the next block are copied with cp.async while the current one runs.
+//
+// 247 warp instructions a locus at 48 slots a lane, issued in 46 % of the cycles with three warps a
+// scheduler: bound by the dependent chain of a locus (row sum, division, multiply, add).  N = 20003, L =
+// 2000, K = 3 x 512: forward / backward 32.3 / 30.2 -> 17.3 / 17.6 ms (before: one word and one bit test,
+// select and count per slot and locus, set ids in registers, two warps a scheduler).
 #pragma once
 
 #include <cstdint>
@@ -35,9 +46,9 @@
 
 namespace lsk {
 
-constexpr int kSparseWarps = 8;  // targets per CTA
-constexpr int kSparseChunk = 32;  // loci per block: one 32-bit haplotype-major word per donor
-constexpr int kSparseScal = 5;    // per-locus constants staged per block: 1-mu, mu, 1-rho, rho, n1
+constexpr int kSparseWarps = 4;   // targets per CTA (three CTAs per SM at 48 slots a lane)
+constexpr int kSparseChunk = 64;  // loci per block: two 32-bit haplotype-major words per donor
+constexpr int kSparseScal = 4;    // per-locus constants staged per block: 1-rho, rho, n1, emission ratio
 
 struct SparseParams {
   const uint32_t* hw;    // [ceil(L/256)][N][8] haplotype-major words: bit b of word k of (w, j) is
@@ -49,8 +60,8 @@ struct SparseParams {
   const int32_t* idx;    // [N][Wn][K] donor ids, ascending, -1 padding at the end
   const float* omr;      // [L-1] 1 - rho
   const float* rho;      // [L-1] rho
-  const float* thm;      // [L] 1 - mu
-  const float* thx;      // [L] mu
+  const float* ratio;    // [L] the smaller of 1 - mu and mu over the larger; negative where the larger is mu
+  double log_base;       // sum over the loci of the logarithm of the larger
   int t_begin, t_count;
   int n_store;
   int store_loci[64];    // processing order
@@ -70,9 +81,16 @@ struct SparseParams {
 // keeps products of small alpha and beta above FP32's underflow
 constexpr float kSparseProdScale = 0x1p100f;
 
-// two buffers of per-locus constants and the per-warp set copies used at window changes
-__host__ __device__ inline int sparse_smem_bytes(int ks) {
-  return 2 * kSparseScal * kSparseChunk * 4 + 2 * kSparseWarps * 32 * ks * 4;
+// 32-slot groups of a lane's slots, and bytes per warp: the block's words [64][groups][32], whose place
+// the copies of the old set (ids and values) take at a window change
+__host__ __device__ constexpr int sparse_groups(int ks) { return (ks + 31) / 32; }
+__host__ __device__ constexpr int sparse_warp_bytes(int ks) {
+  return kSparseChunk * sparse_groups(ks) * 128 > 256 * ks ? kSparseChunk * sparse_groups(ks) * 128 : 256 * ks;
+}
+constexpr int kSparsePool = 2 * kSparseChunk;  // floats per warp: the outside donors' summed and mean emission per locus
+// two buffers of per-locus constants and the per-warp regions
+__host__ __device__ constexpr int sparse_smem_bytes(int ks) {
+  return 2 * kSparseScal * kSparseChunk * 4 + kSparseWarps * (kSparsePool * 4 + sparse_warp_bytes(ks));
 }
 
 __device__ __forceinline__ void cp_async4(void* dst, const void* src) {
@@ -84,34 +102,49 @@ __device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_g
 
 #ifndef LS_SPARSE_PARAMS_ONLY  // the kernels live in ls_sparse.cu only
 
+// 32 x 32 bit transposition: bit c of m[r] and bit r of m[c] change places
+__device__ __forceinline__ void transpose32(uint32_t (&m)[32]) {
+#pragma unroll
+  for (int st = 0; st < 5; ++st) {
+    const int j = 16 >> st;
+    const uint32_t mask = st == 0 ? 0x0000ffffu : st == 1 ? 0x00ff00ffu : st == 2 ? 0x0f0f0f0fu : st == 3 ? 0x33333333u : 0x55555555u;
+#pragma unroll
+    for (int k = 0; k < 32; ++k)
+      if (!(k & j)) {
+        const uint32_t lo = (m[k] & mask) | ((m[k + j] & mask) << j);
+        const uint32_t hi = ((m[k] >> j) & mask) | (m[k + j] & ~mask);
+        m[k] = lo;
+        m[k + j] = hi;
+      }
+  }
+}
+
 template <int DIR, int KS>
-__global__ void __launch_bounds__(kSparseWarps * 32) ls_sparse_kernel(const SparseParams p) {
+__global__ void __launch_bounds__(kSparseWarps * 32, 3) ls_sparse_kernel(const __grid_constant__ SparseParams p) {
+  static_assert(KS % 2 == 0, "slots come in pairs");
   constexpr float eps = 2.220446049250313e-16f;
   constexpr int INF_ID = 0x7fffffff;
-  constexpr int CH = kSparseChunk;
+  constexpr int CH = kSparseChunk, NG = sparse_groups(KS), NT = kSparseWarps * 32;
   extern __shared__ __align__(16) unsigned char smem[];
   float* scal = reinterpret_cast<float*>(smem);  // [2][kSparseScal][CH]
-  int* sid_all = reinterpret_cast<int*>(scal + 2 * kSparseScal * CH);
-  float* sval_all = reinterpret_cast<float*>(sid_all + kSparseWarps * 32 * KS);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float* pool_e = scal + 2 * kSparseScal * CH + warp * kSparsePool;  // [64] sums, [64] means
+  unsigned char* mine = smem + (2 * kSparseScal * CH + kSparseWarps * kSparsePool) * 4 + warp * sparse_warp_bytes(KS);
+  uint32_t* words = reinterpret_cast<uint32_t*>(mine) + lane;  // [locus][group] x 32 lanes
+  int* sid = reinterpret_cast<int*>(mine);                     // window changes: the old set's ids and values
+  float* sval = reinterpret_cast<float*>(mine) + 32 * KS;
   const int i_raw = p.t_begin + blockIdx.x * kSparseWarps + warp;
   const bool active = i_raw < p.t_begin + p.t_count;
   const int i = active ? i_raw : p.t_begin;  // idle warps shadow a valid target and write nothing
-  int* sid = sid_all + warp * 32 * KS;
-  float* sval = sval_all + warp * 32 * KS;
   const int K = p.K, L = p.L, N = p.N;
   const float pi = 1.0f / (float)(N - 1);  // dense uniform prior
 
-  int id[KS];
-  float x[KS];
-  // mismatch words of the current block: bit k of mm[s] is 1 where entry s's donor differs from the
-  // target at locus 32 b + k.  Padding entries (id -1) get all ones: they are updated like
-  // mismatching donors, all start at 0 when their window starts and so hold one common value xs,
-  // which the row sum subtracts (no per-entry branch in the locus loop).
-  uint32_t mm[KS];
-  uint32_t twd = 0u;  // the target's own word of the block
+  float2 x2[KS / 2];  // slots 2k and 2k + 1
+  auto X = [&](int s) -> float& { return (s & 1) ? x2[s >> 1].y : x2[s >> 1].x; };
   float xs = 0.0f;
   int cur_w = -1;
+  int n_enter = 0, nset = 0;  // set entries are indices 0 .. nset - 1
+  uint32_t pad[NG];           // bit s: slot 32 g + s is padding
   auto warp_sum = [&](float v) {
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
@@ -121,29 +154,75 @@ __global__ void __launch_bounds__(kSparseWarps * 32) ls_sparse_kernel(const Spar
     const int q = 32 * s + lane;
     return q < K ? p.idx[((size_t)i * p.Wn + w) * K + q] : -1;
   };
-  // the words of block b (loci 32 b .. 32 b + 31) for the current set
-  auto gather = [&](int b) {
-    const uint32_t* hwb = p.hw + (size_t)(b >> 3) * N * 8 + (b & 7);
-    twd = hwb[(size_t)i * 8];
+  // the words of block b (loci 64 b .. 64 b + 63) for the current set, and the outside donors' emissions
+  // (sc: the block's constants)
+  auto gather = [&](int b, const float* sc) {
+    __syncwarp();
+    const uint32_t* hwb = p.hw + (size_t)(b >> 2) * N * 8 + 2 * (b & 3);
+    const uint2 tw = *reinterpret_cast<const uint2*>(hwb + (size_t)i * 8);
 #pragma unroll
-    for (int s = 0; s < KS; ++s) mm[s] = id[s] >= 0 ? (hwb[(size_t)id[s] * 8] ^ twd) : 0xffffffffu;
+    for (int g = 0; g < NG; ++g) {
+      uint32_t lo[32], hi[32];
+#pragma unroll
+      for (int s = 0; s < 32; ++s) {
+        lo[s] = hi[s] = 0u;
+        if (32 * g + s < KS) {
+          const int id = set_entry(cur_w, 32 * g + s);
+          uint2 v = make_uint2(~tw.x, ~tw.y);  // padding differs everywhere
+          if (id >= 0) v = *reinterpret_cast<const uint2*>(hwb + (size_t)id * 8);
+          lo[s] = v.x ^ tw.x;
+          hi[s] = v.y ^ tw.y;
+        }
+      }
+      transpose32(lo);
+#pragma unroll
+      for (int k = 0; k < 32; ++k) words[(k * NG + g) * 32] = lo[k];
+      transpose32(hi);
+#pragma unroll
+      for (int k = 0; k < 32; ++k) words[((32 + k) * NG + g) * 32] = hi[k];
+    }
+    if (p.pool) {
+      const int nout = N - 1 - nset;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        int mis = 0;  // slots (padding included) that differ from the target at locus 32 h + lane
+#pragma unroll 8
+        for (int k = 0; k < 32; ++k) {
+          int n = 0;
+#pragma unroll
+          for (int g = 0; g < NG; ++g) n += __popc(words[((32 * h + k) * NG + g) * 32]);
+          n = __reduce_add_sync(0xffffffffu, n);
+          if (lane == k) mis = n;
+        }
+        const int kr = 32 * h + lane;
+        const int n1 = __float_as_int(sc[2 * CH + kr]);
+        const int mtot = (((h ? tw.y : tw.x) >> lane) & 1u ? n1 : N - n1) - 1;  // matching donors, the target excluded
+        const int mout = min(max(mtot - (32 * KS - mis), 0), nout);
+        const float q = sc[3 * CH + kr];
+        const float thsum = signbit(q) ? -q * (float)mout + (float)(nout - mout) : (float)mout + q * (float)(nout - mout);
+        pool_e[kr] = thsum;
+        pool_e[CH + kr] = nout > 0 ? thsum / (float)nout : 0.0f;
+      }
+      __syncwarp();
+    }
   };
   // exact sum of the set's values, in the order the window map sums them
   auto set_sum = [&]() -> float {
     float v = 0.0f;
 #pragma unroll
-    for (int s = 0; s < KS; ++s) v += id[s] >= 0 ? x[s] : 0.0f;
+    for (int s = 0; s < KS; ++s) v += 32 * s + lane < nset ? X(s) : 0.0f;
     return warp_sum(v);
   };
   // enter window w: map the values of the old set onto the new one (`fill` for new donors); returns
   // the mapped total, and the number of entering donors and of set entries
-  int n_enter = 0, nset = 0;
   auto enter = [&](int w, bool map, float fill) -> float {
+    __syncwarp();
     if (map) {
 #pragma unroll
       for (int s = 0; s < KS; ++s) {
-        sid[32 * s + lane] = id[s] >= 0 ? id[s] : INF_ID;
-        sval[32 * s + lane] = x[s];
+        const int id = set_entry(cur_w, s);
+        sid[32 * s + lane] = id >= 0 ? id : INF_ID;
+        sval[32 * s + lane] = X(s);
       }
       __syncwarp();
     }
@@ -151,16 +230,16 @@ __global__ void __launch_bounds__(kSparseWarps * 32) ls_sparse_kernel(const Spar
     int ne = 0, nv = 0;
 #pragma unroll
     for (int s = 0; s < KS; ++s) {
-      id[s] = set_entry(w, s);
+      const int id = set_entry(w, s);
       float v = 0.0f;
-      if (map && id[s] >= 0) {
+      if (map && id >= 0) {
         int lo = 0, hi = 32 * KS;  // first position with sid >= id
         while (lo < hi) {
           const int mid = (lo + hi) >> 1;
-          if (sid[mid] < id[s]) lo = mid + 1;
+          if (sid[mid] < id) lo = mid + 1;
           else hi = mid;
         }
-        if (lo < 32 * KS && sid[lo] == id[s]) {
+        if (lo < 32 * KS && sid[lo] == id) {
           v = sval[lo];
           mapped += v;
         } else {
@@ -168,38 +247,63 @@ __global__ void __launch_bounds__(kSparseWarps * 32) ls_sparse_kernel(const Spar
           ++ne;
         }
       }
-      nv += id[s] >= 0;
-      x[s] = v;
+      nv += id >= 0;
+      X(s) = v;
     }
-    if (map) __syncwarp();
+    __syncwarp();
     cur_w = w;
-    xs = 0.0f;  // every padding entry restarts at 0
+    xs = 0.0f;  // every padding slot restarts at 0
     n_enter = __reduce_add_sync(0xffffffffu, ne);
     nset = __reduce_add_sync(0xffffffffu, nv);
+#pragma unroll
+    for (int g = 0; g < NG; ++g) {
+      const int have = min(max((nset - lane + 31) / 32 - 32 * g, 0), 32);  // this lane's set entries in the group
+      pad[g] = have == 32 ? 0u : 0xffffffffu << have;
+    }
     return warp_sum(mapped);
   };
 
   double logacc = 0.0;
+  float keep = 1.0f;      // lane k: the normaliser of the k-th locus since the last fold
+  int nkeep = 0;
   uint32_t stb = 0u;
+  // the kept normalisers: status bits, and (forward) their logarithms summed with an exact error term per
+  // addition into the double accumulator
+  auto fold = [&]() {
+    if (keep < 1.17549435e-38f) stb |= 1u;      // LS_STATUS_UNDERFLOW
+    if (!(keep <= 3.40282347e+38f)) stb |= 2u;  // LS_STATUS_OVERFLOW (infinite or NaN)
+    if (DIR == 0) {
+      float v = logf(keep), e = 0.0f;
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) {
+        const float vo = __shfl_xor_sync(0xffffffffu, v, off), eo = __shfl_xor_sync(0xffffffffu, e, off);
+        const float t = __fadd_rn(v, vo), bb = __fsub_rn(t, v);
+        e = __fadd_rn(__fadd_rn(e, eo), __fadd_rn(__fsub_rn(v, __fsub_rn(t, bb)), __fsub_rn(vo, bb)));
+        v = t;
+      }
+      logacc += (double)v + (double)e;
+    }
+    keep = 1.0f;
+    nkeep = 0;
+  };
   float lost_max = 0.0f;
   float sum_prev = 1.0f;  // forward: sum alpha; backward: sum t (set plus pool)
   float opool = 0.0f;     // outside pool (pool = 1)
   int store_next = 0;
-  // blocks of CH loci aligned to multiples of CH, in processing order; the per-locus constants of
-  // the next block are copied asynchronously (cp.async) while the current one is processed
+  // blocks of CH loci aligned to multiples of CH, in processing order
   const int nb = (L + CH - 1) / CH;
   auto blk_of = [&](int t) { return DIR == 0 ? t : nb - 1 - t; };
   auto issue = [&](int t) {
-    const int b = blk_of(t), base = CH * b, nrows = min(CH, L - base);
-    const int f = threadIdx.x / CH, k = threadIdx.x % CH, l = base + k;
-    if (threadIdx.x < kSparseScal * CH && k < nrows) {
+    const int base = CH * blk_of(t), nrows = min(CH, L - base);
+    for (int e = threadIdx.x; e < kSparseScal * CH; e += NT) {
+      const int f = e / CH, k = e % CH, l = base + k;
+      if (k >= nrows) continue;
       const int m = DIR == 0 ? l - 1 : l;  // interval entering locus l in processing order
       float* d = scal + ((t & 1) * kSparseScal + f) * CH + k;
-      if (f == 0) cp_async4(d, p.thm + l);
-      else if (f == 1) cp_async4(d, p.thx + l);
-      else if (f == 2 && m >= 0 && m < L - 1) cp_async4(d, p.omr + m);
-      else if (f == 3 && m >= 0 && m < L - 1) cp_async4(d, p.rho + m);
-      else if (f == 4 && p.n1) cp_async4(d, p.n1 + l);
+      if (f == 0 && m >= 0 && m < L - 1) cp_async4(d, p.omr + m);
+      else if (f == 1 && m >= 0 && m < L - 1) cp_async4(d, p.rho + m);
+      else if (f == 2 && p.n1) cp_async4(d, p.n1 + l);
+      else if (f == 3) cp_async4(d, p.ratio + l);
     }
   };
   issue(0);
@@ -218,11 +322,10 @@ __global__ void __launch_bounds__(kSparseWarps * 32) ls_sparse_kernel(const Spar
     // branches.
     auto body = [&](const int jj, auto evc) {
       constexpr bool EV = decltype(evc)::value;
-      const int kr = DIR == 0 ? jj : nrows - 1 - jj;  // locus l = base + kr is bit kr of the words
+      const int kr = DIR == 0 ? jj : nrows - 1 - jj;  // locus l = base + kr
       const int l = base + kr;
-      const int w = l / p.WS;
-      const float tm = sc[0 * CH + kr], tx = sc[1 * CH + kr];
       float c, r;
+      const int w = EV ? l / p.WS : cur_w;
       if (EV && cur_w < 0) {  // initial locus: alpha = theta pi ; t = theta (beta = 1)
         enter(w, false, 0.0f);
         need_gather = true;
@@ -238,7 +341,7 @@ __global__ void __launch_bounds__(kSparseWarps * 32) ls_sparse_kernel(const Spar
           if (p.pool) opool = fmaxf(opool + (s_set - mapped) - (float)n_enter * fill, 0.0f);
           need_gather = true;
         }
-        const float om = sc[2 * CH + kr], rh = sc[3 * CH + kr];  // interval entering locus l
+        const float om = sc[kr], rh = sc[CH + kr];  // interval entering locus l
         if (DIR == 0) {
           c = om / sum_prev;
           r = rh * pi;
@@ -249,11 +352,9 @@ __global__ void __launch_bounds__(kSparseWarps * 32) ls_sparse_kernel(const Spar
         }
       }
       if (EV && need_gather) {
-        gather(b);
+        gather(b, sc);
         need_gather = false;
       }
-      const uint32_t tb = (twd >> kr) & 1u;
-      const uint32_t mk = 1u << kr;
       const bool is_store = EV && store_next < p.n_store && p.store_loci[store_next] == l;
       float* srow = is_store ? p.store + ((size_t)p.store_slot[store_next] * N + i) * K : nullptr;
       if (DIR == 1 && is_store) {
@@ -264,7 +365,7 @@ __global__ void __launch_bounds__(kSparseWarps * 32) ls_sparse_kernel(const Spar
 #pragma unroll
         for (int q = 0; q < KS; ++q) {
           const int sq = 32 * q + lane;
-          if (sq < K && id[q] >= 0) zb += srow[sq] * (fmaf(c, x[q], r) * S);
+          if (sq < nset) zb += srow[sq] * (fmaf(c, X(q), r) * S);
         }
         zb = warp_sum(zb);
         const int nout = N - 1 - nset;
@@ -276,48 +377,51 @@ __global__ void __launch_bounds__(kSparseWarps * 32) ls_sparse_kernel(const Spar
         for (int q = 0; q < KS; ++q) {
           const int sq = 32 * q + lane;
           if (active && sq < K)
-            srow[sq] = id[q] < 0 ? 0.0f : (z > 0.0f ? srow[sq] * (fmaf(c, x[q], r) * S) * inv : eps);
+            srow[sq] = sq >= nset ? 0.0f : (z > 0.0f ? srow[sq] * (fmaf(c, X(q), r) * S) * inv : eps);
         }
         if (p.pool && active && lane == 0) p.share[so] = (nout > 0 && z > 0.0f) ? zp * inv / (float)nout : 0.0f;
         if (p.pout && active && lane == 0) p.pout[so] = z > 0.0f ? zp * inv : 0.0f;
       }
-      float s = 0.0f;
-      int nmatch = 0;  // set entries matching the target's allele
+      const float qr = sc[3 * CH + kr], ur = fabsf(qr);
+      const uint32_t flip = signbit(qr) ? 0xffffffffu : 0u;  // mu > 1/2: the matches carry the smaller factor
+      const float2 C2 = make_float2(c, c), R2 = make_float2(r, r);
+      float2 acc[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
 #pragma unroll
-      for (int q = 0; q < KS; ++q) {
-        const bool mis = (mm[q] & mk) != 0u;
-        nmatch += mis ? 0 : 1;
-        x[q] = (mis ? tx : tm) * fmaf(c, x[q], r);  // theta (c x + r)
-        s += x[q];
+      for (int g = 0; g < NG; ++g) {
+        const uint32_t wd = words[(kr * NG + g) * 32];
+        const uint32_t sm = (wd ^ flip) | pad[g];
+#pragma unroll
+        for (int s = 0; s < 32; s += 2) {
+          const int k = (32 * g + s) >> 1;
+          if (32 * g + s < KS) {
+            float2 u = __ffma2_rn(C2, x2[k], R2);
+            if ((sm >> s) & 1u) u.x = __fmul_rn(u.x, ur);
+            if ((sm >> (s + 1)) & 1u) u.y = __fmul_rn(u.y, ur);
+            x2[k] = u;
+            acc[k & 3] = __fadd2_rn(acc[k & 3], u);
+          }
+        }
       }
-      xs = tx * fmaf(c, xs, r);
-      s = warp_sum(s) - (float)(32 * KS - nset) * xs;
-      float tot = s;
+      xs = __fmul_rn(__fmaf_rn(c, xs, r), ur);  // padding slots: always the smaller factor
+      acc[0] = __fadd2_rn(__fadd2_rn(acc[0], acc[2]), __fadd2_rn(acc[1], acc[3]));
+      float tot = warp_sum(acc[0].x + acc[0].y) - (float)(32 * KS - nset) * xs;
       if (p.pool) {
-        // outside donors: their count, how many match the target here, their summed emission
-        const int n1 = __float_as_int(sc[4 * CH + kr]);
-        const int mtot = (tb ? n1 : N - n1) - 1;  // matching donors, the target itself excluded
-        const int nout = N - 1 - nset;
-        const int mout = min(max(mtot - __reduce_add_sync(0xffffffffu, nmatch), 0), nout);
-        const float thsum = tm * (float)mout + tx * (float)(nout - mout);
-        const float thbar = nout > 0 ? thsum / (float)nout : 0.0f;
-        opool = thbar * (c * opool) + r * thsum;
-        tot = s + opool;
+        opool = pool_e[CH + kr] * (c * opool) + r * pool_e[kr];
+        tot += opool;
       }
       if (is_store) {
         if (DIR == 0) {
 #pragma unroll
           for (int q = 0; q < KS; ++q) {
             const int sq = 32 * q + lane;
-            if (active && sq < K) srow[sq] = id[q] >= 0 ? x[q] : 0.0f;
+            if (active && sq < K) srow[sq] = sq < nset ? X(q) : 0.0f;
           }
           if (p.pool && active && lane == 0) p.poolf[(size_t)p.store_slot[store_next] * N + i] = opool;
         }
         ++store_next;
       }
-      if (tot < 1.17549435e-38f) stb |= 1u;      // LS_STATUS_UNDERFLOW
-      if (!(tot <= 3.40282347e+38f)) stb |= 2u;  // LS_STATUS_OVERFLOW (infinite or NaN)
-      if (DIR == 0) logacc += (double)logf(tot);
+      if (lane == nkeep) keep = tot;
+      if (++nkeep == 32) fold();
       sum_prev = tot;
     };
     for (int jj = 0; jj < nrows;) {
@@ -335,11 +439,21 @@ __global__ void __launch_bounds__(kSparseWarps * 32) ls_sparse_kernel(const Spar
       for (; jj < ev; ++jj) body(jj, std::false_type{});
     }
   }
+  fold();
+  stb = __reduce_or_sync(0xffffffffu, stb);
   if (active && lane == 0) {
-    if (DIR == 0 && p.logs) p.logs[i] = logacc;
+    if (DIR == 0 && p.logs) p.logs[i] = logacc + p.log_base;
     if (DIR == 0 && p.lost) p.lost[i] = lost_max;
     if (p.status && stb) atomicOr(p.status + i, stb);
   }
+}
+
+// SparseParams::ratio
+__global__ void emission_kernel(const float* __restrict__ thm, const float* __restrict__ thx, int L, float* __restrict__ ratio) {
+  const int l = blockIdx.x * blockDim.x + threadIdx.x;
+  if (l >= L) return;
+  const float a = thm[l], b = thx[l];
+  ratio[l] = a < b ? -__fdiv_rn(a, b) : __fdiv_rn(b, a);  // 1 - mu and mu: the larger is at least 1/2
 }
 
 // Half distances -log(max(p, eps))/2 of the sparse posteriors into dense [D][N][N] rows.  Every
