@@ -34,7 +34,11 @@ cudaError_t ls_launch_emission(const float* thm, const float* thx, int L, float*
 
 cudaError_t ls_launch_lookahead(const int32_t* idx, int N, int Wn, int K, int span, int32_t* U, cudaStream_t s) {
   const long long n = (long long)N * Wn;
-  lsk::lookahead_sets_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(idx, N, Wn, K, span, U);
+  // up to eight warps a CTA, as many as 48 KB of bitmaps allow (beyond N = 393216 one warp and more)
+  const int bytes = (N + 31) / 32 * 4, warps = bytes * 8 <= 48 * 1024 ? 8 : bytes < 48 * 1024 ? 48 * 1024 / bytes : 1;
+  cudaError_t e = cudaFuncSetAttribute(lsk::lookahead_sets_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, warps * bytes);
+  if (e != cudaSuccess) return e;
+  lsk::lookahead_sets_kernel<<<(unsigned)((n + warps - 1) / warps), warps * 32, warps * bytes, s>>>(idx, N, Wn, K, span, U);
   return cudaGetLastError();
 }
 
@@ -47,7 +51,7 @@ cudaError_t ls_launch_sparse_hdist(const float* P, const int32_t* idx, int N, in
 cudaError_t ls_launch_symmetrize_trust(float* d, int N, int D, const uint8_t* dense_row, float d_trust, uint32_t* mask,
                                        cudaStream_t s) {
   const int nt = (N + 31) / 32;
-  lsk::symmetrize_trust_kernel<<<dim3(nt, nt, D), dim3(32, 8), 0, s>>>(d, N, dense_row, d_trust, mask, nt);
+  lsk::symmetrize_trust_kernel<<<dim3(nt, nt, D), dim3(32, 4), 0, s>>>(d, N, dense_row, d_trust, mask, nt);
   return cudaGetLastError();
 }
 
