@@ -35,6 +35,7 @@ void ls_register_group14(std::vector<PropKernelInfo>& out);
 void ls_register_group15(std::vector<PropKernelInfo>& out);
 void ls_register_group16(std::vector<PropKernelInfo>& out);
 void ls_register_group17(std::vector<PropKernelInfo>& out);
+void ls_register_group18(std::vector<PropKernelInfo>& out);
 
 namespace {
 
@@ -78,6 +79,7 @@ std::vector<PropKernelInfo>& registry() {
     ls_register_group15(v);
     ls_register_group16(v);
     ls_register_group17(v);
+    ls_register_group18(v);
   });
   return v;
 }

@@ -259,6 +259,12 @@ __host__ __device__ __forceinline__ void slice_of(int sigma, int S, int N, int& 
 // indicator) the recursion is the forward one plus a source:
 //   w_j <- theta_j (c w_j + r (W/s + gamma)) + eta H_j x_j,   W = sum_j w_j, s = sum_j x_j.
 // ST 1 takes the recombination term (restarted at every group of intervals), ST 2 the mismatch term.
+template <int W>
+__device__ __forceinline__ void cta_sync() {
+  if (W == 1) __syncwarp();
+  else __syncthreads();
+}
+
 template <int DIR, int TPW, int W, int KQ, int PIM, int ST>
 __global__ void __launch_bounds__(W * 32, ((PIM || ST) && W >= 8) ? 1 : 2) ls_prop_kernel(const PropParams p) {
   static_assert(ST == 0 || (DIR == 0 && PIM == 0), "statistic passes run forward with the uniform prior");
@@ -414,22 +420,24 @@ __global__ void __launch_bounds__(W * 32, ((PIM || ST) && W >= 8) ? 1 : 2) ls_pr
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   // emission table of step 0 (for scalar mu it serves every step)
-  if (tid < 64) {
-    const int e = tid >> 2, k = tid & 3;
+  auto lut_entry = [&](int q) {
+    const int e = q >> 2, k = q & 3;
     if (UNI) {
       const float a = p.thm[p.l_first], b = p.thx[p.l_first];
       const float bs = fmaxf(a, b);
-      lutf[tid] = ((e >> k) & 1) ? 1.0f : (bs > 0.0f ? __fdiv_rn(fminf(a, b), bs) : 0.0f);
+      lutf[q] = ((e >> k) & 1) ? 1.0f : (bs > 0.0f ? __fdiv_rn(fminf(a, b), bs) : 0.0f);
     } else {
-      lutf[tid] = ((e >> k) & 1) ? p.thm[p.l_first] : p.thx[p.l_first];
+      lutf[q] = ((e >> k) & 1) ? p.thm[p.l_first] : p.thx[p.l_first];
     }
-    if (ST == 2) s_hlut[0][tid] = ((e >> k) & 1) ? 0.0f : (p.eta_vec ? p.eta_vec[p.l_first] : p.eta);
-  }
+    if (ST == 2) s_hlut[0][q] = ((e >> k) & 1) ? 0.0f : (p.eta_vec ? p.eta_vec[p.l_first] : p.eta);
+  };
+  if (THREADS < 64) lut_entry(tid + 32);
+  if (tid < 64) lut_entry(tid);
   if (tid < TPW) {
     lgs[tid] = (cta_t + tid < t_end && p.logs && !p.init) ? p.logs[row0 + tid] : 0.0;
     sts[tid] = 0u;
   }
-  __syncthreads();
+  cta_sync<W>();
   if (tid == 0)
     for (int B = 0; B < kSlots && B < nblk; ++B) issue(B);
 
@@ -444,7 +452,7 @@ __global__ void __launch_bounds__(W * 32, ((PIM || ST) && W >= 8) ? 1 : 2) ls_pr
 #pragma unroll
     for (int c = 0; c < C::NCHUNK; ++c) {
       xfer(c, const_cast<float*>(src), nullptr, nullptr, nullptr, false);
-      __syncthreads();
+      cta_sync<W>();
 #pragma unroll
       for (int q = 0; q < 8; ++q) {
         const int k = 8 * c + q;
@@ -461,7 +469,7 @@ __global__ void __launch_bounds__(W * 32, ((PIM || ST) && W >= 8) ? 1 : 2) ls_pr
           }
         }
       }
-      __syncthreads();
+      cta_sync<W>();
     }
   };
   if (p.load_state) {
@@ -485,7 +493,7 @@ __global__ void __launch_bounds__(W * 32, ((PIM || ST) && W >= 8) ? 1 : 2) ls_pr
       if (PIM == 2) my16[s2] = (uint16_t)(__float_as_uint(v) >> 16);  // bfloat16 already: exact
       else my[s2] = v;
     }
-    __syncthreads();
+    cta_sync<W>();
   }
 
   // store the tile (mode 0: x; 1: c x + r; 2: multiply the destination by c x + r)
@@ -505,9 +513,9 @@ __global__ void __launch_bounds__(W * 32, ((PIM || ST) && W >= 8) ? 1 : 2) ls_pr
           *reinterpret_cast<float4*>(stg + tid * C::STG_STRIDE + 4 * q) = make_float4(a.x, a.y, b.x, b.y);
         }
       }
-      __syncthreads();
+      cta_sync<W>();
       xfer(cc, nullptr, w1, m1, w2, true);
-      __syncthreads();
+      cta_sync<W>();
     }
   };
 
@@ -521,16 +529,21 @@ __global__ void __launch_bounds__(W * 32, ((PIM || ST) && W >= 8) ? 1 : 2) ls_pr
       v += __shfl_xor_sync(0xffffffffu, v, off);
       if (ST) u += __shfl_xor_sync(0xffffffffu, u, off);
     }
+    if (W == 1) {  // the warp holds the whole target: every lane has its total
+      __syncwarp();  // publishes the next locus' emission table, frees the ring slot read last
+      tu = u;
+      return v;
+    }
     if (LS_X_RED4 && !ST && W == 4) {  // the W partials of target tl in one 16-byte load
       if (sl == 0) buf[tl * W + warp] = v;
-      __syncthreads();
+      cta_sync<W>();
       const float4 e = *reinterpret_cast<const float4*>(buf + tl * W);
       tu = 0.0f;
       return (e.x + e.y) + (e.z + e.w);
     }
     float2* b2 = reinterpret_cast<float2*>(buf);
     if (sl == 0) b2[tl * W + warp] = make_float2(v, u);
-    __syncthreads();
+    cta_sync<W>();
     float t = 0.0f;
     tu = 0.0f;
 #pragma unroll
@@ -590,7 +603,7 @@ __global__ void __launch_bounds__(W * 32, ((PIM || ST) && W >= 8) ? 1 : 2) ls_pr
       for (int k = 0; k < (ST ? KQ : 1); ++k) sw += (wv[k][0].x + wv[k][0].y) + (wv[k][1].x + wv[k][1].y);
     }
     sig_prev = reduce2(s, sw, part + 2 * TPW * W, wsum_prev);
-    __syncthreads();
+    cta_sync<W>();
   }
 
   // per-step scalars, loaded one step ahead
@@ -849,14 +862,18 @@ __global__ void __launch_bounds__(W * 32, ((PIM || ST) && W >= 8) ? 1 : 2) ls_pr
 
     // emission table of the next locus (mu varying per locus), into the other buffer
     if (MUV && tid < 64 && step + 1 < p.n_steps) {
-      const int e = tid >> 2, k = tid & 3;
-      if (UNI) {
-        const float bs = fmaxf(nx_thm, nx_thx);
-        lutf[((step + 1) & 1) * 64 + tid] = ((e >> k) & 1) ? 1.0f : (bs > 0.0f ? __fdiv_rn(fminf(nx_thm, nx_thx), bs) : 0.0f);
-      } else {
-        lutf[((step + 1) & 1) * 64 + tid] = ((e >> k) & 1) ? nx_thm : nx_thx;
-      }
-      if (ST == 2) s_hlut[(step + 1) & 1][tid] = ((e >> k) & 1) ? 0.0f : p.eta_vec[l + 1];
+      auto entry = [&](int q) {
+        const int e = q >> 2, k = q & 3;
+        if (UNI) {
+          const float bs = fmaxf(nx_thm, nx_thx);
+          lutf[((step + 1) & 1) * 64 + q] = ((e >> k) & 1) ? 1.0f : (bs > 0.0f ? __fdiv_rn(fminf(nx_thm, nx_thx), bs) : 0.0f);
+        } else {
+          lutf[((step + 1) & 1) * 64 + q] = ((e >> k) & 1) ? nx_thm : nx_thx;
+        }
+        if (ST == 2) s_hlut[(step + 1) & 1][q] = ((e >> k) & 1) ? 0.0f : p.eta_vec[l + 1];
+      };
+      if (THREADS < 64) entry(tid + 32);
+      entry(tid);
     }
 
     float wtot = 0.0f;
@@ -907,7 +924,7 @@ __global__ void __launch_bounds__(W * 32, ((PIM || ST) && W >= 8) ? 1 : 2) ls_pr
       store_tile((pend_slot >= 0 && p.wstore) ? p.wstore + (size_t)pend_slot * p.state_rows * N : nullptr, nullptr,
                  pend_save ? p.wstate : nullptr, false, 0.f, 0.f, true);
   }
-  __syncthreads();  // the log scales and status words were last written by other warps
+  cta_sync<W>();  // the log scales and status words were last written by other warps
   if (tid < TPW && cta_t + tid < t_end) {
     const int row = row0 + tid;
     const uint32_t stb = sts[tid] | (*flag ? 4u : 0u);  // 4 = LS_STATUS_TIMEOUT

@@ -211,6 +211,17 @@ void ls_register_group15(std::vector<PropKernelInfo>& out) {
   LS_REGH2P(8);
   LS_REGH2P(14);
 }
+#elif LS_INST_GROUP == 18
+void ls_register_group18(std::vector<PropKernelInfo>& out) {
+  // one warp per target for N up to 1024: small data sets are bound by the latency of a locus, and a
+  // single warp needs no CTA barrier and no exchange through shared memory (N = 64 / 200 / 500: 0.242 /
+  // 0.250 / 0.261 us per locus against 0.285 / 0.269 / 0.293 for the best four-warp variants).  Beyond
+  // 1024 the four-warp variants are faster (N = 2000: 0.69 against 0.89 us, N = 5000: 3.76 against 3.92).
+  LS_REG(1, 1, 8);
+  LS_REG(1, 1, 4);
+  LS_REG(1, 1, 2);
+  LS_REG(1, 1, 1);
+}
 #elif LS_INST_GROUP == 8
 void ls_register_group8(std::vector<PropKernelInfo>& out) {
   // statistic passes of the adjoint (uniform prior), one target per CTA
