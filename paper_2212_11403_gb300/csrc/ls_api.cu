@@ -109,6 +109,7 @@ uint64_t fnv1a(uint64_t h, const void* data, size_t n) {
 struct Launch {
   const PropKernelInfo* k;
   int t_begin, t_count, grid, smem;
+  int per_sm;  // CTAs an SM holds
 };
 
 struct Cand {
@@ -205,13 +206,14 @@ int plan(ls_ctx* c, int t_begin, int t_count, Launch* out, int* nout) {
     const Cand* bt = best_for(cs, nc, t_count - main_t, c->num_sms, &ct);
     if (cm + ct < c1) {
       const int tt = t_count - main_t;
-      out[0] = Launch{b1->k, t_begin, main_t, main_t / b1->k->tpw, b1->smem};
-      out[1] = Launch{bt->k, t_begin + main_t, tt, (tt + bt->k->tpw - 1) / bt->k->tpw, bt->smem};
+      out[0] = Launch{b1->k, t_begin, main_t, main_t / b1->k->tpw, b1->smem, b1->per_sm};
+      out[1] = Launch{bt->k, t_begin + main_t, tt, (tt + bt->k->tpw - 1) / bt->k->tpw, bt->smem,
+                      bt->per_sm};
       *nout = 2;
       return LS_OK;
     }
   }
-  out[0] = Launch{b1->k, t_begin, t_count, (t_count + b1->k->tpw - 1) / b1->k->tpw, b1->smem};
+  out[0] = Launch{b1->k, t_begin, t_count, (t_count + b1->k->tpw - 1) / b1->k->tpw, b1->smem, b1->per_sm};
   *nout = 1;
   return LS_OK;
 }
@@ -234,6 +236,15 @@ void base_params(ls_ctx* c, lsk::PropParams& p, int dir) {
   p.err = c->err;
 }
 
+// the side stream and the events that fork it from and join it to a caller's stream
+int side_stream(ls_ctx* c) {
+  if (c->side) return LS_OK;
+  CUDA_TRY(cudaEventCreateWithFlags(&c->fork_ev, cudaEventDisableTiming));
+  CUDA_TRY(cudaEventCreateWithFlags(&c->join_ev, cudaEventDisableTiming));
+  CUDA_TRY(cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking));
+  return LS_OK;
+}
+
 int run_launches(ls_ctx* c, lsk::PropParams p, int t_begin, int t_count, cudaStream_t s, int* nlaunch = nullptr) {
   Launch lp[2];
   int nlp = 0;
@@ -245,11 +256,7 @@ int run_launches(ls_ctx* c, lsk::PropParams p, int t_begin, int t_count, cudaStr
   // LS_TAIL_OVERLAP=0 (a measurement switch) runs both on the caller's stream, in order.
   const char* ov = getenv("LS_TAIL_OVERLAP");
   if (nlp == 2 && !(ov && ov[0] == '0')) {
-    if (!c->side) {
-      CUDA_TRY(cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking));
-      CUDA_TRY(cudaEventCreateWithFlags(&c->fork_ev, cudaEventDisableTiming));
-      CUDA_TRY(cudaEventCreateWithFlags(&c->join_ev, cudaEventDisableTiming));
-    }
+    if ((rc = side_stream(c))) return rc;
     CUDA_TRY(cudaEventRecord(c->fork_ev, s));
     CUDA_TRY(cudaStreamWaitEvent(c->side, c->fork_ev, 0));
     for (int k = 1; k >= 0; --k) {
@@ -323,10 +330,10 @@ void launch_posterior(const lsk::PostArgs& a, dim3 grid, cudaStream_t s) {
 }
 template <int DEC>
 int launch_posterior(const lsk::PostArgs& a, dim3 grid, cudaStream_t s) {
-  const bool quads = row_quads(a.N, a.out) && (DEC || row_quads(a.N, a.alpha, a.beta));
+  const bool quads = row_quads(a.N, a.out, a.beta) && (DEC || row_quads(a.N, a.alpha));
   if (quads && a.N <= 2048) launch_posterior<DEC, 2>(a, grid, s);
   else if (quads && a.N <= 5120) launch_posterior<DEC, 5>(a, grid, s);
-  else if (DEC) lsk::decode_kernel<<<grid, 256, 0, s>>>(a.out, a.N, a.bits, a.row_words, a.thm, a.thx, a.dl);
+  else if (DEC) lsk::decode_kernel<<<grid, 256, 0, s>>>(a.out, a.beta, a.N, a.bits, a.row_words, a.thm, a.thx, a.dl);
   else if (quads && a.N <= 20480) launch_posterior<0, 10>(a, grid, s);
   else if (quads && a.N <= lsk::kRowMaxPostN) launch_posterior<0, 16>(a, grid, s);
   else lsk::posterior_kernel<<<grid, 256, 0, s>>>(a.alpha, a.beta, a.N, a.t0, a.mode, a.out);
@@ -345,10 +352,12 @@ int posterior_rows(const float* alpha, const float* beta, int N, int t0, int T, 
   a.mode = mode;
   return launch_posterior<0>(a, dim3(T), s);
 }
-// the backward's products at D decode loci into half distances, in place
-int decode_rows(const ls_ctx* c, const int32_t* loci, int D, float* d, cudaStream_t s) {
+// the backward's products at D decode loci into half distances, in place; with t given, d holds alpha and t
+// the backward's values times 2^100
+int decode_rows(const ls_ctx* c, const int32_t* loci, int D, float* d, const float* t, cudaStream_t s) {
   lsk::PostArgs a = {};
   a.out = d;
+  a.beta = t;
   a.N = c->N;
   a.bits = c->bits;
   a.row_words = c->row_words;
@@ -398,6 +407,7 @@ void free_ctx(ls_ctx* c) {
   cudaFree(c->status_scratch);
   cudaFree(c->err);
   cudaFree(c->dscratch);
+  cudaFree(c->tscratch);
   for (auto& e : c->ev)
     if (e) cudaEventDestroy(e);
   if (c->fork_ev) cudaEventDestroy(c->fork_ev);
@@ -981,6 +991,45 @@ int ls_distance(ls_ctx* ctx, const ls_table* fwd, const ls_table* bck, float* d_
   return LS_OK;
 }
 
+// Small data sets leave most of the GPU idle and are bound by the latency of a locus, so ls_run_all runs
+// their two directions side by side: where each is one launch and all CTAs of both are resident at once
+// (one-warp and 8-target CTAs: N up to 1216).  The backward then leaves t 2^100 at the decode loci in
+// scratch of the context (at most kPairBytes, kept until the context is destroyed) and the decode forms the
+// product alpha (t 2^100) that it otherwise finds.  Not while profiling (the phases are timed one after
+// the other), with LS_TAIL_OVERLAP=0, or where the scratch would have to be allocated during a capture.
+// N = 200 / 500 / 1003 / 1200, L = 4000: 2087 / 2175 / 2897 /
+// 3445 -> 1107 / 1262 / 1931 / 2469 us.
+static constexpr size_t kPairBytes = (size_t)256 << 20;
+
+// whether to run the directions side by side, with the scratch for it
+static int plan_pair(ls_ctx* c, int D, cudaStream_t s, bool* both) {
+  *both = false;
+  const char* ov = getenv("LS_TAIL_OVERLAP");
+  const size_t n = (size_t)D * c->N * c->N, bytes = sizeof(float) * n;
+  if (c->profile || (ov && ov[0] == '0') || bytes > kPairBytes) return LS_OK;
+  Launch lp[2];
+  int nlp = 0, rc = plan(c, 0, c->N, lp, &nlp);
+  if (rc) return rc;
+  if (nlp != 1 || 2 * lp[0].grid * lp[0].k->cpt > lp[0].per_sm * c->num_sms) return LS_OK;
+  if (!c->side || c->tscratch_bytes < bytes) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    CUDA_TRY(cudaStreamIsCapturing(s, &cap));
+    if (cap != cudaStreamCaptureStatusNone) return LS_OK;
+    if ((rc = side_stream(c))) return rc;
+    if (c->tscratch_bytes < bytes) {
+      // an earlier call's work on the old scratch may still run on its stream: cudaFree waits for it
+      cudaFree(c->tscratch);
+      c->bytes -= c->tscratch_bytes;
+      c->tscratch = nullptr;
+      c->tscratch_bytes = 0;
+      if (dev_alloc(c, (void**)&c->tscratch, bytes) != LS_OK) return LS_OK;  // no memory to spare: one after the other
+      c->tscratch_bytes = bytes;
+    }
+  }
+  *both = true;
+  return LS_OK;
+}
+
 int ls_run_all(ls_ctx* ctx, const int32_t* decode_loci, int32_t D, float* d_out, double* pac_out, uint32_t* status_out,
                ls_stream_t stream) {
   int rc = check_ctx(ctx);
@@ -1011,6 +1060,18 @@ int ls_run_all(ls_ctx* ctx, const int32_t* decode_loci, int32_t D, float* d_out,
   uint32_t* stat = ctx->status_scratch;
   CUDA_TRY(cudaMemsetAsync(stat, 0, sizeof(uint32_t) * N, s));
   const bool prof = ctx->profile;
+  bool both = false;  // the directions side by side
+  if ((rc = plan_pair(ctx, D, s, &both))) return rc;
+  cudaStream_t sb = both ? ctx->side : s;  // the backward's stream
+  if (both) {
+    CUDA_TRY(cudaEventRecord(ctx->fork_ev, s));
+    CUDA_TRY(cudaStreamWaitEvent(sb, ctx->fork_ev, 0));
+    if (D > 0) {  // the backward multiplies what it finds at the decode loci by t 2^100
+      const long long n = (long long)D * N * N;
+      lsk::fill_kernel<<<(unsigned)std::min<long long>((n + 1023) / 1024, 4096), 256, 0, sb>>>(ctx->tscratch, n, 1.0f);
+      CUDA_TRY(cudaGetLastError());
+    }
+  }
   if (prof) CUDA_TRY(cudaEventRecord(ctx->ev[0], s));
   // forward over all loci: alpha at the decode loci goes straight into the output buffer
   lsk::PropParams p;
@@ -1043,12 +1104,16 @@ int ls_run_all(ls_ctx* ctx, const int32_t* decode_loci, int32_t D, float* d_out,
     p.store_loci[k] = decode_loci[D - 1 - k];
     p.store_slot[k] = D - 1 - k;
   }
-  p.alpha_dec = dd;
-  if ((rc = run_launches(ctx, p, 0, N, s, &ctx->launches[1]))) return rc;
+  p.alpha_dec = both ? ctx->tscratch : dd;
+  if ((rc = run_launches(ctx, p, 0, N, sb, &ctx->launches[1]))) return rc;
+  if (both) {
+    CUDA_TRY(cudaEventRecord(ctx->join_ev, sb));
+    CUDA_TRY(cudaStreamWaitEvent(s, ctx->join_ev, 0));
+  }
   if (prof) CUDA_TRY(cudaEventRecord(ctx->ev[2], s));
   ctx->launches[2] = ctx->launches[3] = 0;
   if (D > 0) {
-    if ((rc = decode_rows(ctx, decode_loci, D, dd, s))) return rc;
+    if ((rc = decode_rows(ctx, decode_loci, D, dd, both ? ctx->tscratch : nullptr, s))) return rc;
     ctx->launches[2] = 1;
   }
   if (prof) CUDA_TRY(cudaEventRecord(ctx->ev[3], s));
@@ -1727,7 +1792,7 @@ extern "C" int ls_run_all_noalloc(ls_ctx* ctx, const int32_t* decode_loci, int32
     }
   }
   if (D > 0) {
-    if ((rc = decode_rows(ctx, decode_loci, D, d_out, s))) return rc;
+    if ((rc = decode_rows(ctx, decode_loci, D, d_out, nullptr, s))) return rc;
     const int nt = (N + 31) / 32;
     lsk::symmetrize_kernel<<<dim3(nt, nt, D), dim3(32, 8), 0, s>>>(d_out, N);
     CUDA_TRY(cudaGetLastError());

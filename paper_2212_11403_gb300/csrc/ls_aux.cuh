@@ -86,6 +86,10 @@ __global__ void double_rows_kernel(const uint32_t* __restrict__ bits, int rw, in
 }
 
 
+__global__ void fill_kernel(float* __restrict__ p, long long n, float v) {
+  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) p[e] = v;
+}
+
 // Pack uint8 [L][N] 0/1 haplotypes into variant-major rows of 32 haplotypes per word, haplotype i
 // in bit i%32 of word i/32 (Sec. 4.1.1).  One warp per output word: a coalesced 32-byte read and a
 // ballot.  Padding words must be zeroed beforehand.
@@ -145,7 +149,8 @@ struct DecodeLoci {
 // allele at l, mu elsewhere, read from the packed row; a zero theta means alpha = 0 too, and the
 // entry is 0).  A zero normaliser gives p = eps for every donor (Sec. 2.2).  Grid (N, D), one CTA
 // per row.
-__global__ void decode_kernel(float* __restrict__ prod, int N, const uint32_t* __restrict__ bits, int row_words,
+// With t, prod holds alpha and t the backward's t 2^100, and the product is formed here.
+__global__ void decode_kernel(float* __restrict__ prod, const float* __restrict__ t, int N, const uint32_t* __restrict__ bits, int row_words,
                               const float* __restrict__ thm, const float* __restrict__ thx, const DecodeLoci dl) {
   constexpr float eps = 2.220446049250313e-16f;
   const int r = blockIdx.x;
@@ -155,7 +160,8 @@ __global__ void decode_kernel(float* __restrict__ prod, int N, const uint32_t* _
   const float tm = thm[l], tx = thx[l];
   const float im = tm > 0.0f ? 1.0f / tm : 0.0f, ix = tx > 0.0f ? 1.0f / tx : 0.0f;
   float* a = prod + ((size_t)blockIdx.y * N + r) * N;
-  auto q = [&](int j) { return a[j] * ((((row[j >> 5] >> (j & 31)) & 1u) == ai) ? im : ix); };
+  const float* b = t ? t + ((size_t)blockIdx.y * N + r) * N : nullptr;
+  auto q = [&](int j) { return (b ? a[j] * b[j] : a[j]) * ((((row[j >> 5] >> (j & 31)) & 1u) == ai) ? im : ix); };
   float s = 0.0f;
   for (int j = threadIdx.x; j < N; j += blockDim.x)
     if (j != r) s += q(j);

@@ -71,6 +71,8 @@ struct ls_ctx {
   int* err = nullptr;             // device error word
   float* dscratch = nullptr;      // host-output staging for ls_run_all
   size_t dscratch_bytes = 0;
+  float* tscratch = nullptr;      // ls_run_all of small data sets: the backward's values at the decode loci
+  size_t tscratch_bytes = 0;
   int num_sms = 0;
   int ntables = 0;
   // profiling of ls_run_all phases

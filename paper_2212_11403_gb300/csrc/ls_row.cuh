@@ -152,7 +152,7 @@ __global__ void __launch_bounds__(kRowMaxThreads) row_steps_kernel(const PropPar
 // on 16-byte boundaries.  Bound by memory (posteriors at N = 10000: 249 us, 4.8 TB/s; before, with the
 // rows read twice, 442 us) and, with distances, by the logarithms too.
 struct PostArgs {
-  const float *alpha, *beta;  // DEC 0
+  const float *alpha, *beta;  // DEC 0; DEC 1: null and, where out holds alpha alone, the backward's t 2^100
   float* out;
   int N, t0, mode;
   const uint32_t* bits;       // DEC 1: packed rows
@@ -189,6 +189,12 @@ __global__ void __launch_bounds__(kRowMaxThreads) row_posterior_kernel(const __g
     if (pos < N) {
       if (DEC) {
         row_load<VEC>(o + pos, q[e]);
+        if (a.beta) {
+          float t[VEC];
+          row_load<VEC>(a.beta + (o - a.out) + pos, t);
+#pragma unroll
+          for (int k = 0; k < VEC; ++k) q[e][k] *= t[k];
+        }
         const uint32_t w = (bits[pos >> 5] ^ inv) >> (pos & 31);
 #pragma unroll
         for (int k = 0; k < VEC; ++k) q[e][k] *= (w >> k) & 1u ? im : ix;
