@@ -36,6 +36,8 @@ void ls_register_group15(std::vector<PropKernelInfo>& out);
 void ls_register_group16(std::vector<PropKernelInfo>& out);
 void ls_register_group17(std::vector<PropKernelInfo>& out);
 void ls_register_group18(std::vector<PropKernelInfo>& out);
+void ls_register_group19(std::vector<PropKernelInfo>& out);
+void ls_register_group20(std::vector<PropKernelInfo>& out);
 
 namespace {
 
@@ -80,6 +82,8 @@ std::vector<PropKernelInfo>& registry() {
     ls_register_group16(v);
     ls_register_group17(v);
     ls_register_group18(v);
+    ls_register_group19(v);
+    ls_register_group20(v);
   });
   return v;
 }
@@ -1167,10 +1171,11 @@ struct StatPick {
   int smem = 0;
 };
 
-int pick_stat(ls_ctx* c, StatPick* out) {
+// most: targets a block may hold (a CTA's targets share its rotation, so blocks are whole CTAs)
+int pick_stat(ls_ctx* c, int most, StatPick* out) {
   double bc = 1e300;
   for (const auto& k : registry()) {
-    if (k.st != 1 || !k.serves(c->N)) continue;
+    if (k.st != 1 || !k.serves(c->N) || k.tpw > most) continue;
     const int smem = k.smem_bytes(c->rw2);
     if (smem > 227 * 1024) continue;
     bool ok = true;
@@ -1306,7 +1311,7 @@ int grad_block(ls_ctx* ctx, const StatPick& sp, int b0, int TB, int L, int G, co
       pos = seg_end;
       k0 = k1;
     } while (k0 < G);
-    lsk::grad_dot_kernel<<<dim3(TB, G), 256, 0, s>>>(A, Wst, B, N, TB, Rg);
+    lsk::grad_dot_kernel<<<(unsigned)(((long long)TB * G + 7) / 8), 256, 0, s>>>(A, Wst, B, N, (long long)TB * G, Rg);
     CUDA_TRY(cudaGetLastError());
     lsk::sum_rows_kernel<<<G, 256, 0, s>>>(Rg, TB, sums);
     CUDA_TRY(cudaGetLastError());
@@ -1337,8 +1342,6 @@ int ls_pac_grad(ls_ctx* ctx, int32_t t_from, int32_t t_to, const int32_t* interv
   }
   for (double m : ctx->mu_h)
     if (!(m < 1.0)) return fail(LS_ERR_ARG, "the gradient needs mu < 1");
-  StatPick sp;
-  if ((rc = pick_stat(ctx, &sp))) return rc;
   const int T = t_to - t_from;
   cudaStream_t s = (cudaStream_t)stream;
   // groups with at least one interval; their end loci e_g (the locus after the group's last interval)
@@ -1363,6 +1366,9 @@ int ls_pac_grad(ls_ctx* ctx, int32_t t_from, int32_t t_to, const int32_t* interv
   // blocks are whole waves of the statistic kernel where possible.
   const size_t per_target = ((size_t)3 * G + 2) * (size_t)N * sizeof(float);
   int Tb = (int)std::min<size_t>((size_t)T, std::max<size_t>(1, grad_budget() / per_target));
+  StatPick sp;
+  if ((rc = pick_stat(ctx, Tb < T ? Tb : N, &sp))) return rc;
+  if (Tb < T) Tb -= Tb % sp.k->tpw;
   if (Tb < T) {
     int nb = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, sp.k->func[0], sp.k->w * 32, sp.smem);

@@ -224,13 +224,28 @@ void ls_register_group18(std::vector<PropKernelInfo>& out) {
 }
 #elif LS_INST_GROUP == 8
 void ls_register_group8(std::vector<PropKernelInfo>& out) {
-  // statistic passes of the adjoint (uniform prior), one target per CTA
+  // statistic passes of the adjoint (uniform prior): two tiles per lane.  As many targets per CTA as keep a
+  // lane's slices long, because the work per locus that does not scale with the slice is the larger part of a
+  // short one (N = 2003, L = 1999, one target of 16 slots a lane against four of 63: 7.8 / 8.5 -> 3.7 / 3.3 ms
+  // for the two passes).  Every N up to 10240 is served; the ranges do not overlap beyond 512.
   LS_REGS(1, 4, 1);
-  LS_REGS(1, 4, 8);
+  LS_REGS(8, 4, 4);
+  LS_REGS(8, 4, 8);
 }
 #elif LS_INST_GROUP == 9
 void ls_register_group9(std::vector<PropKernelInfo>& out) {
   LS_REGS(1, 4, 16);
   LS_REGS(1, 4, 20);
+}
+#elif LS_INST_GROUP == 19
+void ls_register_group19(std::vector<PropKernelInfo>& out) {
+  LS_REGS(8, 4, 16);
+  LS_REGS(4, 4, 16);
+}
+#elif LS_INST_GROUP == 20
+void ls_register_group20(std::vector<PropKernelInfo>& out) {
+  LS_REGS(4, 4, 20);
+  LS_REGS(2, 4, 16);
+  LS_REGS(2, 4, 20);
 }
 #endif
