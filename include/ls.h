@@ -148,7 +148,7 @@ int ls_table_info(const ls_table* t, int32_t* kind, int32_t* locus, int32_t* t_f
 int ls_table_read(const ls_table* t, float* state, double* logscale, ls_stream_t stream);
 
 /* Sizes the propagation calls (ls_forward, ls_backward, ls_checkpoints, ls_run_all and their
- * callers) serve: the uniform prior for N up to 114688 (register-tile kernels to N = 20480, one
+ * callers) serve: the uniform prior for N up to 114688 (register-tile kernels to N = 40960, one
  * CTA per target to 57344, two-CTA clusters beyond); a prior matrix up to N = 20480 in either
  * prior format and up to N = 106496 in the BF16 format.  Beyond these the launch planner returns
  * LS_ERR_UNSUPPORTED before anything is enqueued. */

@@ -38,6 +38,7 @@ void ls_register_group17(std::vector<PropKernelInfo>& out);
 void ls_register_group18(std::vector<PropKernelInfo>& out);
 void ls_register_group19(std::vector<PropKernelInfo>& out);
 void ls_register_group20(std::vector<PropKernelInfo>& out);
+void ls_register_group21(std::vector<PropKernelInfo>& out);
 
 namespace {
 
@@ -84,6 +85,7 @@ std::vector<PropKernelInfo>& registry() {
     ls_register_group18(v);
     ls_register_group19(v);
     ls_register_group20(v);
+    ls_register_group21(v);
   });
   return v;
 }

@@ -54,9 +54,6 @@ constexpr int kMaxStore = 64;    // store loci per launch
 #ifndef LS_X_NACC
 #define LS_X_NACC 4
 #endif
-#ifndef LS_X_RED4
-#define LS_X_RED4 0
-#endif
 constexpr int kAluMod = LS_X_ALUMOD;
 constexpr float kEps = 2.220446049250313e-16f;  // DBL_EPSILON = 2^-52, exact in FP32 (Eq. distmat)
 // alpha * beta products for the posterior (Eq. postprob) are formed as alpha * (beta * 2^100): the
@@ -266,7 +263,7 @@ __device__ __forceinline__ void cta_sync() {
 }
 
 template <int DIR, int TPW, int W, int KQ, int PIM, int ST>
-__global__ void __launch_bounds__(W * 32, ((PIM || ST) && W >= 8) ? 1 : 2) ls_prop_kernel(const PropParams p) {
+__global__ void __launch_bounds__(W * 32, ((PIM || ST) && W >= 8) || (W >= 8 && KQ > 20) ? 1 : 2) ls_prop_kernel(const PropParams p) {
   static_assert(ST == 0 || (DIR == 0 && PIM == 0), "statistic passes run forward with the uniform prior");
   // UNI (uniform prior, no statistic): theta = base * f with base = max(1-mu, mu) and f in {1, ratio},
   // ratio = min(1-mu, mu) / base; a cell is c' x + r' (c' = c base, r' = r base), then multiplied by
@@ -324,10 +321,11 @@ __global__ void __launch_bounds__(W * 32, ((PIM || ST) && W >= 8) ? 1 : 2) ls_pr
   // The backward of the tiles with up to 255 registers a thread takes a thread's elements in batches
   // of kXB and issues a batch's loads before its stores (the compiler cannot tell the stores from
   // later loads, so the read-modify-write of the decode products would otherwise wait one memory
-  // latency per element); the forward, which only reads when it resumes from a table, and the
-  // 8-warp tiles (128 registers) keep one element at a time (measured faster, and no spills).
+  // latency per element: 21.4 against 16.5 ms for a backward of 100 loci with one decode locus at N =
+  // 26000); the forward, which only reads when it resumes from a table, and the 8-warp tiles of 128
+  // registers keep one element at a time (measured faster, and no spills).
   auto xfer = [&](int c, float* gbase, float* w1, float* m1, float* w2, bool to_global) {
-    if constexpr (DIR == 0 || W >= 8) {
+    if constexpr (DIR == 0 || (W >= 8 && KQ <= 20 && PIM == 0)) {
       for (int idx = tid; idx < THREADS * 32; idx += THREADS) {
         const int src = idx >> 5, s = idx & 31;
         const int ln = src & 31;
@@ -534,12 +532,12 @@ __global__ void __launch_bounds__(W * 32, ((PIM || ST) && W >= 8) ? 1 : 2) ls_pr
       tu = u;
       return v;
     }
-    if (LS_X_RED4 && !ST && W == 4) {  // the W partials of target tl in one 16-byte load
+    if (!ST && W == 8) {  // the W partials of target tl in two 16-byte loads
       if (sl == 0) buf[tl * W + warp] = v;
       cta_sync<W>();
-      const float4 e = *reinterpret_cast<const float4*>(buf + tl * W);
+      const float4 e = *reinterpret_cast<const float4*>(buf + tl * W), f = *reinterpret_cast<const float4*>(buf + tl * W + 4);
       tu = 0.0f;
-      return (e.x + e.y) + (e.z + e.w);
+      return ((e.x + e.y) + (e.z + e.w)) + ((f.x + f.y) + (f.z + f.w));
     }
     float2* b2 = reinterpret_cast<float2*>(buf);
     if (sl == 0) b2[tl * W + warp] = make_float2(v, u);

@@ -165,12 +165,18 @@ void ls_register_group11(std::vector<PropKernelInfo>& out) {
 }
 #elif LS_INST_GROUP == 12
 void ls_register_group12(std::vector<PropKernelInfo>& out) {
-  // register + shared-memory state, N in (20480, 40960]
-  LS_REGH(0);
-  LS_REGH(2);
-  LS_REGH(4);
-  LS_REGH(6);
-  LS_REGH(8);
+  // one target per CTA of 8 warps with the whole state in registers: N in (16384, 40960].  Against the
+  // large-N kernel (state in registers and shared memory, 16 warps) forward / backward of 100 loci take 14.9 /
+  // 16.5 against 16.5 / 17.4 ms at N = 26000, 18.2 / 22.8 against 21.1 / 21.4 at N = 30000 and 29.2 / 33.6
+  // against 36.8 / 37.9 at N = 40960; N <= 20480 runs faster with two CTAs of 4 warps an SM.
+  LS_REG(1, 8, 24);
+  LS_REG(1, 8, 28);
+  LS_REG(1, 8, 32);
+}
+#elif LS_INST_GROUP == 21
+void ls_register_group21(std::vector<PropKernelInfo>& out) {
+  LS_REG(1, 8, 36);
+  LS_REG(1, 8, 40);
 }
 #elif LS_INST_GROUP == 13
 void ls_register_group13(std::vector<PropKernelInfo>& out) {
