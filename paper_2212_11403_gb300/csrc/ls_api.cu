@@ -457,6 +457,72 @@ int ls_fail(int code, const char* fmt, ...) {
 
 int ls_dev_alloc(void** p, size_t bytes) { return dev_alloc(nullptr, p, bytes); }
 
+// ---- per-call scratch ------------------------------------------------------------------------
+namespace {
+struct TmpPool {
+  cudaMemPool_t pool = nullptr;
+  int users = 0;
+};
+std::mutex g_tmp_mu;
+std::vector<TmpPool> g_tmp;  // by device
+
+TmpPool& tmp_of(int device) {  // with g_tmp_mu held
+  if ((int)g_tmp.size() <= device) g_tmp.resize(device + 1);
+  return g_tmp[device];
+}
+}  // namespace
+
+void ls_tmp_hold(int device) {
+  std::lock_guard<std::mutex> lk(g_tmp_mu);
+  ++tmp_of(device).users;
+}
+
+void ls_tmp_release(int device) {
+  std::lock_guard<std::mutex> lk(g_tmp_mu);
+  TmpPool& t = tmp_of(device);
+  if (--t.users == 0 && t.pool) cudaMemPoolTrimTo(t.pool, 0);
+}
+
+int ls_tmp_alloc(void** p, size_t bytes, cudaStream_t s) {
+  *p = nullptr;
+  if (bytes == 0) bytes = 16;
+  int device = 0;
+  CUDA_TRY(cudaGetDevice(&device));
+  cudaMemPool_t pool;
+  {
+    std::lock_guard<std::mutex> lk(g_tmp_mu);
+    TmpPool& t = tmp_of(device);
+    if (!t.pool) {
+      cudaMemPoolProps props = {};
+      props.allocType = cudaMemAllocationTypePinned;
+      props.handleTypes = cudaMemHandleTypeNone;
+      props.location.type = cudaMemLocationTypeDevice;
+      props.location.id = device;
+      CUDA_TRY(cudaMemPoolCreate(&t.pool, &props));
+      unsigned long long keep = kTmpKeep;
+      CUDA_TRY(cudaMemPoolSetAttribute(t.pool, cudaMemPoolAttrReleaseThreshold, &keep));
+    }
+    pool = t.pool;
+  }
+  cudaError_t e = cudaMallocFromPoolAsync(p, bytes, pool, s);
+  if (e == cudaErrorMemoryAllocation) {  // what the pool keeps may be what is missing
+    cudaGetLastError();
+    cudaStreamSynchronize(s);
+    cudaMemPoolTrimTo(pool, 0);
+    e = cudaMallocFromPoolAsync(p, bytes, pool, s);
+  }
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    *p = nullptr;
+    return fail(LS_ERR_OOM, "allocating %zu bytes of scratch: %s", bytes, cudaGetErrorString(e));
+  }
+  return LS_OK;
+}
+
+void ls_tmp_free(void* p, cudaStream_t s) {
+  if (p) cudaFreeAsync(p, s);
+}
+
 extern "C" {
 
 const char* ls_version(void) {
@@ -495,6 +561,7 @@ int ls_create(ls_ctx** out, const uint8_t* haps, int32_t N, int32_t L) {
   if (e != cudaSuccess) { free_ctx(c); return fail(LS_ERR_CUDA, "packing haplotypes: %s", cudaGetErrorString(e)); }
   rc = init_ctx_common(c);
   if (rc) { free_ctx(c); return rc; }
+  ls_tmp_hold(c->device);
   *out = c;
   return LS_OK;
 }
@@ -526,6 +593,7 @@ int ls_create_packed(ls_ctx** out, const uint32_t* packed, int32_t N, int32_t L,
   if (e != cudaSuccess) { free_ctx(c); return fail(LS_ERR_CUDA, "copying packed haplotypes: %s", cudaGetErrorString(e)); }
   rc = init_ctx_common(c);
   if (rc) { free_ctx(c); return rc; }
+  ls_tmp_hold(c->device);
   *out = c;
   return LS_OK;
 }
@@ -533,8 +601,10 @@ int ls_create_packed(ls_ctx** out, const uint32_t* packed, int32_t N, int32_t L,
 int ls_destroy(ls_ctx* ctx) {
   if (!ctx) return fail(LS_ERR_ARG, "null context");
   if (ctx->ntables) return fail(LS_ERR_STATE, "%d tables still alive", ctx->ntables);
-  cudaSetDevice(ctx->device);
+  const int device = ctx->device;
+  cudaSetDevice(device);
   free_ctx(ctx);
+  ls_tmp_release(device);
   return LS_OK;
 }
 
@@ -1201,14 +1271,17 @@ int pick_stat(ls_ctx* c, int most, StatPick* out) {
   return LS_OK;
 }
 
-struct DevBufs {
+struct DevBufs {  // scratch of one call, in the order of its stream
+  cudaStream_t s;
   std::vector<void*> v;
+  explicit DevBufs(cudaStream_t stream) : s(stream) {}
+  DevBufs(const DevBufs&) = delete;
   ~DevBufs() {
-    for (void* p : v) cudaFree(p);
+    for (void* p : v) ls_tmp_free(p, s);
   }
   template <class T>
   int get(T** p, size_t n) {
-    int rc = dev_alloc(nullptr, (void**)p, sizeof(T) * std::max<size_t>(n, 1));
+    int rc = ls_tmp_alloc((void**)p, sizeof(T) * std::max<size_t>(n, 1), s);
     if (!rc) v.push_back(*p);
     return rc;
   }
@@ -1378,7 +1451,7 @@ int ls_pac_grad(ls_ctx* ctx, int32_t t_from, int32_t t_to, const int32_t* interv
     if (Tb >= wave) Tb = (Tb / wave) * wave;
   }
   Tb = std::min(Tb, T);
-  DevBufs db;
+  DevBufs db(s);
   float *d_gam, *d_eta, *A, *Wst, *B, *xst, *wst;
   uint8_t* d_rst;
   double *logF, *EM, *Rg, *sums;
@@ -1477,7 +1550,7 @@ int ls_sparse_run_all(ls_ctx* ctx, const int32_t* idx, int32_t K, int32_t WS, in
   if (pout_out && !is_device_ptr(pout_out)) return fail(LS_ERR_ARG, "pout_out must be device memory");
   const int Wn = (L + WS - 1) / WS;
   cudaStream_t s = (cudaStream_t)stream;
-  DevBufs db;
+  DevBufs db(s);
   float *P, *lost, *poolf = nullptr, *share = nullptr;
   double* logs;
   uint32_t* stat;

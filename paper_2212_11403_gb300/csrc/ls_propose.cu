@@ -38,14 +38,17 @@ int dev_alloc(void*, void** p, size_t n) { return ls_dev_alloc(p, n); }
     if (e_ != cudaSuccess) return fail(LS_ERR_CUDA, "%s: %s", #x, cudaGetErrorString(e_));     \
   } while (0)
 
-struct Bufs {
+struct Bufs {  // scratch of one call, in the order of its stream
+  cudaStream_t s;
   std::vector<void*> v;
+  explicit Bufs(cudaStream_t stream) : s(stream) {}
+  Bufs(const Bufs&) = delete;
   ~Bufs() {
-    for (void* q : v) cudaFree(q);
+    for (void* q : v) ls_tmp_free(q, s);
   }
   template <class T>
   int get(T** q, size_t n) {
-    int rc = dev_alloc(nullptr, (void**)q, sizeof(T) * std::max<size_t>(n, 1));
+    int rc = ls_tmp_alloc((void**)q, sizeof(T) * std::max<size_t>(n, 1), s);
     if (!rc) v.push_back(*q);
     return rc;
   }
@@ -201,9 +204,11 @@ int ls_mlp_create(const float* params, uint64_t seed, ls_mlp** out) {
   cudaMemset(m->m, 0, sizeof(float) * P);
   cudaMemset(m->v, 0, sizeof(float) * P);
   if ((rc = refresh(m))) {
+    ls_tmp_hold(m->device);
     ls_mlp_destroy(m);
     return rc;
   }
+  ls_tmp_hold(m->device);
   *out = m;
   return LS_OK;
 }
@@ -218,6 +223,7 @@ int ls_mlp_destroy(ls_mlp* m) {
   cudaFree(m->w1t);
   cudaFree(m->w2t);
   cudaFree(m->err);
+  ls_tmp_release(m->device);
   delete m;
   return LS_OK;
 }
@@ -247,7 +253,7 @@ int ls_mlp_forward(const ls_mlp* m, const float* X, int64_t n, float* scores, ls
 int ls_mlp_grad(ls_mlp* m, const float* X, const float* y, int32_t n, float* grad, double* loss, ls_stream_t stream) {
   if (!m || !X || !y || n < 1) return fail(LS_ERR_ARG, "bad arguments");
   cudaStream_t s = (cudaStream_t)stream;
-  Bufs b;
+  Bufs b(s);
   GradWork gw;
   int rc = gw.setup(m, b, n, 1, s);
   if (rc) return rc;
@@ -272,7 +278,7 @@ int ls_mlp_train(ls_mlp* m, const float* X, const float* y, int64_t n, int32_t s
                  uint64_t seed, double* loss_out, ls_stream_t stream) {
   if (!m || !X || !y || n < 1 || steps < 0 || batch < 1) return fail(LS_ERR_ARG, "bad arguments");
   cudaStream_t s = (cudaStream_t)stream;
-  Bufs b;
+  Bufs b(s);
   GradWork gw;
   const int ntail = std::min(steps, std::max(1, steps / 10));  // the steps whose losses are averaged
   int rc = gw.setup(m, b, batch, ntail, s);
@@ -391,7 +397,7 @@ int ls_propose_window(ls_ctx* ctx, int32_t C, int32_t w, int32_t* cand_out, floa
   if (!ctx || C < 1 || !cand_out) return fail(LS_ERR_ARG, "bad arguments");
   cudaSetDevice(ctx->device);
   cudaStream_t s = (cudaStream_t)stream;
-  Bufs b;
+  Bufs b(s);
   PropWork pw;
   int rc = prop_setup(ctx, b, pw, s);
   if (rc) return rc;
@@ -416,7 +422,7 @@ int ls_propose(ls_ctx* ctx, int32_t C, int32_t K, const ls_mlp* mlp, int32_t* id
   if (mlp && (C < K || C > 2048)) return fail(LS_ERR_ARG, "need K <= C <= 2048 candidates for the MLP stage");
   cudaSetDevice(ctx->device);
   cudaStream_t s = (cudaStream_t)stream;
-  Bufs b;
+  Bufs b(s);
   PropWork pw;
   int rc = prop_setup(ctx, b, pw, s);
   if (rc) return rc;
