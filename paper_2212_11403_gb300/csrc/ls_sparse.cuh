@@ -34,10 +34,11 @@
 // when their window starts and so hold one common value xs, which the row sum subtracts.  The
 // per-locus constants of the next block are copied with cp.async while the current one runs.
 //
-// 247 warp instructions a locus at 48 slots a lane, issued in 46 % of the cycles with three warps a
-// scheduler: bound by the dependent chain of a locus (row sum, division, multiply, add).  N = 20003, L =
-// 2000, K = 3 x 512: forward / backward 32.3 / 30.2 -> 17.3 / 17.6 ms (before: one word and one bit test,
-// select and count per slot and locus, set ids in registers, two warps a scheduler).
+// Bound by the dependent chain of a locus (row sum, division, multiply, add), so what counts is the warps that
+// cover it: 128 registers and 12.8 KB a warp leave four a scheduler (bits are gathered and transposed 16 slots
+// at a time for that).  N = 20003, L = 2000, K = 3 x 512: forward / backward 32.3 / 30.2 -> 14.5 / 14.7 ms
+// (before: one word and one bit test, select and count per slot and locus, set ids in registers, two warps a
+// scheduler; with three warps, transposing 32 slots at a time, 17.4 / 17.5).
 #pragma once
 
 #include <cstdint>
@@ -46,7 +47,7 @@
 
 namespace lsk {
 
-constexpr int kSparseWarps = 4;   // targets per CTA (three CTAs per SM at 48 slots a lane)
+constexpr int kSparseWarps = 4;   // targets per CTA (four CTAs per SM)
 constexpr int kSparseChunk = 64;  // loci per block: two 32-bit haplotype-major words per donor
 constexpr int kSparseScal = 4;    // per-locus constants staged per block: 1-rho, rho, n1, emission ratio
 
@@ -81,11 +82,13 @@ struct SparseParams {
 // keeps products of small alpha and beta above FP32's underflow
 constexpr float kSparseProdScale = 0x1p100f;
 
-// 32-slot groups of a lane's slots, and bytes per warp: the block's words [64][groups][32], whose place
-// the copies of the old set (ids and values) take at a window change
+// Words per lane and locus (bit s of word g: slot 32 g + s), the second one of 16 bits where a lane has 48
+// slots; bytes per warp of a block's words [64][32 lanes] (32-bit), [64][32 lanes] (16-bit), whose place the
+// copies of the old set (ids and values) take at a window change.
 __host__ __device__ constexpr int sparse_groups(int ks) { return (ks + 31) / 32; }
 __host__ __device__ constexpr int sparse_warp_bytes(int ks) {
-  return kSparseChunk * sparse_groups(ks) * 128 > 256 * ks ? kSparseChunk * sparse_groups(ks) * 128 : 256 * ks;
+  const int words = kSparseChunk * 128 + (ks > 32 ? kSparseChunk * 64 : 0);
+  return words > 256 * ks ? words : 256 * ks;
 }
 constexpr int kSparsePool = 2 * kSparseChunk;  // floats per warp: the outside donors' summed and mean emission per locus
 // two buffers of per-locus constants and the per-warp regions
@@ -102,14 +105,15 @@ __device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_g
 
 #ifndef LS_SPARSE_PARAMS_ONLY  // the kernels live in ls_sparse.cu only
 
-// 32 x 32 bit transposition: bit c of m[r] and bit r of m[c] change places
-__device__ __forceinline__ void transpose32(uint32_t (&m)[32]) {
+// Two 16 x 16 bit transpositions at once: the low half of m[c] becomes the bits c of the low halves of all
+// m[r], the high half those of the high halves
+__device__ __forceinline__ void transpose16x2(uint32_t (&m)[16]) {
 #pragma unroll
-  for (int st = 0; st < 5; ++st) {
-    const int j = 16 >> st;
-    const uint32_t mask = st == 0 ? 0x0000ffffu : st == 1 ? 0x00ff00ffu : st == 2 ? 0x0f0f0f0fu : st == 3 ? 0x33333333u : 0x55555555u;
+  for (int st = 0; st < 4; ++st) {
+    const int j = 8 >> st;
+    const uint32_t mask = st == 0 ? 0x00ff00ffu : st == 1 ? 0x0f0f0f0fu : st == 2 ? 0x33333333u : 0x55555555u;
 #pragma unroll
-    for (int k = 0; k < 32; ++k)
+    for (int k = 0; k < 16; ++k)
       if (!(k & j)) {
         const uint32_t lo = (m[k] & mask) | ((m[k + j] & mask) << j);
         const uint32_t hi = ((m[k] >> j) & mask) | (m[k + j] & ~mask);
@@ -120,7 +124,7 @@ __device__ __forceinline__ void transpose32(uint32_t (&m)[32]) {
 }
 
 template <int DIR, int KS>
-__global__ void __launch_bounds__(kSparseWarps * 32, 3) ls_sparse_kernel(const __grid_constant__ SparseParams p) {
+__global__ void __launch_bounds__(kSparseWarps * 32, 4) ls_sparse_kernel(const __grid_constant__ SparseParams p) {
   static_assert(KS % 2 == 0, "slots come in pairs");
   constexpr float eps = 2.220446049250313e-16f;
   constexpr int INF_ID = 0x7fffffff;
@@ -130,7 +134,9 @@ __global__ void __launch_bounds__(kSparseWarps * 32, 3) ls_sparse_kernel(const _
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   float* pool_e = scal + 2 * kSparseScal * CH + warp * kSparsePool;  // [64] sums, [64] means
   unsigned char* mine = smem + (2 * kSparseScal * CH + kSparseWarps * kSparsePool) * 4 + warp * sparse_warp_bytes(KS);
-  uint32_t* words = reinterpret_cast<uint32_t*>(mine) + lane;  // [locus][group] x 32 lanes
+  uint32_t* words = reinterpret_cast<uint32_t*>(mine) + lane;                     // [locus] x 32 lanes
+  uint16_t* words2 = reinterpret_cast<uint16_t*>(mine + kSparseChunk * 128) + lane;  // 48 slots: the last 16
+  auto word_at = [&](int kr, int g) -> uint32_t { return g == 0 ? words[32 * kr] : (uint32_t)words2[32 * kr]; };
   int* sid = reinterpret_cast<int*>(mine);                     // window changes: the old set's ids and values
   float* sval = reinterpret_cast<float*>(mine) + 32 * KS;
   const int i_raw = p.t_begin + blockIdx.x * kSparseWarps + warp;
@@ -160,26 +166,37 @@ __global__ void __launch_bounds__(kSparseWarps * 32, 3) ls_sparse_kernel(const _
     __syncwarp();
     const uint32_t* hwb = p.hw + (size_t)(b >> 2) * N * 8 + 2 * (b & 3);
     const uint2 tw = *reinterpret_cast<const uint2*>(hwb + (size_t)i * 8);
+#pragma unroll 1
+    for (int g = 0; g < (KS + 15) / 16; ++g) {  // 16 slots at a time
+      uint32_t lo[16], hi[16];
 #pragma unroll
-    for (int g = 0; g < NG; ++g) {
-      uint32_t lo[32], hi[32];
-#pragma unroll
-      for (int s = 0; s < 32; ++s) {
+      for (int s = 0; s < 16; ++s) {
         lo[s] = hi[s] = 0u;
-        if (32 * g + s < KS) {
-          const int id = set_entry(cur_w, 32 * g + s);
+        if (s < KS) {
+          const int id = set_entry(cur_w, 16 * g + s);
           uint2 v = make_uint2(~tw.x, ~tw.y);  // padding differs everywhere
           if (id >= 0) v = *reinterpret_cast<const uint2*>(hwb + (size_t)id * 8);
           lo[s] = v.x ^ tw.x;
           hi[s] = v.y ^ tw.y;
         }
       }
-      transpose32(lo);
+      // group g's 16 bits: halves of the 32-bit words, or the 16-bit words
+      const int step = g < 2 ? 64 : 32;
+      uint16_t* dst = g < 2 ? reinterpret_cast<uint16_t*>(words) + g : words2;
+      auto put = [&](uint32_t (&m)[16], int k0) {
+        transpose16x2(m);
 #pragma unroll
-      for (int k = 0; k < 32; ++k) words[(k * NG + g) * 32] = lo[k];
-      transpose32(hi);
+        for (int k = 0; k < 16; ++k) {
+          dst[(k0 + k) * step] = (uint16_t)m[k];
+          dst[(k0 + 16 + k) * step] = (uint16_t)(m[k] >> 16);
+        }
+        if (KS <= 16) {
 #pragma unroll
-      for (int k = 0; k < 32; ++k) words[((32 + k) * NG + g) * 32] = hi[k];
+          for (int k = 0; k < 32; ++k) dst[(k0 + k) * step + 1] = 0;
+        }
+      };
+      put(lo, 0);
+      put(hi, 32);
     }
     if (p.pool) {
       const int nout = N - 1 - nset;
@@ -190,7 +207,7 @@ __global__ void __launch_bounds__(kSparseWarps * 32, 3) ls_sparse_kernel(const _
         for (int k = 0; k < 32; ++k) {
           int n = 0;
 #pragma unroll
-          for (int g = 0; g < NG; ++g) n += __popc(words[((32 * h + k) * NG + g) * 32]);
+          for (int g = 0; g < NG; ++g) n += __popc(word_at(32 * h + k, g));
           n = __reduce_add_sync(0xffffffffu, n);
           if (lane == k) mis = n;
         }
@@ -388,7 +405,7 @@ __global__ void __launch_bounds__(kSparseWarps * 32, 3) ls_sparse_kernel(const _
       float2 acc[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
 #pragma unroll
       for (int g = 0; g < NG; ++g) {
-        const uint32_t wd = words[(kr * NG + g) * 32];
+        const uint32_t wd = word_at(kr, g);
         const uint32_t sm = (wd ^ flip) | pad[g];
 #pragma unroll
         for (int s = 0; s < 32; s += 2) {
