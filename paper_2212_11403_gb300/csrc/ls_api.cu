@@ -288,60 +288,67 @@ int run_launches(ls_ctx* c, lsk::PropParams p, int t_begin, int t_count, cudaStr
   return LS_OK;
 }
 
-// 16-byte accesses need rows of whole quads on 16-byte boundaries (stored rows are the caller's)
-bool row_quads(int N, const void* a, const void* b = nullptr) {
-  return N % 4 == 0 && ((reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b)) & 15) == 0;
+// Rows of N floats in buffers on 16-byte boundaries all lie the same way on the quad grid; where N is a
+// multiple of four they start on it.
+bool on_quads(const void* a, const void* b = nullptr, const void* c = nullptr) {
+  return ((reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b) | reinterpret_cast<uintptr_t>(c)) & 15) == 0;
 }
+// threads of a row kernel: E4 quads each, and room for a row that starts within a quad
+int row_threads(int N, int E4) { return 32 * ((N + (N % 4 ? 3 : 0) + 128 * E4 - 1) / (128 * E4)); }
 
 // Table calls of few steps with the uniform prior go to the row kernel (one target per CTA, the row in
 // registers).  It costs less per call and more per step than the register-tile kernels: one / eight /
 // sixteen loci forward take 158 / 533 / 988 us against 658 / 762 / 875 us at N = 10000, 16 / 22 / 30
 // against 30 / 29 / 33 us at N = 1000 and 654 / 2264 / 4211 against 2412 / 2775 / 3214 us at N = 20000.
-// Rows off the 16-byte grid cost twice as much per step beyond N = 2048 (N = 4999, one / four / eight
-// loci: 83 / 177 / 311 against 160 / 169 / 182 us), so the line lies lower there.
+// Rows off the quad grid cost about a tenth more (N = 10001, one / eight loci: 174 / 588 us; with 4-byte accesses
+// N = 4999 took 83 / 311 us, now 56 / 156).
 bool row_steps_serve(const ls_ctx* c, const lsk::PropParams& p) {
-  const int most = row_quads(p.N, p.state, p.store) || p.N <= 2048 ? 8 : 3;
-  return !c->Pi && p.N <= lsk::kRowMaxN && p.n_steps <= most;
+  return !c->Pi && (p.N <= lsk::kRowMaxN || p.N == lsk::kRowMaxN + 3) && p.n_steps <= 8;
 }
 
-template <int E4, int VEC>
+template <int E4>
 void launch_row_steps(const lsk::PropParams& p, cudaStream_t s) {
-  const int nt = 32 * ((p.N + 128 * E4 - 1) / (128 * E4));
-  if (p.dir == 0) lsk::row_steps_kernel<0, E4, VEC><<<p.t_count, nt, 0, s>>>(p);
-  else lsk::row_steps_kernel<1, E4, VEC><<<p.t_count, nt, 0, s>>>(p);
+  const int nt = row_threads(p.N, E4);
+  if (p.N % 4 || !on_quads(p.store)) {
+    if (p.dir == 0) lsk::row_steps_kernel<0, E4, true><<<p.t_count, nt, 0, s>>>(p);
+    else lsk::row_steps_kernel<1, E4, true><<<p.t_count, nt, 0, s>>>(p);
+  } else {
+    if (p.dir == 0) lsk::row_steps_kernel<0, E4, false><<<p.t_count, nt, 0, s>>>(p);
+    else lsk::row_steps_kernel<1, E4, false><<<p.t_count, nt, 0, s>>>(p);
+  }
 }
 
 int run_row_steps(lsk::PropParams p, int t_begin, int t_count, cudaStream_t s) {
   p.t_begin = t_begin;
   p.t_count = t_count;
-  const bool vec = row_quads(p.N, p.state, p.store);
   // 8, 20 or 40 elements a thread: at most 256 threads a CTA up to N = 10240
-  if (p.N <= 2048) vec ? launch_row_steps<2, 4>(p, s) : launch_row_steps<2, 1>(p, s);
-  else if (p.N <= 5120) vec ? launch_row_steps<5, 4>(p, s) : launch_row_steps<5, 1>(p, s);
-  else vec ? launch_row_steps<10, 4>(p, s) : launch_row_steps<10, 1>(p, s);
+  if (p.N <= 2048) launch_row_steps<2>(p, s);
+  else if (p.N <= 5120) launch_row_steps<5>(p, s);
+  else launch_row_steps<10>(p, s);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(LS_ERR_CUDA, "row step launch: %s", cudaGetErrorString(e));
   return LS_OK;
 }
 
-// Posterior rows: DEC 0 grid (rows), DEC 1 grid (N, D).  The row kernel takes rows of whole quads on
-// 16-byte boundaries: posteriors up to 64 elements a thread (N = 5000 / 10000 / 20000 / 26000: 100 / 442 /
-// 893 / 1170 -> 64 / 249 / 637 / 902 us), the decode in place up to 20 (N = 2500 / 5000: 25 / 74 -> 16 / 49
-// us; at N = 10000 both take 0.31 ms, bound by the logarithms).  Other rows are faster with the two-pass
-// kernels (N = 10001: 443 against 683 us with 4-byte accesses held in registers).
+// Posterior rows: DEC 0 grid (rows), DEC 1 grid (N, D).  The row kernel takes buffers on 16-byte boundaries:
+// posteriors up to 64 elements a thread (N = 5000 / 10000 / 20000 / 26000: 100 / 442 / 893 / 1170 -> 64 / 249 /
+// 637 / 902 us), the decode in place up to 20 (N = 2500 / 5000: 25 / 74 -> 16 / 49 us; at N = 10000 both take
+// 0.31 ms, bound by the logarithms), on or off the quad grid (N = 10001: 443 -> 258 us).  The two-pass kernels
+// take the others.
 template <int DEC, int E4>
 void launch_posterior(const lsk::PostArgs& a, dim3 grid, cudaStream_t s) {
-  const int nt = 32 * ((a.N + 128 * E4 - 1) / (128 * E4));
-  lsk::row_posterior_kernel<DEC, E4><<<grid, nt, 0, s>>>(a);
+  const int nt = row_threads(a.N, E4);
+  if (a.N % 4) lsk::row_posterior_kernel<DEC, E4, true><<<grid, nt, 0, s>>>(a);
+  else lsk::row_posterior_kernel<DEC, E4, false><<<grid, nt, 0, s>>>(a);
 }
 template <int DEC>
 int launch_posterior(const lsk::PostArgs& a, dim3 grid, cudaStream_t s) {
-  const bool quads = row_quads(a.N, a.out, a.beta) && (DEC || row_quads(a.N, a.alpha));
+  const bool quads = on_quads(a.out, a.alpha, a.beta);
   if (quads && a.N <= 2048) launch_posterior<DEC, 2>(a, grid, s);
   else if (quads && a.N <= 5120) launch_posterior<DEC, 5>(a, grid, s);
   else if (DEC) lsk::decode_kernel<<<grid, 256, 0, s>>>(a.out, a.beta, a.N, a.bits, a.row_words, a.thm, a.thx, a.dl);
-  else if (quads && a.N <= 20480) launch_posterior<0, 10>(a, grid, s);
-  else if (quads && a.N <= lsk::kRowMaxPostN) launch_posterior<0, 16>(a, grid, s);
+  else if (quads && (a.N <= lsk::kRowMaxN || a.N == lsk::kRowMaxN + 3)) launch_posterior<0, 10>(a, grid, s);
+  else if (quads && (a.N <= lsk::kRowMaxPostN || a.N == lsk::kRowMaxPostN + 3)) launch_posterior<0, 16>(a, grid, s);
   else lsk::posterior_kernel<<<grid, 256, 0, s>>>(a.alpha, a.beta, a.N, a.t0, a.mode, a.out);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(LS_ERR_CUDA, "posterior launch: %s", cudaGetErrorString(e));

@@ -2,9 +2,10 @@
 // table, and posteriors / half distances of a row.
 //
 // Both are bound by memory: a row is read once, stays in registers across its reductions and is
-// written once, with 16-byte accesses where rows are 16-byte multiples (VEC = 4) and 4-byte ones
-// otherwise (VEC = 1).  Thread t of nt holds 4 E4 elements: quads t, t + nt, .. (VEC = 4) or elements
-// t, t + nt, .. (VEC = 1), so a warp's accesses are contiguous either way.
+// written once, in quads on 16-byte boundaries: thread t of nt holds E4 quads, t, t + nt, ..  Rows that do
+// not start on a boundary (SHIFT: N not a multiple of four) begin with the quad that holds their first
+// element; the parts of the first and last quad outside the row are left alone, and a quad's bits are
+// funnel-shifted out of two words.
 #pragma once
 
 #include <cstdint>
@@ -15,8 +16,8 @@
 namespace lsk {
 
 constexpr int kRowMaxThreads = 512;
-constexpr int kRowMaxN = 40 * kRowMaxThreads;  // single steps (E4 = 10)
-constexpr int kRowMaxPostN = 64 * kRowMaxThreads;  // posteriors (E4 = 16)
+constexpr int kRowMaxN = 40 * kRowMaxThreads - 3;  // single steps (E4 = 10); three elements for the shift
+constexpr int kRowMaxPostN = 64 * kRowMaxThreads - 3;  // posteriors (E4 = 16)
 
 // sum over the CTA, the same value in every thread; buf holds 32 floats and alternates between calls
 __device__ __forceinline__ float row_sum(float v, float* buf) {
@@ -32,39 +33,52 @@ __device__ __forceinline__ float row_sum(float v, float* buf) {
   return v;
 }
 
-template <int E4, int VEC>
-struct RowPos {  // first position of the e-th access and the number of accesses
-  static constexpr int COUNT = VEC == 4 ? E4 : 4 * E4;
-  __device__ static int at(int e) { return VEC * ((int)threadIdx.x + e * (int)blockDim.x); }
-};
-
-template <int VEC>
-__device__ __forceinline__ void row_load(const float* p, float* v) {
-  if (VEC == 4) {
-    const float4 q = __ldcs(reinterpret_cast<const float4*>(p));
-    v[0] = q.x, v[1] = q.y, v[2] = q.z, v[3] = q.w;
-  } else {
-    v[0] = __ldcs(p);
+// The quads of a row: `at(e)` is the position of the first element of this thread's e-th quad
+template <bool SHIFT>
+struct RowQuads {
+  int N, mis;  // mis: elements between the boundary before the row and the row
+  __device__ RowQuads(int n, const float* row) : N(n), mis(SHIFT ? (int)((reinterpret_cast<uintptr_t>(row) >> 2) & 3) : 0) {}
+  __device__ int at(int e) const { return 4 * ((int)threadIdx.x + e * (int)blockDim.x) - mis; }
+  __device__ bool in(int pos) const { return !SHIFT || (unsigned)pos < (unsigned)N; }  // element of a quad with at(e) < N
+  __device__ bool whole(int pos) const { return !SHIFT || (pos >= 0 && pos + 4 <= N); }
+  __device__ void load(const float* row, int pos, float (&v)[4]) const {
+    if (whole(pos)) {
+      const float4 q = __ldcs(reinterpret_cast<const float4*>(row + pos));
+      v[0] = q.x, v[1] = q.y, v[2] = q.z, v[3] = q.w;
+      return;
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = in(pos + k) ? __ldcs(row + pos + k) : 0.0f;
   }
-}
-template <int VEC>
-__device__ __forceinline__ void row_store(float* p, const float* v) {
-  if (VEC == 4) __stcs(reinterpret_cast<float4*>(p), make_float4(v[0], v[1], v[2], v[3]));
-  else __stcs(p, v[0]);
-}
+  __device__ void store(float* row, int pos, const float (&v)[4]) const {
+    if (whole(pos)) {
+      __stcs(reinterpret_cast<float4*>(row + pos), make_float4(v[0], v[1], v[2], v[3]));
+      return;
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (in(pos + k)) __stcs(row + pos + k, v[k]);
+  }
+  // bit k: element pos + k of a packed row (which ends in at least one spare word)
+  __device__ uint32_t bits(const uint32_t* b, int pos) const {
+    if (!SHIFT) return b[pos >> 5] >> (pos & 31);
+    if (pos < 0) return b[0] << -pos;
+    return funnel(b[pos >> 5], b[(pos >> 5) + 1], (uint32_t)(pos & 31));
+  }
+};
 
 // A few steps of a table (uniform prior; PropParams as for ls_prop_kernel, without alpha_dec and
 // tlist), one target per CTA.  The register-tile kernel loads and saves its tile through shared memory
 // element by element; a table moved by one locus is all load and save, so this kernel takes calls of
 // few steps.  N = 10000, one locus forward / backward: 658 / 520 -> 158 / 186 us (0.8 GB moved, 75 / 63 % of
 // the measured copy rate); the two reductions between load and save are what keeps it from the rest.
-template <int DIR, int E4, int VEC>
+template <int DIR, int E4, bool SHIFT>
 __global__ void __launch_bounds__(kRowMaxThreads) row_steps_kernel(const PropParams p) {
-  using P = RowPos<E4, VEC>;
   __shared__ float buf[2][32];
   const int N = p.N, i = p.t_begin + blockIdx.x, row = i - p.tab_t0;
   float* state = p.state + (size_t)row * N;
-  float x[P::COUNT][VEC];
+  const RowQuads<SHIFT> P(N, state);
+  float x[E4][4];
   int ph = 0;
   auto total = [&](float s) {
     ph ^= 1;
@@ -74,13 +88,13 @@ __global__ void __launch_bounds__(kRowMaxThreads) row_steps_kernel(const PropPar
   {
     float s = 0.0f;
 #pragma unroll
-    for (int e = 0; e < P::COUNT; ++e) {
-      const int pos = P::at(e);
+    for (int e = 0; e < E4; ++e) {
+      const int pos = P.at(e);
 #pragma unroll
-      for (int k = 0; k < VEC; ++k) x[e][k] = 0.0f;
-      if (p.load_state && pos < N) row_load<VEC>(state + pos, x[e]);
+      for (int k = 0; k < 4; ++k) x[e][k] = 0.0f;
+      if (p.load_state && pos < N) P.load(state, pos, x[e]);
 #pragma unroll
-      for (int k = 0; k < VEC; ++k) s += x[e][k];
+      for (int k = 0; k < 4; ++k) s += x[e][k];
     }
     if (p.load_state && DIR == 0) sig_prev = total(s);
   }
@@ -111,20 +125,26 @@ __global__ void __launch_bounds__(kRowMaxThreads) row_steps_kernel(const PropPar
     const float tm = p.thm[l], tx = p.thx[l];
     float s = 0.0f;
 #pragma unroll
-    for (int e = 0; e < P::COUNT; ++e) {
-      const int pos = P::at(e);
+    for (int e = 0; e < E4; ++e) {
+      const int pos = P.at(e);
       if (pos < N) {
-        const uint32_t w = (bits[pos >> 5] ^ inv) >> (pos & 31);
-        float b[VEC];
+        const uint32_t w = P.bits(bits, pos) ^ inv;
+        float b[4];
 #pragma unroll
-        for (int k = 0; k < VEC; ++k) {
-          b[k] = pos + k == i ? 0.0f : fmaf(c, x[e][k], r);  // alpha before its emission, or beta
+        for (int k = 0; k < 4; ++k) {
+          b[k] = pos + k == i || !P.in(pos + k) ? 0.0f : fmaf(c, x[e][k], r);  // alpha before its emission, or beta
           x[e][k] = ((w >> k) & 1u ? tm : tx) * b[k];
           s += x[e][k];
         }
-        const float* v = DIR == 0 ? x[e] : b;
-        if (out) row_store<VEC>(out + pos, v);
-        if (last && p.save_state) row_store<VEC>(state + pos, v);
+        const float(&v)[4] = DIR == 0 ? x[e] : b;
+        if (out && SHIFT) {  // a stored row need not lie on the boundaries of the table's
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            if (P.in(pos + k)) out[pos + k] = v[k];
+        } else if (out) {
+          P.store(out, pos, v);
+        }
+        if (last && p.save_state) P.store(state, pos, v);
       }
     }
     if (DIR == 0 || !last) {
@@ -148,8 +168,7 @@ __global__ void __launch_bounds__(kRowMaxThreads) row_steps_kernel(const PropPar
 // pass left in out at D decode loci ([D][N][N], row i = recipient i), t = theta beta, are divided by their
 // emission theta^l (1 - mu where the donor carries the target's allele at l, mu elsewhere; a zero theta
 // means alpha = 0 too, and the entry is 0) and replaced by half distances.  A zero normaliser gives p =
-// eps for every donor (Sec. 2.2); the target's own entry is 0.  Rows are whole quads
-// on 16-byte boundaries.  Bound by memory (posteriors at N = 10000: 249 us, 4.8 TB/s; before, with the
+// eps for every donor (Sec. 2.2); the target's own entry is 0.  Bound by memory (posteriors at N = 10000: 249 us, 4.8 TB/s; before, with the
 // rows read twice, 442 us) and, with distances, by the logarithms too.
 struct PostArgs {
   const float *alpha, *beta;  // DEC 0; DEC 1: null and, where out holds alpha alone, the backward's t 2^100
@@ -161,14 +180,13 @@ struct PostArgs {
   DecodeLoci dl;
 };
 
-template <int DEC, int E4>
+template <int DEC, int E4, bool SHIFT>
 __global__ void __launch_bounds__(kRowMaxThreads) row_posterior_kernel(const __grid_constant__ PostArgs a) {
   constexpr float eps = 2.220446049250313e-16f;
-  constexpr int VEC = 4;
-  using P = RowPos<E4, VEC>;
   __shared__ float buf[32];
   const int N = a.N, r = blockIdx.x, i = DEC ? r : a.t0 + r;
   float* o = a.out + ((size_t)(DEC ? blockIdx.y : 0) * (DEC ? N : 0) + r) * N;
+  const RowQuads<SHIFT> P(N, o);
   const uint32_t* bits = nullptr;
   uint32_t inv = 0u;
   float im = 0.0f, ix = 0.0f;
@@ -179,35 +197,35 @@ __global__ void __launch_bounds__(kRowMaxThreads) row_posterior_kernel(const __g
     im = a.thm[l] > 0.0f ? 1.0f / a.thm[l] : 0.0f;
     ix = a.thx[l] > 0.0f ? 1.0f / a.thx[l] : 0.0f;
   }
-  float q[P::COUNT][VEC];
+  float q[E4][4];
   float s = 0.0f;
 #pragma unroll
-  for (int e = 0; e < P::COUNT; ++e) {
-    const int pos = P::at(e);
+  for (int e = 0; e < E4; ++e) {
+    const int pos = P.at(e);
 #pragma unroll
-    for (int k = 0; k < VEC; ++k) q[e][k] = 0.0f;
+    for (int k = 0; k < 4; ++k) q[e][k] = 0.0f;
     if (pos < N) {
       if (DEC) {
-        row_load<VEC>(o + pos, q[e]);
+        P.load(o, pos, q[e]);
         if (a.beta) {
-          float t[VEC];
-          row_load<VEC>(a.beta + (o - a.out) + pos, t);
+          float t[4];
+          P.load(a.beta + (o - a.out), pos, t);
 #pragma unroll
-          for (int k = 0; k < VEC; ++k) q[e][k] *= t[k];
+          for (int k = 0; k < 4; ++k) q[e][k] *= t[k];
         }
-        const uint32_t w = (bits[pos >> 5] ^ inv) >> (pos & 31);
+        const uint32_t w = P.bits(bits, pos) ^ inv;
 #pragma unroll
-        for (int k = 0; k < VEC; ++k) q[e][k] *= (w >> k) & 1u ? im : ix;
+        for (int k = 0; k < 4; ++k) q[e][k] *= (w >> k) & 1u ? im : ix;
       } else {
-        float b[VEC];
-        row_load<VEC>(a.alpha + (size_t)r * N + pos, q[e]);
-        row_load<VEC>(a.beta + (size_t)r * N + pos, b);
+        float b[4];
+        P.load(a.alpha + (size_t)r * N, pos, q[e]);
+        P.load(a.beta + (size_t)r * N, pos, b);
 #pragma unroll
-        for (int k = 0; k < VEC; ++k) q[e][k] *= b[k] * kProdScale;
+        for (int k = 0; k < 4; ++k) q[e][k] *= b[k] * kProdScale;
       }
 #pragma unroll
-      for (int k = 0; k < VEC; ++k) {
-        if (pos + k == i) q[e][k] = 0.0f;
+      for (int k = 0; k < 4; ++k) {
+        if (pos + k == i || !P.in(pos + k)) q[e][k] = 0.0f;
         s += q[e][k];
       }
     }
@@ -215,16 +233,16 @@ __global__ void __launch_bounds__(kRowMaxThreads) row_posterior_kernel(const __g
   const float Z = row_sum(s, buf);
   const float invZ = Z > 0.0f ? 1.0f / Z : 0.0f;
 #pragma unroll
-  for (int e = 0; e < P::COUNT; ++e) {
-    const int pos = P::at(e);
+  for (int e = 0; e < E4; ++e) {
+    const int pos = P.at(e);
     if (pos < N) {
-      float v[VEC];
+      float v[4];
 #pragma unroll
-      for (int k = 0; k < VEC; ++k) {
+      for (int k = 0; k < 4; ++k) {
         const float p = Z > 0.0f ? q[e][k] * invZ : eps;
         v[k] = pos + k == i ? 0.0f : (DEC || a.mode == 1 ? -0.5f * logf(fmaxf(p, eps)) : p);
       }
-      row_store<VEC>(o + pos, v);
+      P.store(o, pos, v);
     }
   }
 }

@@ -27,12 +27,14 @@
 // run in blocks of 64.  At the start of a block (and at a window change) a lane loads the block's 64
 // bits of each of its donors from the haplotype-major words (8 bytes of a 32-byte sector), XORs them
 // with the target's and transposes them in registers to one word per locus and 32 slots, bit s = slot
-// s differs from the target; the words wait in shared memory.  A locus then needs its words, a packed
-// FFMA2 and FADD2 per pair of slots and one predicated multiply per slot: theta (c x + r) = f (c b x + r b)
-// with b = max(1-mu, mu) and f in {1, min/b}, the number of matching slots is a population count, and
-// the per-locus logarithms are taken 32 at a time.  Padding slots count as mismatches; they start at 0
-// when their window starts and so hold one common value xs, which the row sum subtracts.  The
-// per-locus constants of the next block are copied with cp.async while the current one runs.
+// s differs from the target; the words wait in shared memory, and the outside donors' emissions at the
+// block's loci are worked out a locus per lane.  A locus then needs its words, a packed FFMA2 and FADD2
+// per pair of slots and one predicated multiply per slot, and its logarithm is taken with 31 others.
+// Emissions are divided by b = max(1-mu, mu) throughout, f in {1, min(1-mu, mu)/b}: the factor cancels in
+// every ratio of the chain, and the log-likelihood gets the sum of log b back at the end (multiplying
+// it into c and r would round 1 - rho the same way at every locus).  Padding slots take the smaller
+// factor; they start at 0 when their window starts and so hold one common value xs, which the row sum
+// subtracts.  The per-locus constants of the next block are copied with cp.async while the current one runs.
 //
 // Bound by the dependent chain of a locus (row sum, division, multiply, add), so what counts is the warps that
 // cover it: 128 registers and 12.8 KB a warp leave four a scheduler (bits are gathered and transposed 16 slots
