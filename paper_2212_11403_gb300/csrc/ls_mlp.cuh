@@ -6,16 +6,17 @@
 // two-float sums.
 //
 // One gradient is three launches:
-//   mlp_rows_kernel    tiles of 64 rows: both layers forward, the loss, dZ2, dH1 = dZ2 W2^T and the
+//   mlp_rows_kernel    tiles of up to 64 rows: both layers forward, the loss, dZ2, dH1 = dZ2 W2^T and the
 //                      gradients of W1, b1, b2, w3, b3 (one partial per CTA); only H1 and dZ2 go to memory
 //   mlp_dw2_kernel     H1^T dZ2 in 128 x 128 tiles, split over the rows
 //   mlp_update_kernel  the partials' sums in a fixed order, and the Adam update or the gradient itself
 // What bounds them is the FP32 pipe (3 x 2 x 65536 FLOP per row): packed FFMA2 on an 8 x 8 tile of
-// outputs per thread, both operands from shared memory.  64 rows per CTA (96 KB, two CTAs per SM) keep
-// every SM busy from 9728 rows on and hold a whole row of the hidden layers, so nothing but H1 and dZ2
-// is written between the layers.
-// Twenty training steps of 16384 rows: 195.7 -> 4.2 ms (before: naive 16 x 16 GEMM tiles, one thread
-// per column sum, twelve launches, seven allocations and a synchronisation a step).
+// outputs per thread, both operands from shared memory.  A CTA holds whole rows of the hidden layers, so
+// nothing but H1 and dZ2 is written between the layers, and its time goes with its rows: the tile is 2, 4,
+// 6, 7 or 8 rows a warp, whichever has the fewest rows in the fullest SM (two CTAs each).
+// Twenty training steps of 16384 / 2048 rows: 195.7 / 33.9 -> 3.4 / 1.5 ms (before: naive 16 x 16 GEMM
+// tiles, one thread per column sum, twelve launches, seven allocations and a synchronisation a step; with
+// 64-row tiles and a serial sum of the partials 4.0 ms at 16384).
 //
 // Inference uses the BF16 MMA kernel of ls_mlp_tc.cuh.
 #pragma once
@@ -36,8 +37,8 @@ constexpr int kOffW3 = kOffB2 + 256;
 constexpr int kOffB3 = kOffW3 + 256;
 constexpr int kMlpParams = kOffB3 + 1;
 
-constexpr int kTrRows = 64;      // rows per tile of mlp_rows_kernel
-constexpr int kTrThreads = 256;  // 8 warps: warp w holds rows 8w..8w+7, lane q columns 4q.. and 128 + 4q..
+constexpr int kTrRows = 64;      // most rows per tile of mlp_rows_kernel
+constexpr int kTrThreads = 256;  // 8 warps: warp w holds RW rows from RW w, lane q columns 4q.. and 128 + 4q..
 constexpr int kTrK = 16;         // weight rows per staged chunk
 // dynamic shared memory: hidden tile [64][256], two weight chunks [16][256]
 constexpr int kTrSmem = (kTrRows * 256 + 2 * kTrK * 256) * 4;
@@ -85,9 +86,10 @@ __device__ __forceinline__ void two_sum(float& s, float& e, float v) {
   s = t;
 }
 
-// acc[r][.] += A[8 warp + r][k] Bg[k][columns of the lane], k < 256: A in shared memory, Bg [256][256]
+// acc[r][.] += A[RW warp + r][k] Bg[k][columns of the lane], k < 256: A in shared memory, Bg [256][256]
 // in global memory staged through the two chunks at Wc.  Starts and ends with a CTA barrier behind it.
-__device__ __forceinline__ void mlp_tile_gemm(const float* A, const float* __restrict__ Bg, float* Wc, float2 (&acc)[8][4]) {
+template <int RW>
+__device__ __forceinline__ void mlp_tile_gemm(const float* A, const float* __restrict__ Bg, float* Wc, float2 (&acc)[RW][4]) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   auto stage = [&](int c) {
     float* d = Wc + (c & 1) * kTrK * 256;
@@ -99,7 +101,7 @@ __device__ __forceinline__ void mlp_tile_gemm(const float* A, const float* __res
     mlp_cp_commit();
   };
 #pragma unroll
-  for (int r = 0; r < 8; ++r)
+  for (int r = 0; r < RW; ++r)
 #pragma unroll
     for (int j = 0; j < 4; ++j) acc[r][j] = make_float2(0.f, 0.f);
   stage(0);
@@ -109,18 +111,18 @@ __device__ __forceinline__ void mlp_tile_gemm(const float* A, const float* __res
     __syncthreads();  // chunk c is complete, and everyone is done with the chunk the next copies overwrite
     if (c + 1 < 256 / kTrK) stage(c + 1);
     const float* b = Wc + (c & 1) * kTrK * 256 + 4 * lane;
-    const float* a = A + (8 * warp) * 256 + c * kTrK;
+    const float* a = A + (RW * warp) * 256 + c * kTrK;
 #pragma unroll
     for (int k = 0; k < kTrK; k += 2) {
-      float2 av[8];
+      float2 av[RW];
 #pragma unroll
-      for (int r = 0; r < 8; ++r) av[r] = *reinterpret_cast<const float2*>(a + r * 256 + k);
+      for (int r = 0; r < RW; ++r) av[r] = *reinterpret_cast<const float2*>(a + r * 256 + k);
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
         const float4 b0 = *reinterpret_cast<const float4*>(b + (k + q) * 256);
         const float4 b1 = *reinterpret_cast<const float4*>(b + (k + q) * 256 + 128);
 #pragma unroll
-        for (int r = 0; r < 8; ++r) {
+        for (int r = 0; r < RW; ++r) {
           const float v = q ? av[r].y : av[r].x;
           const float2 vv = make_float2(v, v);
           acc[r][0] = __ffma2_rn(vv, make_float2(b0.x, b0.y), acc[r][0]);
@@ -134,23 +136,25 @@ __device__ __forceinline__ void mlp_tile_gemm(const float* A, const float* __res
   __syncthreads();
 }
 
+template <int RW>
 __global__ void __launch_bounds__(kTrThreads, 2) mlp_rows_kernel(const MlpBatch m) {
+  constexpr int ROWS = 8 * RW;
   extern __shared__ __align__(16) float tr_smem[];
-  float* A = tr_smem;                  // [64][256]: H1, then dZ2
+  float* A = tr_smem;                  // [ROWS][256]: H1, then dZ2
   float* Wc = A + kTrRows * 256;       // weight chunks; between the products, scratch of the column sums
-  __shared__ float Xs[kTrRows][kMlpIn];
-  __shared__ float ys[kTrRows];
+  __shared__ float Xs[ROWS][kMlpIn];
+  __shared__ float ys[ROWS];
   __shared__ double redd[8][2];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int row0 = 8 * warp;
+  const int row0 = RW * warp;
   auto col = [&](int j) { return (j >> 2) * 128 + 4 * lane + (j & 3); };  // j-th of the lane's 8 columns
   const float* p = m.p;
   float* part = m.part + (size_t)blockIdx.x * kTrPart;
-  double lsum = 0.0, dsum = 0.0;  // lanes < 8: row row0 + lane of every tile
+  double lsum = 0.0, dsum = 0.0;  // lanes < RW: row row0 + lane of every tile
   bool first = true;
-  for (long long r0 = (long long)blockIdx.x * kTrRows; r0 < m.B; r0 += (long long)gridDim.x * kTrRows, first = false) {
-    const int rows = (int)min((long long)kTrRows, m.B - r0);
-    for (int e = tid; e < kTrRows * kMlpIn; e += kTrThreads) {
+  for (long long r0 = (long long)blockIdx.x * ROWS; r0 < m.B; r0 += (long long)gridDim.x * ROWS, first = false) {
+    const int rows = (int)min((long long)ROWS, m.B - r0);
+    for (int e = tid; e < ROWS * kMlpIn; e += kTrThreads) {
       const int r = e / kMlpIn, k = e % kMlpIn;
       long long src = r0 + r;
       if (m.drawn) src = (long long)(splitmix_at(m.seed, m.first + (uint64_t)src + 1) % (uint64_t)m.n_src);
@@ -164,7 +168,7 @@ __global__ void __launch_bounds__(kTrThreads, 2) mlp_rows_kernel(const MlpBatch 
       for (int k = 0; k < kMlpIn; ++k) w1[k] = p[kOffW1 + k * 256 + tid];
       const float b1 = p[kOffB1 + tid];
 #pragma unroll 4
-      for (int r = 0; r < kTrRows; ++r) {
+      for (int r = 0; r < ROWS; ++r) {
         float z = 0.0f;
 #pragma unroll
         for (int k = 0; k < kMlpIn; ++k) z = fmaf(Xs[r][k], w1[k], z);
@@ -176,20 +180,20 @@ __global__ void __launch_bounds__(kTrThreads, 2) mlp_rows_kernel(const MlpBatch 
     __syncthreads();
     uint32_t live[2] = {0u, 0u};  // H1 > 0 at this thread's outputs of the last product, bit 4 r + j
 #pragma unroll
-    for (int r = 0; r < 8; ++r)
+    for (int r = 0; r < RW; ++r)
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const float4 v = *reinterpret_cast<const float4*>(A + (row0 + r) * 256 + 128 * h + 4 * lane);
         live[h] |= ((v.x > 0.f ? 1u : 0u) | (v.y > 0.f ? 2u : 0u) | (v.z > 0.f ? 4u : 0u) | (v.w > 0.f ? 8u : 0u)) << (4 * r);
       }
-    float2 acc[8][4];
+    float2 acc[RW][4];
     mlp_tile_gemm(A, p + kOffW2, Wc, acc);  // Z2 before its bias
     {
       // score, loss and ds of the warp's rows, dZ2 into A; column sums of dZ2 (db2) and of ds H2 (dw3)
       const float b3 = p[kOffB3];
-      float ds[8];
+      float ds[RW];
 #pragma unroll
-      for (int r = 0; r < 8; ++r) {
+      for (int r = 0; r < RW; ++r) {
         float s = 0.0f;
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
@@ -212,7 +216,7 @@ __global__ void __launch_bounds__(kTrThreads, 2) mlp_rows_kernel(const MlpBatch 
         const float w3 = p[kOffW3 + col(j)];
         float g3 = 0.0f, gs = 0.0f, ge = 0.0f;
 #pragma unroll
-        for (int r = 0; r < 8; ++r) {
+        for (int r = 0; r < RW; ++r) {
           float& z = (j & 1) ? acc[r][j >> 1].y : acc[r][j >> 1].x;
           g3 = fmaf(ds[r], fmaxf(z, 0.0f), g3);
           z = z > 0.0f ? ds[r] * w3 : 0.0f;
@@ -223,7 +227,7 @@ __global__ void __launch_bounds__(kTrThreads, 2) mlp_rows_kernel(const MlpBatch 
         Wc[(16 + warp) * 256 + col(j)] = ge;
       }
 #pragma unroll
-      for (int r = 0; r < 8; ++r)
+      for (int r = 0; r < RW; ++r)
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           const float4 v = make_float4(acc[r][2 * h].x, acc[r][2 * h].y, acc[r][2 * h + 1].x, acc[r][2 * h + 1].y);
@@ -254,7 +258,7 @@ __global__ void __launch_bounds__(kTrThreads, 2) mlp_rows_kernel(const MlpBatch 
 #pragma unroll
         for (int k = 0; k < kMlpIn; ++k) gw[k] = 0.0f;
 #pragma unroll
-        for (int r = 0; r < 8; ++r) {
+        for (int r = 0; r < RW; ++r) {
           const float a = (j & 1) ? acc[r][j >> 1].y : acc[r][j >> 1].x;
           const float z = (live[j >> 2] >> (4 * r + (j & 3))) & 1u ? a : 0.0f;
           two_sum(gs, ge, z);
@@ -381,9 +385,10 @@ struct MlpUpdate {
 };
 
 // The gradient of every parameter from the partials, in a fixed order, and its Adam update:
-// m = b1 m + (1-b1) g; v = b2 v + (1-b2) g^2; p -= lr * mhat / (sqrt(vhat) + eps).  Blocks 0..255: W2, a
-// thread per weight; 256..343: 32 parameters of W1, b1, b2 and w3 each (8 threads a parameter, sums in
-// double); the last block: b3 and the loss.
+// m = b1 m + (1-b1) g; v = b2 v + (1-b2) g^2; p -= lr * mhat / (sqrt(vhat) + eps).  Blocks 0..255: 256 weights
+// of W2 each (four threads of 16-byte loads per quad, each a quarter of the splits); 256..343: 32 parameters of
+// W1, b1, b2 and w3 each (8 threads a parameter, pairs of floats joined in double); the last block: b3 and the
+// loss.
 constexpr int kUpdBlocks = 256 + 11 * 256 / 32 + 1;
 __global__ void __launch_bounds__(256) mlp_update_kernel(const MlpUpdate u) {
   const int tid = threadIdx.x;
@@ -401,11 +406,21 @@ __global__ void __launch_bounds__(256) mlp_update_kernel(const MlpUpdate u) {
     if (e >= kOffW2 && e < kOffB2) u.w2t[((e - kOffW2) & 255) * 256 + ((e - kOffW2) >> 8)] = pn;
   };
   if (blockIdx.x < 256) {
-    const int e = blockIdx.x * 256 + tid;
-    float g = 0.0f;
+    __shared__ float4 part[4][64];
+    const int q = tid & 63, grp = tid >> 6;
+    float4 g = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 8
-    for (int s = 0; s < u.splits; ++s) g += u.partw[(size_t)s * 65536 + e];
-    apply(kOffW2 + e, g);
+    for (int s = grp; s < u.splits; s += 4) {
+      const float4 v = *reinterpret_cast<const float4*>(u.partw + (size_t)s * 65536 + blockIdx.x * 256 + 4 * q);
+      g.x += v.x;
+      g.y += v.y;
+      g.z += v.z;
+      g.w += v.w;
+    }
+    part[grp][q] = g;
+    __syncthreads();
+    const float* f = reinterpret_cast<const float*>(&part[0][0]) + tid;
+    apply(kOffW2 + blockIdx.x * 256 + tid, (f[0] + f[256]) + (f[512] + f[768]));
     return;
   }
   if (blockIdx.x + 1 < gridDim.x) {
@@ -413,16 +428,26 @@ __global__ void __launch_bounds__(256) mlp_update_kernel(const MlpUpdate u) {
     const int q = (blockIdx.x - 256) * 32 + (tid & 31), sec = q >> 8, c = q & 255;  // sec 0..7 W1, 8 b1, 9 b2, 10 w3
     const int o0 = (sec < 9 ? sec : sec == 9 ? kMlpIn + 2 : kMlpIn + 4) * 256 + c;
     const bool pair = sec == 8 || sec == 9;  // (sum, error)
-    double t = 0.0;
-    for (int b = tid >> 5; b < u.ctas; b += 8) {
-      const float* o = u.part + (size_t)b * kTrPart + o0;
-      t += (double)o[0];
-      if (pair) t += (double)o[256];
+    float ps = 0.0f, pe = 0.0f;
+    for (int b0 = tid >> 5; b0 < u.ctas; b0 += 64) {  // eight CTAs' loads ahead of their sums
+      float v[8], w[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const int b = b0 + 8 * k;
+        const float* o = u.part + (size_t)min(b, u.ctas - 1) * kTrPart + o0;
+        v[k] = b < u.ctas ? o[0] : 0.0f;
+        w[k] = pair && b < u.ctas ? o[256] : 0.0f;
+      }
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        two_sum(ps, pe, v[k]);
+        pe += w[k];
+      }
     }
-    red[tid >> 5][tid & 31] = t;
+    red[tid >> 5][tid & 31] = (double)ps + (double)pe;
     __syncthreads();
     if (tid < 32) {
-      t = 0.0;
+      double t = 0.0;
       for (int k = 0; k < 8; ++k) t += red[k][tid];
       apply(sec < 8 ? kOffW1 + q : (sec == 8 ? kOffB1 : sec == 9 ? kOffB2 : kOffW3) + c, (float)t);
     }

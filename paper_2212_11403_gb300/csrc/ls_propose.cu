@@ -120,14 +120,22 @@ unsigned blocks(long long n, int t = 256) { return (unsigned)((n + t - 1) / t); 
 
 // Scratch of the gradient of up to B rows and its launches.
 struct GradWork {
-  int ctas = 0, splits = 0, split_rows = 0;
+  int ctas = 0, splits = 0, split_rows = 0, rw = 8;  // rw: rows per warp of mlp_rows_kernel
   float *H1, *dZ2, *part, *partw, *w2t;
   double *partd, *loss;
   int setup(const ls_mlp* m, Bufs& b, int B, int nloss, cudaStream_t s) {
     int nsm = 0, rc;
     TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, m->device));
-    TRY(cudaFuncSetAttribute(lsk::mlp_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, lsk::kTrSmem));
-    ctas = std::min(2 * nsm, (int)((B + (long long)lsk::kTrRows - 1) / lsk::kTrRows));  // two CTAs per SM
+    // two CTAs per SM; the tile with the fewest rows in the fullest one
+    long long best = -1;
+    for (int w : {8, 7, 6, 4, 2}) {
+      const long long tiles = (B + 8ll * w - 1) / (8 * w), rows = (tiles + 2 * nsm - 1) / (2 * nsm) * w;
+      if (best >= 0 && rows >= best) continue;
+      best = rows;
+      rw = w;
+      ctas = (int)std::min<long long>(2 * nsm, tiles);
+    }
+    TRY(rows_kernel([](auto k) { return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, lsk::kTrSmem); }));
     // four quarter tiles of dW2 per split, two CTAs per SM, at least 128 rows a split
     const int most = std::max(1, 2 * nsm / 4);
     split_rows = std::max(128, (int)((B + (long long)most - 1) / most));
@@ -141,6 +149,17 @@ struct GradWork {
     TRY(cudaGetLastError());
     return LS_OK;
   }
+  // f applied to the rows kernel of rw rows a warp
+  template <class F>
+  cudaError_t rows_kernel(F f) const {
+    switch (rw) {
+      case 2: return f(lsk::mlp_rows_kernel<2>);
+      case 4: return f(lsk::mlp_rows_kernel<4>);
+      case 6: return f(lsk::mlp_rows_kernel<6>);
+      case 7: return f(lsk::mlp_rows_kernel<7>);
+      default: return f(lsk::mlp_rows_kernel<8>);
+    }
+  }
   // gradient of the batch (its rows and source in mb), then into u.g or, with u.g null, an Adam update
   int run(const ls_mlp* m, lsk::MlpBatch mb, lsk::MlpUpdate u, cudaStream_t s) const {
     mb.p = m->p;
@@ -149,7 +168,10 @@ struct GradWork {
     mb.dZ2 = dZ2;
     mb.part = part;
     mb.partd = partd;
-    lsk::mlp_rows_kernel<<<ctas, lsk::kTrThreads, lsk::kTrSmem, s>>>(mb);
+    TRY(rows_kernel([&](auto k) {
+      k<<<ctas, lsk::kTrThreads, lsk::kTrSmem, s>>>(mb);
+      return cudaGetLastError();
+    }));
     lsk::mlp_dw2_kernel<<<dim3(4, splits), 256, lsk::kDwSmem, s>>>(H1, dZ2, mb.B, split_rows, partw);
     u.partw = partw;
     u.splits = splits;

@@ -40,6 +40,30 @@ def test_gradient_row_tiles(ls, n):
     assert float(np.linalg.norm(g - rg)) <= 1e-5 * float(np.linalg.norm(rg))
 
 
+# every tile height (2, 4, 6, 7, 8 rows a warp) with its most CTAs, ragged
+@pytest.mark.parametrize("n", [15, 17, 304 * 16, 304 * 32 - 5, 304 * 48 - 1, 304 * 56 - 3, 304 * 64])
+def test_gradient_tile_heights(ls, n):
+    import torch
+    p, X, y = problem(n + n // 8 + 50, n)
+    # rows with a pre-activation at the kink of a ReLU are left out: FP32 and float64 may take different
+    # sides there, which moves the gradient by a row's whole share of a unit
+    W1, b1, W2, b2, _, _ = op.unpack(p)
+    Z1 = X.astype(np.float64) @ W1 + b1
+    Z2 = np.maximum(Z1, 0.0) @ W2 + b2
+    keep = np.flatnonzero((np.abs(Z1).min(1) > 1e-5) & (np.abs(Z2).min(1) > 1e-5))[:n]
+    assert len(keep) == n
+    X, y = X[keep], y[keep]
+    m = ls.ls_mlp_create(p)
+    try:
+        g, loss = ls.ls_mlp_grad(m, torch.from_numpy(X).cuda(), torch.from_numpy(y).cuda())
+    finally:
+        ls.ls_mlp_destroy(m)
+    rl, rg = op.mlp_loss_grad(p.astype(np.float64), X.astype(np.float64), y.astype(np.float64))
+    assert abs(loss - rl) <= 1e-5 * rl
+    # FP32 products and sums of 256 terms of either sign: about sqrt(256) 2^-24 of the terms' size
+    assert float(np.linalg.norm(g - rg)) <= 1e-5 * float(np.linalg.norm(rg))
+
+
 @pytest.mark.parametrize("n,batch", [(5, 64), (1000, 100), (3000, 777)])
 def test_training_matches_adam_in_float64(ls, n, batch):
     import torch
