@@ -221,7 +221,8 @@ int ls_distance(ls_ctx* ctx, const ls_table* fwd, const ls_table* bck, float* d_
  * device or host memory (host: the result is copied back before the call returns).  pac_out
  * (host, may be NULL) receives the PAC log-likelihood sum_i log P(h_i | h_-i) (Sec. 1).
  * status_out (device uint32 [N], may be NULL) receives per-target status bits.  Uses library-
- * owned scratch of D*N*N floats (cached in the context).  Synchronous when pac_out is given or
+ * owned scratch: D*N*N floats for host output (cached in the context), and as many for the call only, up to
+ * 256 MB, where small data sets run their two directions side by side.  Synchronous when pac_out is given or
  * d_out is host memory; returns LS_WARN_* when such a call saw underflow/overflow. */
 int ls_run_all(ls_ctx* ctx, const int32_t* decode_loci, int32_t D, float* d_out, double* pac_out,
                uint32_t* status_out, ls_stream_t stream);
@@ -236,7 +237,9 @@ int ls_run_all(ls_ctx* ctx, const int32_t* decode_loci, int32_t D, float* d_out,
  * of Eq. transition and App. A.3's emission), computed by two forward statistic passes and one
  * backward pass in FP32 with FP64 sums.  Outputs are host doubles (any may be NULL); dlogrho has
  * K entries, 0 for groups without intervals.  Device memory: (3 * (number of nonempty groups) + 2)
- * floats per target and donor, allocated for the call and freed before it returns; the targets
+ * floats per target and donor, held for the call only (the scratch of this and the other calls
+ * that need some comes from a pool per device, which keeps at most 4 GB between calls until the
+ * device's last context and network is destroyed); the targets
  * are processed in blocks whose scratch stays within 16 GiB (the environment variable
  * LS_GRAD_BUDGET_MB, a positive number of MiB, sets another ceiling; one target is the minimum).
  * Synchronous.  Requires the uniform prior (LS_ERR_UNSUPPORTED otherwise), rho < 1 and mu < 1.
@@ -353,8 +356,9 @@ int ls_sparse_run_all(ls_ctx* ctx, const int32_t* idx, int32_t K, int32_t WS, in
  * address (cudaGetSymbolAddress) with the context's device current, so make the first call before
  * any stream capture.  All calls share the one area and reuse it: the call clears what must start
  * at zero, and calls whose GPU work overlaps (different streams, or different contexts on one
- * device running at once) race on it.  It launches exactly the kernels ls_run_all launches (the
- * same planner), on the caller's stream only.  N > LS_NOALLOC_MAX_N gives LS_ERR_UNSUPPORTED; D is
+ * device running at once) race on it.  It launches the propagation kernels that ls_run_all launches (the
+ * same planner), one after the other on the caller's stream only; ls_run_all runs the two
+ * directions of small data sets (N up to 1216) side by side, with bit-identical results.  N > LS_NOALLOC_MAX_N gives LS_ERR_UNSUPPORTED; D is
  * limited to 64 as for ls_run_all.  Synchronous when pac_out is given (it waits for the PAC sum and
  * returns LS_WARN_* like ls_run_all), asynchronous otherwise.  A device wait that ran out of time
  * is recorded in the scratch area and reported as LS_ERR_DEVICE by the next call that passes

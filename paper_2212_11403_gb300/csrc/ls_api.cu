@@ -242,12 +242,22 @@ void base_params(ls_ctx* c, lsk::PropParams& p, int dir) {
   p.err = c->err;
 }
 
-// the side stream and the events that fork it from and join it to a caller's stream
-int side_stream(ls_ctx* c) {
-  if (c->side) return LS_OK;
-  CUDA_TRY(cudaEventCreateWithFlags(&c->fork_ev, cudaEventDisableTiming));
-  CUDA_TRY(cudaEventCreateWithFlags(&c->join_ev, cudaEventDisableTiming));
-  CUDA_TRY(cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking));
+// The side stream: what follows on it waits for the work on s so far (fork), and s for the work on it (join)
+int fork_side(ls_ctx* c, cudaStream_t s) {
+  std::lock_guard<std::mutex> lk(c->side_mu);
+  if (!c->side) {
+    if (!c->fork_ev) CUDA_TRY(cudaEventCreateWithFlags(&c->fork_ev, cudaEventDisableTiming));
+    if (!c->join_ev) CUDA_TRY(cudaEventCreateWithFlags(&c->join_ev, cudaEventDisableTiming));
+    CUDA_TRY(cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking));
+  }
+  CUDA_TRY(cudaEventRecord(c->fork_ev, s));
+  CUDA_TRY(cudaStreamWaitEvent(c->side, c->fork_ev, 0));
+  return LS_OK;
+}
+int join_side(ls_ctx* c, cudaStream_t s) {
+  std::lock_guard<std::mutex> lk(c->side_mu);
+  CUDA_TRY(cudaEventRecord(c->join_ev, c->side));
+  CUDA_TRY(cudaStreamWaitEvent(s, c->join_ev, 0));
   return LS_OK;
 }
 
@@ -262,9 +272,7 @@ int run_launches(ls_ctx* c, lsk::PropParams p, int t_begin, int t_count, cudaStr
   // LS_TAIL_OVERLAP=0 (a measurement switch) runs both on the caller's stream, in order.
   const char* ov = getenv("LS_TAIL_OVERLAP");
   if (nlp == 2 && !(ov && ov[0] == '0')) {
-    if ((rc = side_stream(c))) return rc;
-    CUDA_TRY(cudaEventRecord(c->fork_ev, s));
-    CUDA_TRY(cudaStreamWaitEvent(c->side, c->fork_ev, 0));
+    if ((rc = fork_side(c, s))) return rc;
     for (int k = 1; k >= 0; --k) {
       const Launch& L = lp[k];
       p.t_begin = L.t_begin;
@@ -273,9 +281,7 @@ int run_launches(ls_ctx* c, lsk::PropParams p, int t_begin, int t_count, cudaStr
       if (e != cudaSuccess) return fail(LS_ERR_CUDA, "propagation launch (TPW=%d W=%d KQ=%d): %s", L.k->tpw, L.k->w,
                                         L.k->kq, cudaGetErrorString(e));
     }
-    CUDA_TRY(cudaEventRecord(c->join_ev, c->side));
-    CUDA_TRY(cudaStreamWaitEvent(s, c->join_ev, 0));
-    return LS_OK;
+    return join_side(c, s);
   }
   for (int i = 0; i < nlp; ++i) {
     const Launch& L = lp[i];
@@ -329,6 +335,22 @@ int run_row_steps(lsk::PropParams p, int t_begin, int t_count, cudaStream_t s) {
   if (e != cudaSuccess) return fail(LS_ERR_CUDA, "row step launch: %s", cudaGetErrorString(e));
   return LS_OK;
 }
+
+struct DevBufs {  // scratch of one call, in the order of its stream
+  cudaStream_t s;
+  std::vector<void*> v;
+  explicit DevBufs(cudaStream_t stream) : s(stream) {}
+  DevBufs(const DevBufs&) = delete;
+  ~DevBufs() {
+    for (void* p : v) ls_tmp_free(p, s);
+  }
+  template <class T>
+  int get(T** p, size_t n) {
+    int rc = ls_tmp_alloc((void**)p, sizeof(T) * std::max<size_t>(n, 1), s);
+    if (!rc) v.push_back(*p);
+    return rc;
+  }
+};
 
 // Posterior rows: DEC 0 grid (rows), DEC 1 grid (N, D).  The row kernel takes buffers on 16-byte boundaries:
 // posteriors up to 64 elements a thread (N = 5000 / 10000 / 20000 / 26000: 100 / 442 / 893 / 1170 -> 64 / 249 /
@@ -420,7 +442,6 @@ void free_ctx(ls_ctx* c) {
   cudaFree(c->status_scratch);
   cudaFree(c->err);
   cudaFree(c->dscratch);
-  cudaFree(c->tscratch);
   for (auto& e : c->ev)
     if (e) cudaEventDestroy(e);
   if (c->fork_ev) cudaEventDestroy(c->fork_ev);
@@ -1077,41 +1098,45 @@ int ls_distance(ls_ctx* ctx, const ls_table* fwd, const ls_table* bck, float* d_
 // Small data sets leave most of the GPU idle and are bound by the latency of a locus, so ls_run_all runs
 // their two directions side by side: where each is one launch and all CTAs of both are resident at once
 // (one-warp and 8-target CTAs: N up to 1216).  The backward then leaves t 2^100 at the decode loci in
-// scratch of the context (at most kPairBytes, kept until the context is destroyed) and the decode forms the
-// product alpha (t 2^100) that it otherwise finds.  Not while profiling (the phases are timed one after
-// the other), with LS_TAIL_OVERLAP=0, or where the scratch would have to be allocated during a capture.
-// N = 200 / 500 / 1003 / 1200, L = 4000: 2087 / 2175 / 2897 /
-// 3445 -> 1107 / 1262 / 1931 / 2469 us.
+// scratch of the call (at most kPairBytes) and the decode forms the product alpha (t 2^100) that it otherwise
+// finds.  Not while profiling (the phases are timed one after the other), with LS_TAIL_OVERLAP=0, in a
+// captured call, or where the scratch cannot be had.  Calls on other streams that run at the same time have
+// scratch of their own; their backwards follow one another on the side stream.
+// N = 200 / 500 / 1003 / 1200, L = 4000: 2087 / 2175 / 2897 / 3445 -> 1107 / 1262 / 1931 / 2469 us with
+// scratch kept in the context; the call's own costs about 10 us more (N = 200, L = 1000: 371 -> 380).
 static constexpr size_t kPairBytes = (size_t)256 << 20;
 
-// whether to run the directions side by side, with the scratch for it
-static int plan_pair(ls_ctx* c, int D, cudaStream_t s, bool* both) {
-  *both = false;
-  const char* ov = getenv("LS_TAIL_OVERLAP");
-  const size_t n = (size_t)D * c->N * c->N, bytes = sizeof(float) * n;
-  if (c->profile || (ov && ov[0] == '0') || bytes > kPairBytes) return LS_OK;
-  Launch lp[2];
-  int nlp = 0, rc = plan(c, 0, c->N, lp, &nlp);
-  if (rc) return rc;
-  if (nlp != 1 || 2 * lp[0].grid * lp[0].k->cpt > lp[0].per_sm * c->num_sms) return LS_OK;
-  if (!c->side || c->tscratch_bytes < bytes) {
+struct Pair {  // one call's side-by-side run; the side stream is joined before the scratch goes back
+  ls_ctx* c;
+  DevBufs db;
+  float* t = nullptr;  // [D][N][N]
+  bool both = false, forked = false;
+  Pair(ls_ctx* ctx, cudaStream_t s) : c(ctx), db(s) {}
+  ~Pair() { join(); }
+  int prepare(int D) {
+    const char* ov = getenv("LS_TAIL_OVERLAP");
+    const size_t n = (size_t)D * c->N * c->N;
+    if (c->profile || (ov && ov[0] == '0') || sizeof(float) * n > kPairBytes) return LS_OK;
+    Launch lp[2];
+    int nlp = 0, rc = plan(c, 0, c->N, lp, &nlp);
+    if (rc) return rc;
+    if (nlp != 1 || 2 * lp[0].grid * lp[0].k->cpt > lp[0].per_sm * c->num_sms) return LS_OK;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    CUDA_TRY(cudaStreamIsCapturing(s, &cap));
-    if (cap != cudaStreamCaptureStatusNone) return LS_OK;
-    if ((rc = side_stream(c))) return rc;
-    if (c->tscratch_bytes < bytes) {
-      // an earlier call's work on the old scratch may still run on its stream: cudaFree waits for it
-      cudaFree(c->tscratch);
-      c->bytes -= c->tscratch_bytes;
-      c->tscratch = nullptr;
-      c->tscratch_bytes = 0;
-      if (dev_alloc(c, (void**)&c->tscratch, bytes) != LS_OK) return LS_OK;  // no memory to spare: one after the other
-      c->tscratch_bytes = bytes;
-    }
+    CUDA_TRY(cudaStreamIsCapturing(db.s, &cap));
+    both = cap == cudaStreamCaptureStatusNone && db.get(&t, n) == LS_OK;
+    return LS_OK;
   }
-  *both = true;
-  return LS_OK;
-}
+  int fork() {
+    const int rc = fork_side(c, db.s);
+    forked = rc == LS_OK;
+    return rc;
+  }
+  int join() {
+    const bool f = forked;
+    forked = false;
+    return f ? join_side(c, db.s) : LS_OK;
+  }
+};
 
 int ls_run_all(ls_ctx* ctx, const int32_t* decode_loci, int32_t D, float* d_out, double* pac_out, uint32_t* status_out,
                ls_stream_t stream) {
@@ -1143,15 +1168,15 @@ int ls_run_all(ls_ctx* ctx, const int32_t* decode_loci, int32_t D, float* d_out,
   uint32_t* stat = ctx->status_scratch;
   CUDA_TRY(cudaMemsetAsync(stat, 0, sizeof(uint32_t) * N, s));
   const bool prof = ctx->profile;
-  bool both = false;  // the directions side by side
-  if ((rc = plan_pair(ctx, D, s, &both))) return rc;
+  Pair pair(ctx, s);
+  if ((rc = pair.prepare(D))) return rc;
+  const bool both = pair.both;  // the directions side by side
+  if (both && (rc = pair.fork())) return rc;
   cudaStream_t sb = both ? ctx->side : s;  // the backward's stream
   if (both) {
-    CUDA_TRY(cudaEventRecord(ctx->fork_ev, s));
-    CUDA_TRY(cudaStreamWaitEvent(sb, ctx->fork_ev, 0));
     if (D > 0) {  // the backward multiplies what it finds at the decode loci by t 2^100
       const long long n = (long long)D * N * N;
-      lsk::fill_kernel<<<(unsigned)std::min<long long>((n + 1023) / 1024, 4096), 256, 0, sb>>>(ctx->tscratch, n, 1.0f);
+      lsk::fill_kernel<<<(unsigned)std::min<long long>((n + 1023) / 1024, 4096), 256, 0, sb>>>(pair.t, n, 1.0f);
       CUDA_TRY(cudaGetLastError());
     }
   }
@@ -1187,16 +1212,13 @@ int ls_run_all(ls_ctx* ctx, const int32_t* decode_loci, int32_t D, float* d_out,
     p.store_loci[k] = decode_loci[D - 1 - k];
     p.store_slot[k] = D - 1 - k;
   }
-  p.alpha_dec = both ? ctx->tscratch : dd;
+  p.alpha_dec = both ? pair.t : dd;
   if ((rc = run_launches(ctx, p, 0, N, sb, &ctx->launches[1]))) return rc;
-  if (both) {
-    CUDA_TRY(cudaEventRecord(ctx->join_ev, sb));
-    CUDA_TRY(cudaStreamWaitEvent(s, ctx->join_ev, 0));
-  }
+  if ((rc = pair.join())) return rc;
   if (prof) CUDA_TRY(cudaEventRecord(ctx->ev[2], s));
   ctx->launches[2] = ctx->launches[3] = 0;
   if (D > 0) {
-    if ((rc = decode_rows(ctx, decode_loci, D, dd, both ? ctx->tscratch : nullptr, s))) return rc;
+    if ((rc = decode_rows(ctx, decode_loci, D, dd, both ? pair.t : nullptr, s))) return rc;
     ctx->launches[2] = 1;
   }
   if (prof) CUDA_TRY(cudaEventRecord(ctx->ev[3], s));
@@ -1278,21 +1300,6 @@ int pick_stat(ls_ctx* c, int most, StatPick* out) {
   return LS_OK;
 }
 
-struct DevBufs {  // scratch of one call, in the order of its stream
-  cudaStream_t s;
-  std::vector<void*> v;
-  explicit DevBufs(cudaStream_t stream) : s(stream) {}
-  DevBufs(const DevBufs&) = delete;
-  ~DevBufs() {
-    for (void* p : v) ls_tmp_free(p, s);
-  }
-  template <class T>
-  int get(T** p, size_t n) {
-    int rc = ls_tmp_alloc((void**)p, sizeof(T) * std::max<size_t>(n, 1), s);
-    if (!rc) v.push_back(*p);
-    return rc;
-  }
-};
 // Device scratch ceiling of ls_pac_grad (targets are processed in blocks that fit it): 16 GiB, or
 // the environment variable LS_GRAD_BUDGET_MB when it is set to a positive number of MiB.
 size_t grad_budget() {

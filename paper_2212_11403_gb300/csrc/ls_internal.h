@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cstdint>
+#include <mutex>
 #include <vector>
 
 #include <cuda_runtime.h>
@@ -82,17 +83,17 @@ struct ls_ctx {
   int* err = nullptr;             // device error word
   float* dscratch = nullptr;      // host-output staging for ls_run_all
   size_t dscratch_bytes = 0;
-  float* tscratch = nullptr;      // ls_run_all of small data sets: the backward's values at the decode loci
-  size_t tscratch_bytes = 0;
   int num_sms = 0;
   int ntables = 0;
   // profiling of ls_run_all phases
   bool profile = false;
   bool profiled = false;
   cudaEvent_t ev[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
-  // side stream for the tail launch of a main/tail plan (fork/join events on the caller's stream)
+  // side stream for the tail launch of a main/tail plan and for the backward of small data sets (fork/join
+  // events on the caller's stream; the mutex keeps each record and its wait together)
   cudaStream_t side = nullptr;
   cudaEvent_t fork_ev = nullptr, join_ev = nullptr;
+  std::mutex side_mu;
   int launches[4] = {0, 0, 0, 0};
 };
 
