@@ -1,7 +1,7 @@
 // ls_mlp_tc.cuh -- the proposal network's scorer on the fifth-generation tensor cores (tcgen05).
 //
 // scores[r] = w3 . relu(W2^T relu(W1^T x_r + b1) + b2) + b3 for n rows of BF16 features, in tiles
-// of 128 rows, one persistent CTA of 256 threads per SM.  Both products run on the tensor cores,
+// of 128 rows, one persistent CTA of 18 warps per SM.  Both products run on the tensor cores,
 // issued by one thread, FP32 accumulators in tensor memory:
 //   layer 1: one tcgen05.mma (M = 128, N = 256, K = 16: the 7 features zero-padded) of the feature
 //            tile by W1;
