@@ -1272,11 +1272,15 @@ struct StatPick {
   int smem = 0;
 };
 
-// most: targets a block may hold (a CTA's targets share its rotation, so blocks are whole CTAs)
-int pick_stat(ls_ctx* c, int most, StatPick* out) {
+// The tile for blocks of `targets` targets.  Where each can have an SM of its own, one target per CTA: its
+// slices are the shortest (N = 4096, L = 300, 20 groups, 16 / 150 targets: 670 / 681 against 776 / 815 us with
+// two per CTA), and it fits any scratch ceiling.  Otherwise the tile that is cheapest for all targets, whose
+// blocks are whole CTAs (a CTA's targets share its rotation).
+int pick_stat(ls_ctx* c, int targets, StatPick* out) {
+  const bool single = targets <= c->num_sms;
   double bc = 1e300;
   for (const auto& k : registry()) {
-    if (k.st != 1 || !k.serves(c->N) || k.tpw > most) continue;
+    if (k.st != 1 || !k.serves(c->N) || (single && k.tpw > 1)) continue;
     const int smem = k.smem_bytes(c->rw2);
     if (smem > 227 * 1024) continue;
     bool ok = true;
@@ -1456,7 +1460,7 @@ int ls_pac_grad(ls_ctx* ctx, int32_t t_from, int32_t t_to, const int32_t* interv
   const size_t per_target = ((size_t)3 * G + 2) * (size_t)N * sizeof(float);
   int Tb = (int)std::min<size_t>((size_t)T, std::max<size_t>(1, grad_budget() / per_target));
   StatPick sp;
-  if ((rc = pick_stat(ctx, Tb < T ? Tb : N, &sp))) return rc;
+  if ((rc = pick_stat(ctx, Tb, &sp))) return rc;
   if (Tb < T) Tb -= Tb % sp.k->tpw;
   if (Tb < T) {
     int nb = 0;

@@ -230,11 +230,13 @@ void ls_register_group18(std::vector<PropKernelInfo>& out) {
 }
 #elif LS_INST_GROUP == 8
 void ls_register_group8(std::vector<PropKernelInfo>& out) {
-  // statistic passes of the adjoint (uniform prior): two tiles per lane.  As many targets per CTA as keep a
-  // lane's slices long, because the work per locus that does not scale with the slice is the larger part of a
-  // short one (N = 2003, L = 1999, one target of 16 slots a lane against four of 63: 7.8 / 8.5 -> 3.7 / 3.3 ms
-  // for the two passes).  Every N up to 10240 is served; the ranges do not overlap beyond 512.
+  // statistic passes of the adjoint (uniform prior): two tiles per lane.  With many targets, as many per CTA as
+  // keep a lane's slices long, because the work per locus that does not scale with the slice is the larger
+  // part of a short one (N = 2003, L = 1999, one target of 16 slots a lane against four of 63: 7.8 / 8.5 ->
+  // 3.7 / 3.3 ms for the two passes).  One target per CTA serves every N up to 10240 too: it is the faster
+  // tile where the targets would not fill the GPU otherwise, and the one that fits any scratch ceiling.
   LS_REGS(1, 4, 1);
+  LS_REGS(1, 4, 8);
   LS_REGS(8, 4, 4);
   LS_REGS(8, 4, 8);
 }
