@@ -90,9 +90,16 @@ std::vector<PropKernelInfo>& registry() {
   return v;
 }
 
+void tmp_trim();
+
 int dev_alloc(ls_ctx* c, void** p, size_t bytes) {
   if (bytes == 0) bytes = 16;
   cudaError_t e = cudaMalloc(p, bytes);
+  if (e == cudaErrorMemoryAllocation) {  // the scratch kept between calls may be what is missing
+    cudaGetLastError();
+    tmp_trim();
+    e = cudaMalloc(p, bytes);
+  }
   if (e != cudaSuccess) {
     cudaGetLastError();
     *p = nullptr;
@@ -497,6 +504,17 @@ std::vector<TmpPool> g_tmp;  // by device
 TmpPool& tmp_of(int device) {  // with g_tmp_mu held
   if ((int)g_tmp.size() <= device) g_tmp.resize(device + 1);
   return g_tmp[device];
+}
+
+// gives back what the current device's pool keeps, the scratch of calls in flight included once they are done
+void tmp_trim() {
+  int device = 0;
+  if (cudaGetDevice(&device) == cudaSuccess) {
+    cudaDeviceSynchronize();
+    std::lock_guard<std::mutex> lk(g_tmp_mu);
+    if (cudaMemPool_t pool = tmp_of(device).pool) cudaMemPoolTrimTo(pool, 0);
+  }
+  cudaGetLastError();
 }
 }  // namespace
 
