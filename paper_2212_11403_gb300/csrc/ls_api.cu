@@ -343,22 +343,6 @@ int run_row_steps(lsk::PropParams p, int t_begin, int t_count, cudaStream_t s) {
   return LS_OK;
 }
 
-struct DevBufs {  // scratch of one call, in the order of its stream
-  cudaStream_t s;
-  std::vector<void*> v;
-  explicit DevBufs(cudaStream_t stream) : s(stream) {}
-  DevBufs(const DevBufs&) = delete;
-  ~DevBufs() {
-    for (void* p : v) ls_tmp_free(p, s);
-  }
-  template <class T>
-  int get(T** p, size_t n) {
-    int rc = ls_tmp_alloc((void**)p, sizeof(T) * std::max<size_t>(n, 1), s);
-    if (!rc) v.push_back(*p);
-    return rc;
-  }
-};
-
 // Posterior rows: DEC 0 grid (rows), DEC 1 grid (N, D).  The row kernel takes buffers on 16-byte boundaries:
 // posteriors up to 64 elements a thread (N = 5000 / 10000 / 20000 / 26000: 100 / 442 / 893 / 1170 -> 64 / 249 /
 // 637 / 902 us), the decode in place up to 20 (N = 2500 / 5000: 25 / 74 -> 16 / 49 us; at N = 10000 both take
@@ -1126,7 +1110,7 @@ static constexpr size_t kPairBytes = (size_t)256 << 20;
 
 struct Pair {  // one call's side-by-side run; the side stream is joined before the scratch goes back
   ls_ctx* c;
-  DevBufs db;
+  CallScratch db;
   float* t = nullptr;  // [D][N][N]
   bool both = false, forked = false;
   Pair(ls_ctx* ctx, cudaStream_t s) : c(ctx), db(s) {}
@@ -1487,7 +1471,7 @@ int ls_pac_grad(ls_ctx* ctx, int32_t t_from, int32_t t_to, const int32_t* interv
     if (Tb >= wave) Tb = (Tb / wave) * wave;
   }
   Tb = std::min(Tb, T);
-  DevBufs db(s);
+  CallScratch db(s);
   float *d_gam, *d_eta, *A, *Wst, *B, *xst, *wst;
   uint8_t* d_rst;
   double *logF, *EM, *Rg, *sums;
@@ -1586,7 +1570,7 @@ int ls_sparse_run_all(ls_ctx* ctx, const int32_t* idx, int32_t K, int32_t WS, in
   if (pout_out && !is_device_ptr(pout_out)) return fail(LS_ERR_ARG, "pout_out must be device memory");
   const int Wn = (L + WS - 1) / WS;
   cudaStream_t s = (cudaStream_t)stream;
-  DevBufs db(s);
+  CallScratch db(s);
   float *P, *lost, *poolf = nullptr, *share = nullptr;
   double* logs;
   uint32_t* stat;

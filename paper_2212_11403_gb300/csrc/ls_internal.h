@@ -1,6 +1,7 @@
 // ls_internal.h -- host-side structures shared by the libls translation units.
 #pragma once
 
+#include <algorithm>
 #include <cstdint>
 #include <mutex>
 #include <vector>
@@ -40,6 +41,32 @@ int ls_tmp_alloc(void** p, size_t bytes, cudaStream_t s);
 void ls_tmp_free(void* p, cudaStream_t s);
 void ls_tmp_hold(int device);
 void ls_tmp_release(int device);
+
+// Scratch of one call.  What goes beyond kTmpKeep is the call's own allocation: from the pool it would be
+// mapped and unmapped by every call, which takes longer (a gradient with 16 GB of scratch at N = 9000: 62.2
+// against 48.3 ms, a proposal at N = 60000: 76.1 against 48.8 ms).
+struct CallScratch {
+  cudaStream_t s;
+  std::vector<void*> pooled, own;
+  size_t taken = 0;
+  explicit CallScratch(cudaStream_t stream) : s(stream) {}
+  CallScratch(const CallScratch&) = delete;
+  ~CallScratch() {
+    for (void* p : pooled) ls_tmp_free(p, s);
+    if (!own.empty()) cudaStreamSynchronize(s);
+    for (void* p : own) cudaFree(p);
+  }
+  template <class T>
+  int get(T** p, size_t n) {
+    const size_t bytes = sizeof(T) * std::max<size_t>(n, 1);
+    const bool pool = taken + bytes <= kTmpKeep;
+    const int rc = pool ? ls_tmp_alloc((void**)p, bytes, s) : ls_dev_alloc((void**)p, bytes);
+    if (rc) return rc;
+    if (pool) taken += bytes;
+    (pool ? pooled : own).push_back(*p);
+    return 0;
+  }
+};
 
 namespace lsk {
 struct SparseParams;

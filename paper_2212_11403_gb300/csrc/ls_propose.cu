@@ -38,22 +38,6 @@ int dev_alloc(void*, void** p, size_t n) { return ls_dev_alloc(p, n); }
     if (e_ != cudaSuccess) return fail(LS_ERR_CUDA, "%s: %s", #x, cudaGetErrorString(e_));     \
   } while (0)
 
-struct Bufs {  // scratch of one call, in the order of its stream
-  cudaStream_t s;
-  std::vector<void*> v;
-  explicit Bufs(cudaStream_t stream) : s(stream) {}
-  Bufs(const Bufs&) = delete;
-  ~Bufs() {
-    for (void* q : v) ls_tmp_free(q, s);
-  }
-  template <class T>
-  int get(T** q, size_t n) {
-    int rc = ls_tmp_alloc((void**)q, sizeof(T) * std::max<size_t>(n, 1), s);
-    if (!rc) v.push_back(*q);
-    return rc;
-  }
-};
-
 // BF16 transposed copies for the MMA kernel
 __global__ void mlp_refresh_kernel(const float* __restrict__ p, __nv_bfloat16* __restrict__ w1t,
                                    __nv_bfloat16* __restrict__ w2t) {
@@ -123,7 +107,7 @@ struct GradWork {
   int ctas = 0, splits = 0, split_rows = 0, rw = 8;  // rw: rows per warp of mlp_rows_kernel
   float *H1, *dZ2, *part, *partw, *w2t;
   double *partd, *loss;
-  int setup(const ls_mlp* m, Bufs& b, int B, int nloss, cudaStream_t s) {
+  int setup(const ls_mlp* m, CallScratch& b, int B, int nloss, cudaStream_t s) {
     int nsm = 0, rc;
     TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, m->device));
     // two CTAs per SM; the tile with the fewest rows in the fullest one
@@ -275,7 +259,7 @@ int ls_mlp_forward(const ls_mlp* m, const float* X, int64_t n, float* scores, ls
 int ls_mlp_grad(ls_mlp* m, const float* X, const float* y, int32_t n, float* grad, double* loss, ls_stream_t stream) {
   if (!m || !X || !y || n < 1) return fail(LS_ERR_ARG, "bad arguments");
   cudaStream_t s = (cudaStream_t)stream;
-  Bufs b(s);
+  CallScratch b(s);
   GradWork gw;
   int rc = gw.setup(m, b, n, 1, s);
   if (rc) return rc;
@@ -300,7 +284,7 @@ int ls_mlp_train(ls_mlp* m, const float* X, const float* y, int64_t n, int32_t s
                  uint64_t seed, double* loss_out, ls_stream_t stream) {
   if (!m || !X || !y || n < 1 || steps < 0 || batch < 1) return fail(LS_ERR_ARG, "bad arguments");
   cudaStream_t s = (cudaStream_t)stream;
-  Bufs b(s);
+  CallScratch b(s);
   GradWork gw;
   const int ntail = std::min(steps, std::max(1, steps / 10));  // the steps whose losses are averaged
   int rc = gw.setup(m, b, batch, ntail, s);
@@ -349,7 +333,7 @@ struct PropWork {
   std::vector<int> nv;
 };
 
-int prop_setup(ls_ctx* c, Bufs& b, PropWork& pw, cudaStream_t s) {
+int prop_setup(ls_ctx* c, CallScratch& b, PropWork& pw, cudaStream_t s) {
   pw.N = c->N;
   pw.L = c->L;
   pw.Wn = (c->L + lsk::kPropWS - 1) / lsk::kPropWS;
@@ -419,7 +403,7 @@ int ls_propose_window(ls_ctx* ctx, int32_t C, int32_t w, int32_t* cand_out, floa
   if (!ctx || C < 1 || !cand_out) return fail(LS_ERR_ARG, "bad arguments");
   cudaSetDevice(ctx->device);
   cudaStream_t s = (cudaStream_t)stream;
-  Bufs b(s);
+  CallScratch b(s);
   PropWork pw;
   int rc = prop_setup(ctx, b, pw, s);
   if (rc) return rc;
@@ -444,7 +428,7 @@ int ls_propose(ls_ctx* ctx, int32_t C, int32_t K, const ls_mlp* mlp, int32_t* id
   if (mlp && (C < K || C > 2048)) return fail(LS_ERR_ARG, "need K <= C <= 2048 candidates for the MLP stage");
   cudaSetDevice(ctx->device);
   cudaStream_t s = (cudaStream_t)stream;
-  Bufs b(s);
+  CallScratch b(s);
   PropWork pw;
   int rc = prop_setup(ctx, b, pw, s);
   if (rc) return rc;

@@ -2,7 +2,9 @@
 import numpy as np
 import pytest
 
+import oracle
 from paper_2212_11403_gb300 import synth
+from tests.test_gpu_grad import check_grad
 
 pytestmark = pytest.mark.gpu
 
@@ -39,3 +41,23 @@ def test_table_fits_beside_kept_scratch(ls):
             ls.ls_table_destroy(table)
         ls.ls_destroy(big)
         ls.ls_destroy(ctx)
+
+
+def test_scratch_beyond_what_is_kept(ls):
+    """4.8 GB of scratch: the oracle's gradient, and no more than 4 GB held afterwards."""
+    import torch
+    N, L, K = 1000, 420, 400
+    w = synth.make_workload("ls_n10000_l10000", N=N, L=L, seed=4)
+    iv = synth.rho_intervals(L, K)
+    ctx = ls.ls_create(w["h"])
+    try:
+        ls.ls_set_params(ctx, w["rho"], w["mu"])
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        rc, pac, gm, gr = ls.ls_pac_grad(ctx, iv, K)
+        torch.cuda.synchronize()
+        assert before - torch.cuda.mem_get_info()[0] <= 4 << 30
+    finally:
+        ls.ls_destroy(ctx)
+    assert rc == 0
+    check_grad(pac, gm, gr, oracle.pac_grad(w["h"], w["rho"], w["mu"], iv, K), w["rho"], w["mu"], L, iv, K, N, N)
