@@ -221,9 +221,11 @@ int ls_distance(ls_ctx* ctx, const ls_table* fwd, const ls_table* bck, float* d_
  * device or host memory (host: the result is copied back before the call returns).  pac_out
  * (host, may be NULL) receives the PAC log-likelihood sum_i log P(h_i | h_-i) (Sec. 1).
  * status_out (device uint32 [N], may be NULL) receives per-target status bits.  Uses library-
- * owned scratch: D*N*N floats for host output (cached in the context), and as many for the call only, up to
- * 256 MB, where small data sets run their two directions side by side.  Synchronous when pac_out is given or
- * d_out is host memory; returns LS_WARN_* when such a call saw underflow/overflow. */
+ * owned scratch: D*N*N floats for host output (cached in the context, so such calls of one context follow one
+ * another), N doubles and words for the results read back, and D*N*N floats, up to 256 MB, where small data sets
+ * run their two directions side by side (both for the call only).  Other calls of one context may be in flight
+ * on several streams at once.  Synchronous when pac_out is given or d_out is host memory; returns LS_WARN_*
+ * when such a call saw underflow/overflow. */
 int ls_run_all(ls_ctx* ctx, const int32_t* decode_loci, int32_t D, float* d_out, double* pac_out,
                uint32_t* status_out, ls_stream_t stream);
 

@@ -1102,8 +1102,8 @@ int ls_distance(ls_ctx* ctx, const ls_table* fwd, const ls_table* bck, float* d_
 // (one-warp and 8-target CTAs: N up to 1216).  The backward then leaves t 2^100 at the decode loci in
 // scratch of the call (at most kPairBytes) and the decode forms the product alpha (t 2^100) that it otherwise
 // finds.  Not while profiling (the phases are timed one after the other), with LS_TAIL_OVERLAP=0, in a
-// captured call, or where the scratch cannot be had.  Calls on other streams that run at the same time have
-// scratch of their own; their backwards follow one another on the side stream.
+// captured call, or where the scratch cannot be had.  Calls in flight at the same time on other streams follow
+// one another on the side stream.
 // N = 200 / 500 / 1003 / 1200, L = 4000: 2087 / 2175 / 2897 / 3445 -> 1107 / 1262 / 1931 / 2469 us with
 // scratch kept in the context; the call's own costs about 10 us more (N = 200, L = 1000: 371 -> 380).
 static constexpr size_t kPairBytes = (size_t)256 << 20;
@@ -1167,10 +1167,21 @@ int ls_run_all(ls_ctx* ctx, const int32_t* decode_loci, int32_t D, float* d_out,
     }
     dd = ctx->dscratch;
   }
-  uint32_t* stat = ctx->status_scratch;
-  CUDA_TRY(cudaMemsetAsync(stat, 0, sizeof(uint32_t) * N, s));
   const bool prof = ctx->profile;
   Pair pair(ctx, s);
+  // What the call reads back (log scales, then status words) is the call's own, so that calls in flight on other
+  // streams do not write to it; an asynchronous call leaves its status words in status_out.  The context's
+  // arrays take what nobody reads, and stand in where scratch cannot be had.
+  const bool sync = host_out || pac_out;
+  const size_t rbytes = (sizeof(double) + sizeof(uint32_t)) * N;
+  double* logs = ctx->logs_scratch;
+  uint32_t* stat = status_out && !sync ? status_out : ctx->status_scratch;
+  char* own = nullptr;
+  if (sync && pair.db.get(&own, rbytes) == LS_OK) {
+    logs = reinterpret_cast<double*>(own);
+    stat = reinterpret_cast<uint32_t*>(logs + N);
+  }
+  CUDA_TRY(cudaMemsetAsync(stat, 0, sizeof(uint32_t) * N, s));
   if ((rc = pair.prepare(D))) return rc;
   const bool both = pair.both;  // the directions side by side
   if (both && (rc = pair.fork())) return rc;
@@ -1191,7 +1202,7 @@ int ls_run_all(ls_ctx* ctx, const int32_t* decode_loci, int32_t D, float* d_out,
   p.init = 1;
   p.tab_t0 = 0;
   p.state_rows = N;
-  p.logs = ctx->logs_scratch;
+  p.logs = logs;
   p.status = stat;
   p.n_store = D;
   for (int k = 0; k < D; ++k) {
@@ -1234,14 +1245,19 @@ int ls_run_all(ls_ctx* ctx, const int32_t* decode_loci, int32_t D, float* d_out,
     CUDA_TRY(cudaEventRecord(ctx->ev[4], s));
     ctx->profiled = true;
   }
-  if (status_out) CUDA_TRY(cudaMemcpyAsync(status_out, stat, sizeof(uint32_t) * N, cudaMemcpyDeviceToDevice, s));
-  const bool sync = host_out || pac_out;
+  if (status_out && stat != status_out)
+    CUDA_TRY(cudaMemcpyAsync(status_out, stat, sizeof(uint32_t) * N, cudaMemcpyDeviceToDevice, s));
   if (host_out) CUDA_TRY(cudaMemcpyAsync(d_out, dd, dbytes, cudaMemcpyDeviceToHost, s));
   if (!sync) return LS_OK;
-  std::vector<double> lf(N);
-  std::vector<uint32_t> sh(N);
-  CUDA_TRY(cudaMemcpyAsync(lf.data(), ctx->logs_scratch, sizeof(double) * N, cudaMemcpyDeviceToHost, s));
-  CUDA_TRY(cudaMemcpyAsync(sh.data(), stat, sizeof(uint32_t) * N, cudaMemcpyDeviceToHost, s));
+  std::vector<char> back(rbytes);
+  const double* lf = reinterpret_cast<const double*>(back.data());
+  const uint32_t* sh = reinterpret_cast<const uint32_t*>(lf + N);
+  if (own) {
+    CUDA_TRY(cudaMemcpyAsync(back.data(), own, rbytes, cudaMemcpyDeviceToHost, s));
+  } else {
+    CUDA_TRY(cudaMemcpyAsync(back.data(), logs, sizeof(double) * N, cudaMemcpyDeviceToHost, s));
+    CUDA_TRY(cudaMemcpyAsync(back.data() + sizeof(double) * N, stat, sizeof(uint32_t) * N, cudaMemcpyDeviceToHost, s));
+  }
   if ((rc = read_err_word(ctx, s))) return rc;
   if (pac_out) {
     double pac = 0.0;
@@ -1249,7 +1265,7 @@ int ls_run_all(ls_ctx* ctx, const int32_t* decode_loci, int32_t D, float* d_out,
     *pac_out = pac;
   }
   uint32_t any = 0;
-  for (auto v : sh) any |= v;
+  for (int i = 0; i < N; ++i) any |= sh[i];
   // total underflow is reported first: the NaNs it leaves behind also trip the overflow check
   if (any & 1u) return LS_WARN_UNDERFLOW;
   if (any & 2u) return LS_WARN_OVERFLOW;

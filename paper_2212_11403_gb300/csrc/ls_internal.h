@@ -104,7 +104,7 @@ struct ls_ctx {
   float pi_u = 0.0f;
   int mu_vec = 0;                 // mu given per locus
   std::vector<double> rho_h, mu_h;  // host copies (the gradient's constant terms)
-  // scratch
+  // scratch (log scales and status words that no call reads back)
   double* logs_scratch = nullptr; // [N]
   uint32_t* status_scratch = nullptr;  // [N]
   int* err = nullptr;             // device error word
