@@ -34,10 +34,9 @@ cudaError_t ls_launch_emission(const float* thm, const float* thx, int L, float*
 
 cudaError_t ls_launch_lookahead(const int32_t* idx, int N, int Wn, int K, int span, int32_t* U, cudaStream_t s) {
   const long long n = (long long)N * Wn;
-  // up to eight warps a CTA, as many as 48 KB of bitmaps allow (beyond N = 393216 one warp and more)
-  const int bytes = (N + 31) / 32 * 4, warps = bytes * 8 <= 48 * 1024 ? 8 : bytes < 48 * 1024 ? 48 * 1024 / bytes : 1;
-  cudaError_t e = cudaFuncSetAttribute(lsk::lookahead_sets_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, warps * bytes);
-  if (e != cudaSuccess) return e;
+  // up to eight warps a CTA, as many as 48 KB of bitmaps allow (one warp's take more only beyond N = 393216,
+  // whose distance matrix would not fit any memory)
+  const int bytes = (N + 31) / 32 * 4, warps = std::max(1, std::min(8, 48 * 1024 / bytes));
   lsk::lookahead_sets_kernel<<<(unsigned)((n + warps - 1) / warps), warps * 32, warps * bytes, s>>>(idx, N, Wn, K, span, U);
   return cudaGetLastError();
 }
