@@ -134,6 +134,16 @@ struct Cand {
 // in fixed arrays so that the allocation-free pipeline shares it).
 constexpr int kMaxCand = 64;
 
+// Leave for a variant's kernels to be launched with `smem` bytes of dynamic shared memory.  The limit is set to one
+// value for every N (the SM's 227 KB less 1 KB for what the kernels declare statically), so that threads with
+// contexts of different sizes never lower it for each other.
+constexpr int kMaxDynSmem = 226 * 1024;
+bool allow_smem(const PropKernelInfo& k, int smem) {
+  for (int d = 0; d < 2 && smem <= kMaxDynSmem; ++d)
+    if (cudaFuncSetAttribute(k.func[d], cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem) != cudaSuccess) return false;
+  return smem <= kMaxDynSmem;
+}
+
 // Every compiled propagation variant (no statistic passes) that serves N with the context's prior
 // kind, fits the shared-memory limit and can be resident.  LS_PROP_VARIANT="tpw,w,kq" keeps only
 // that variant: a measurement switch for tuning sweeps, honoured by every entry point alike.
@@ -151,10 +161,7 @@ int candidates(ls_ctx* c, Cand* out, int* nout) {
     if (pim && k.pi16 != c->prior_bf16) continue;
     if (pin && !(k.tpw == pa && k.w == pb && k.kq == pk)) continue;
     const int smem = k.smem_bytes(c->rw2);
-    if (smem > 227 * 1024) continue;
-    bool ok = true;
-    for (int d = 0; d < 2 && ok; ++d)
-      if (cudaFuncSetAttribute(k.func[d], cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) ok = false;
+    bool ok = allow_smem(k, smem);
     int nb = 0;
     if (ok && (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k.func[0], k.w * 32, smem) != cudaSuccess || nb < 1)) ok = false;
     if (!ok) {
@@ -1300,10 +1307,7 @@ int pick_stat(ls_ctx* c, int targets, StatPick* out) {
   for (const auto& k : registry()) {
     if (k.st != 1 || !k.serves(c->N) || (single && k.tpw > 1)) continue;
     const int smem = k.smem_bytes(c->rw2);
-    if (smem > 227 * 1024) continue;
-    bool ok = true;
-    for (int d = 0; d < 2 && ok; ++d)
-      if (cudaFuncSetAttribute(k.func[d], cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) ok = false;
+    bool ok = allow_smem(k, smem);
     int nb = 0;
     if (ok && (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k.func[1], k.w * 32, smem) != cudaSuccess || nb < 1))
       ok = false;

@@ -77,3 +77,45 @@ def test_widened_sets(ls):
     finally:
         for c in ctxs:
             ls.ls_destroy(c)
+
+
+@pytest.mark.parametrize("sizes,L,loci", [((16500, 20000), 40, 30), ((21000, 40900), 20, 12)])
+def test_table_moves(ls, sizes, L, loci):
+    import torch
+    ctxs = contexts(ls, sizes, L)
+    tables = [ls.ls_table_create(c, ls.LS_FWD, 0, 4) for c in ctxs]
+
+    def call(k):
+        a = torch.empty(4, sizes[k], device="cuda")
+
+        def f():
+            ls.ls_table_reset(tables[k])
+            ls.ls_forward(ctxs[k], tables[k], loci)
+            ls.ls_table_read(tables[k], a)
+            return a.clone()
+        return f
+
+    try:
+        in_threads([call(0), call(1)], 500)
+    finally:
+        for t in tables:
+            ls.ls_table_destroy(t)
+        for c in ctxs:
+            ls.ls_destroy(c)
+
+
+def test_gradients(ls):
+    import torch
+    sizes, L, K = (9100, 10000), 12, 2
+    ctxs = contexts(ls, sizes, L)
+
+    def call(k):
+        def f():
+            return torch.tensor(ls.ls_pac_grad(ctxs[k], synth.rho_intervals(L, K), K, 0, 3)[3])
+        return f
+
+    try:
+        in_threads([call(0), call(1)], 300)
+    finally:
+        for c in ctxs:
+            ls.ls_destroy(c)
