@@ -125,14 +125,7 @@ struct Launch {
   int per_sm;  // CTAs an SM holds
 };
 
-struct Cand {
-  const PropKernelInfo* k;
-  int smem, per_sm;
-};
-
-// Upper bound on compiled variants (the registry is a fixed list; the planner keeps its candidates
-// in fixed arrays so that the allocation-free pipeline shares it).
-constexpr int kMaxCand = 64;
+using Cand = PropCand;
 
 // Leave for a variant's kernels to be launched with `smem` bytes of dynamic shared memory.  The limit is set to one
 // value for every N (the SM's 227 KB less 1 KB for what the kernels declare statically), so that threads with
@@ -145,8 +138,10 @@ bool allow_smem(const PropKernelInfo& k, int smem) {
 }
 
 // Every compiled propagation variant (no statistic passes) that serves N with the context's prior
-// kind, fits the shared-memory limit and can be resident.  LS_PROP_VARIANT="tpw,w,kq" keeps only
-// that variant: a measurement switch for tuning sweeps, honoured by every entry point alike.
+// kind, fits the shared-memory limit and can be resident: asked for once and kept in the context (attributes and
+// occupancies of seven variants, twice a call, were 10 of the 60 us of a call of 8 loci at N = 200).
+// LS_PROP_VARIANT="tpw,w,kq" keeps only that variant: a measurement switch for tuning sweeps, honoured by every
+// entry point alike.
 int candidates(ls_ctx* c, Cand* out, int* nout) {
   *nout = 0;
   const int N = c->N;
@@ -154,21 +149,36 @@ int candidates(ls_ctx* c, Cand* out, int* nout) {
   int pa = 0, pb = 0, pk = 0;
   const char* ov = getenv("LS_PROP_VARIANT");
   const bool pin = ov && sscanf(ov, "%d,%d,%d", &pa, &pb, &pk) == 3;
-  for (const auto& k : registry()) {
-    if (*nout >= kMaxCand) break;
-    if (k.st != 0 || (k.pim != 0) != (pim != 0) || !k.serves(N)) continue;
-    // a prior matrix runs on the variants that hold it as bfloat16 exactly when it has the BF16 format
-    if (pim && k.pi16 != c->prior_bf16) continue;
-    if (pin && !(k.tpw == pa && k.w == pb && k.kq == pk)) continue;
-    const int smem = k.smem_bytes(c->rw2);
-    bool ok = allow_smem(k, smem);
-    int nb = 0;
-    if (ok && (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k.func[0], k.w * 32, smem) != cudaSuccess || nb < 1)) ok = false;
-    if (!ok) {
-      cudaGetLastError();
-      continue;
+  auto take = [&](const Cand& cd) {
+    if (!pin || (cd.k->tpw == pa && cd.k->w == pb && cd.k->kq == pk)) out[(*nout)++] = cd;
+  };
+  {
+    std::lock_guard<std::mutex> lk(c->cand_mu);
+    auto& kept = c->cand[pim ? 1 + (c->prior_bf16 ? 1 : 0) : 0];
+    if (kept.n < 0) {
+      int n = 0;
+      bool clean = true;  // after an error, which may pass, the next call asks again
+      for (const auto& k : registry()) {
+        if (n >= kMaxCand) break;
+        if (k.st != 0 || (k.pim != 0) != (pim != 0) || !k.serves(N)) continue;
+        // a prior matrix runs on the variants that hold it as bfloat16 exactly when it has the BF16 format
+        if (pim && k.pi16 != c->prior_bf16) continue;
+        const int smem = k.smem_bytes(c->rw2);
+        if (smem > kMaxDynSmem) continue;
+        int nb = 0;
+        if (!allow_smem(k, smem) ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k.func[0], k.w * 32, smem) != cudaSuccess) {
+          cudaGetLastError();
+          clean = false;
+        } else if (nb > 0) {
+          kept.c[n++] = Cand{&k, smem, nb};
+        }
+      }
+      for (int i = 0; i < n; ++i) take(kept.c[i]);
+      if (clean) kept.n = n;
+    } else {
+      for (int i = 0; i < kept.n; ++i) take(kept.c[i]);
     }
-    out[(*nout)++] = Cand{&k, smem, nb};
   }
   if (*nout == 0) {
     if (pin) return fail(LS_ERR_UNSUPPORTED, "LS_PROP_VARIANT=%s does not serve N=%d", ov, N);
@@ -1193,13 +1203,6 @@ int ls_run_all(ls_ctx* ctx, const int32_t* decode_loci, int32_t D, float* d_out,
   const bool both = pair.both;  // the directions side by side
   if (both && (rc = pair.fork())) return rc;
   cudaStream_t sb = both ? ctx->side : s;  // the backward's stream
-  if (both) {
-    if (D > 0) {  // the backward multiplies what it finds at the decode loci by t 2^100
-      const long long n = (long long)D * N * N;
-      lsk::fill_kernel<<<(unsigned)std::min<long long>((n + 1023) / 1024, 4096), 256, 0, sb>>>(pair.t, n, 1.0f);
-      CUDA_TRY(cudaGetLastError());
-    }
-  }
   if (prof) CUDA_TRY(cudaEventRecord(ctx->ev[0], s));
   // forward over all loci: alpha at the decode loci goes straight into the output buffer
   lsk::PropParams p;
@@ -1219,6 +1222,13 @@ int ls_run_all(ls_ctx* ctx, const int32_t* decode_loci, int32_t D, float* d_out,
   p.store = dd;
   if ((rc = run_launches(ctx, p, 0, N, s, &ctx->launches[0]))) return rc;
   if (prof) CUDA_TRY(cudaEventRecord(ctx->ev[1], s));
+  if (both && D > 0) {
+    // the backward multiplies what it finds at the decode loci by t 2^100.  Behind the forward's launch, whose CTAs
+    // would otherwise go where this kernel leaves room (N = 500, L = 500, 64 decode loci: 600 against 480 us)
+    const long long n = (long long)D * N * N;
+    lsk::fill_kernel<<<(unsigned)std::min<long long>((n + 1023) / 1024, 4096), 256, 0, sb>>>(pair.t, n, 1.0f);
+    CUDA_TRY(cudaGetLastError());
+  }
   // backward over all loci: alpha * beta overwrites alpha at the decode loci
   base_params(ctx, p, 1);
   p.l_first = L - 1;

@@ -24,6 +24,15 @@ struct PropKernelInfo {
   int pi16 = 0; // 1: holds the prior matrix on chip as bfloat16 (needs the BF16 prior format)
 };
 
+// a variant that serves a context, the dynamic shared memory it takes there and the CTAs an SM holds
+struct PropCand {
+  const PropKernelInfo* k;
+  int smem, per_sm;
+};
+// Upper bound on compiled variants (the registry is a fixed list; the candidates sit in fixed arrays so that the
+// allocation-free pipeline shares the planner).
+constexpr int kMaxCand = 64;
+
 void ls_register_prop_kernels(std::vector<PropKernelInfo>& out);
 
 // shared by the translation units: set the thread's error message and return code; device
@@ -121,6 +130,12 @@ struct ls_ctx {
   cudaStream_t side = nullptr;
   cudaEvent_t fork_ev = nullptr, join_ev = nullptr;
   std::mutex side_mu;
+  // the variants that serve the context, by prior kind (none, FP32, BF16), from the first plan on
+  struct {
+    int n = -1;
+    PropCand c[kMaxCand];
+  } cand[3];
+  std::mutex cand_mu;
   int launches[4] = {0, 0, 0, 0};
 };
 
