@@ -39,6 +39,7 @@ void ls_register_group18(std::vector<PropKernelInfo>& out);
 void ls_register_group19(std::vector<PropKernelInfo>& out);
 void ls_register_group20(std::vector<PropKernelInfo>& out);
 void ls_register_group21(std::vector<PropKernelInfo>& out);
+void ls_register_group22(std::vector<PropKernelInfo>& out);
 
 namespace {
 
@@ -86,6 +87,7 @@ std::vector<PropKernelInfo>& registry() {
     ls_register_group19(v);
     ls_register_group20(v);
     ls_register_group21(v);
+    ls_register_group22(v);
   });
   return v;
 }
@@ -217,15 +219,32 @@ const Cand* best_for(const Cand* cs, int nc, int count, int nsm, double* cost) {
   return best;
 }
 
-// Launch plan for targets [t_begin, t_begin + t_count): full waves of the best variant, then the
+// Where a variant and its rival serve the same N, keeps the faster one for the call: a wide tile from
+// PropKernelInfo::even loci per row transfer on (a stored row counts as one, the table's row loaded or saved as
+// two), else the others.
+void keep_faster(const lsk::PropParams& p, Cand* cs, int* nc) {
+  const Cand* wide = nullptr;
+  for (int i = 0; i < *nc; ++i)
+    if (cs[i].k->even && (!wide || cs[i].k->kq < wide->k->kq)) wide = &cs[i];
+  if (!wide || p.N <= 20480) return;
+  const int even = wide->k->even[p.dir][p.mu_vec ? 1 : 0];
+  const bool keep = even > 0 && p.n_steps >= even * (p.n_store + 2 * ((p.load_state ? 1 : 0) + (p.save_state ? 1 : 0)));
+  int n = 0;
+  for (int i = 0; i < *nc; ++i)
+    if ((cs[i].k->even != nullptr) == keep) cs[n++] = cs[i];
+  if (n) *nc = n;
+}
+
+// Launch plan of p (null: any call up to N = 20480) for targets [t_begin, t_begin + t_count): full waves of the best variant, then the
 // remainder with the variant best for it when that is cheaper.  At most two launches; no heap use
 // (the allocation-free pipeline plans with it too).
-int plan(ls_ctx* c, int t_begin, int t_count, Launch* out, int* nout) {
+int plan(ls_ctx* c, const lsk::PropParams* p, int t_begin, int t_count, Launch* out, int* nout) {
   *nout = 0;
   Cand cs[kMaxCand];
   int nc = 0;
   int rc = candidates(c, cs, &nc);
   if (rc) return rc;
+  if (p) keep_faster(*p, cs, &nc);
   double c1 = 0;
   const Cand* b1 = best_for(cs, nc, t_count, c->num_sms, &c1);
   const int per_wave_t = std::max(1, c->num_sms * b1->per_sm * b1->k->tpw / b1->k->cpt);
@@ -288,7 +307,7 @@ int join_side(ls_ctx* c, cudaStream_t s) {
 int run_launches(ls_ctx* c, lsk::PropParams p, int t_begin, int t_count, cudaStream_t s, int* nlaunch = nullptr) {
   Launch lp[2];
   int nlp = 0;
-  int rc = plan(c, t_begin, t_count, lp, &nlp);
+  int rc = plan(c, &p, t_begin, t_count, lp, &nlp);
   if (rc) return rc;
   if (nlaunch) *nlaunch = nlp;
   // A main/tail plan: the tail (few targets, one small CTA per SM, latency-bound) goes first on a
@@ -1137,7 +1156,7 @@ struct Pair {  // one call's side-by-side run; the side stream is joined before 
     const size_t n = (size_t)D * c->N * c->N;
     if (c->profile || (ov && ov[0] == '0') || sizeof(float) * n > kPairBytes) return LS_OK;
     Launch lp[2];
-    int nlp = 0, rc = plan(c, 0, c->N, lp, &nlp);
+    int nlp = 0, rc = plan(c, nullptr, 0, c->N, lp, &nlp);
     if (rc) return rc;
     if (nlp != 1 || 2 * lp[0].grid * lp[0].k->cpt > lp[0].per_sm * c->num_sms) return LS_OK;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -1560,6 +1579,7 @@ int run_list(ls_ctx* c, lsk::PropParams p, const int* d_tlist, int nf, cudaStrea
   int nc = 0, no = 0;
   int rc = candidates(c, cs, &nc);
   if (rc) return rc;
+  keep_faster(p, cs, &nc);
   for (int i = 0; i < nc; ++i)
     if (cs[i].k->tpw == 1) one[no++] = cs[i];
   if (no == 0) return fail(LS_ERR_UNSUPPORTED, "no one-target propagation variant serves N=%d", c->N);
@@ -1884,9 +1904,15 @@ extern "C" int ls_run_all_noalloc(ls_ctx* ctx, const int32_t* decode_loci, int32
   if (D > 0 && !is_device_ptr(d_out)) return fail(LS_ERR_ARG, "ls_run_all_noalloc needs d_out in device memory");
   // the same launch plan as ls_run_all (one planner, fixed arrays); planned before anything is
   // enqueued, so that an N no variant serves is refused with nothing queued
-  Launch lp[2];
-  int nl = 0;
-  if ((rc = plan(ctx, 0, N, lp, &nl))) return rc;
+  Launch lp[2][2];
+  int nl[2] = {0, 0};
+  for (int dir = 0; dir < 2; ++dir) {
+    lsk::PropParams p;
+    base_params(ctx, p, dir);
+    p.n_steps = L;
+    p.n_store = D;
+    if ((rc = plan(ctx, &p, 0, N, lp[dir], &nl[dir]))) return rc;
+  }
   NoallocScratch* sc = nullptr;
   if ((rc = noalloc_scratch(ctx->device, &sc))) return rc;
   cudaStream_t s = (cudaStream_t)stream;
@@ -1915,10 +1941,11 @@ extern "C" int ls_run_all_noalloc(ls_ctx* ctx, const int32_t* decode_loci, int32
     } else {
       p.alpha_dec = d_out;
     }
-    for (int i = 0; i < nl; ++i) {
-      p.t_begin = lp[i].t_begin;
-      p.t_count = lp[i].t_count;
-      cudaError_t e = lp[i].k->launch(dir, p, lp[i].grid, lp[i].smem, s);
+    for (int i = 0; i < nl[dir]; ++i) {
+      const Launch& launch = lp[dir][i];
+      p.t_begin = launch.t_begin;
+      p.t_count = launch.t_count;
+      cudaError_t e = launch.k->launch(dir, p, launch.grid, launch.smem, s);
       if (e != cudaSuccess) return fail(LS_ERR_CUDA, "propagation launch: %s", cudaGetErrorString(e));
     }
   }

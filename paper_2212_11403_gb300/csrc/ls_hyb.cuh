@@ -77,10 +77,10 @@ struct HybCfg {
   static constexpr int PART_OFF = STG_OFF + (PIM ? 0 : kHybQR * kHybThreads * 16);
   static constexpr int BYTES = PART_OFF + 2 * 32 * 4;
   __host__ __device__ static int smem_bytes() { return BYTES; }
-  // beyond the register-tile kernels' range (N <= 40960; with a prior matrix N <= 20480); with CL CTAs
-  // per target, beyond the one-CTA range (N <= 57344; with a prior matrix N <= 53248)
+  // beyond the range of the register-tile kernels of four warps (N <= 20480); with CL CTAs per target, beyond the
+  // one-CTA range (N <= 57344; with a prior matrix N <= 53248)
   __host__ __device__ static bool serves(int N, int CL = 1) {
-    return CL == 1 ? (N > (PIM ? 20480 : 40960) && N <= NP) : (N > (PIM ? kHybPimMaxN1 : 57344) && N <= CL * NP);
+    return CL == 1 ? (N > 20480 && N <= NP) : (N > (PIM ? kHybPimMaxN1 : 57344) && N <= CL * NP);
   }
 };
 

@@ -22,6 +22,9 @@ struct PropKernelInfo {
   bool (*serves)(int N);
   int cpt = 1;  // CTAs per target (2: a thread-block cluster of two CTAs shares one target)
   int pi16 = 0; // 1: holds the prior matrix on chip as bfloat16 (needs the BF16 prior format)
+  // a variant with a slower rival in long runs only: loci per row transfer from which it is the faster one, by
+  // direction and by kind of mu (scalar, per locus); 0: never; null: no such rival
+  const short (*even)[2] = nullptr;
 };
 
 // a variant that serves a context, the dynamic shared memory it takes there and the CTAs an SM holds

@@ -325,7 +325,8 @@ __global__ void __launch_bounds__(W * 32, ((PIM || ST) && W >= 8) || (W >= 8 && 
   // 26000); the forward, which only reads when it resumes from a table, and the 8-warp tiles of 128
   // registers keep one element at a time (measured faster, and no spills).
   auto xfer = [&](int c, float* gbase, float* w1, float* m1, float* w2, bool to_global) {
-    if constexpr (DIR == 0 || (W >= 8 && KQ <= 20 && PIM == 0)) {
+    constexpr bool ONE = W >= 8 && KQ <= 20 && PIM == 0;  // one element at a time
+    if (ONE || (DIR == 0 && (to_global || !(W == 1 || (W >= 8 && KQ > 20))))) {
       for (int idx = tid; idx < THREADS * 32; idx += THREADS) {
         const int src = idx >> 5, s = idx & 31;
         const int ln = src & 31;

@@ -66,6 +66,18 @@ bool serves_hyb(int N) {
   return lsk::HybCfg<QS, PIM>::serves(N, CL);
 }
 
+// Wide tiles (one target per CTA of 8 warps, the whole state in 24, 28, .., 40 quads of registers a lane) against the
+// large-N kernel (16 warps, state in registers and shared memory).  In us for eight targets an SM, tile / large-N:
+//   N                     24576        28672        32768        36864        40960
+//   forward, a locus      5.76 / 7.17  6.45 / 7.50  7.02 / 8.26  7.53 / 9.69  8.14 / 10.52
+//   with mu per locus     7.51 / 7.34  7.84 / 7.85  8.38 / 8.28  8.67 / 9.47  9.07 / 10.15
+//   backward, a locus     5.99 / 6.91  6.54 / 7.45  8.25 / 7.89  8.35 / 9.04  8.77 / 10.27
+//   with mu per locus     7.77 / 7.33  7.49 / 7.94  8.78 / 8.43  9.03 / 9.25  10.12 / 10.28
+//   load and save a row   158 / 131    204 / 148    207 / 160    253 / 181    255 / 201
+// and decode products cost the tile more (N = 28672, L = 64, 8 decode loci: backward 37.0 / 29.4 ms; L = 200: 57.4 /
+// 59.0; N = 26000, L = 100, 4 decode loci: 60.6 / 56.6 in all), so the tile needs enough loci per row transfer.
+constexpr short kWideEven[5][2][2] = {{{10, 0}, {30, 0}}, {{14, 0}, {40, 400}}, {{10, 0}, {0, 0}}, {{10, 22}, {45, 80}}, {{8, 14}, {30, 90}}};
+
 }  // namespace
 
 // large-N variants: one target per CTA of 16 warps, 12 quads per thread in registers and QS in
@@ -88,6 +100,10 @@ bool serves_hyb(int N) {
                                 (const void*)lsk::ls_prop_kernel<1, T, Wp, K, P, 0>},               \
                                launch_prop<T, Wp, K, P>, smem_prop<T, Wp, K, P>, serves_prop<T, Wp, K>, 1, P == 2})
 #define LS_REG(T, Wp, K) LS_REGP(T, Wp, K, 0)
+// one target per CTA of 8 warps with the whole state in registers, up to 160 slots a lane
+#define LS_REGW(K)                                                                                  \
+  LS_REG(1, 8, K);                                                                                  \
+  out.back().even = kWideEven[(K - 24) / 4]
 // statistic-pass variants: func[0] = ST 1, func[1] = ST 2
 #define LS_REGS(T, Wp, K)                                                                           \
   out.push_back(PropKernelInfo{T, Wp, K, 0, 1,                                                      \
@@ -165,18 +181,25 @@ void ls_register_group11(std::vector<PropKernelInfo>& out) {
 }
 #elif LS_INST_GROUP == 12
 void ls_register_group12(std::vector<PropKernelInfo>& out) {
-  // one target per CTA of 8 warps with the whole state in registers: N in (16384, 40960].  Against the
-  // large-N kernel (state in registers and shared memory, 16 warps) forward / backward of 100 loci take 14.9 /
-  // 16.5 against 16.5 / 17.4 ms at N = 26000, 18.2 / 22.8 against 21.1 / 21.4 at N = 30000 and 29.2 / 33.6
-  // against 36.8 / 37.9 at N = 40960; N <= 20480 runs faster with two CTAs of 4 warps an SM.
-  LS_REG(1, 8, 24);
-  LS_REG(1, 8, 28);
-  LS_REG(1, 8, 32);
+  // one target per CTA of 8 warps with the whole state in registers: N in (16384, 40960], where kWideEven says so
+  // beyond 20480; N <= 20480 runs faster with two CTAs of 4 warps an SM
+  LS_REGW(24);
+  LS_REGW(28);
+  LS_REGW(32);
 }
 #elif LS_INST_GROUP == 21
 void ls_register_group21(std::vector<PropKernelInfo>& out) {
-  LS_REG(1, 8, 36);
-  LS_REG(1, 8, 40);
+  LS_REGW(36);
+  LS_REGW(40);
+}
+#elif LS_INST_GROUP == 22
+void ls_register_group22(std::vector<PropKernelInfo>& out) {
+  // register + shared-memory state, N in (20480, 40960]
+  LS_REGH(0);
+  LS_REGH(2);
+  LS_REGH(4);
+  LS_REGH(6);
+  LS_REGH(8);
 }
 #elif LS_INST_GROUP == 13
 void ls_register_group13(std::vector<PropKernelInfo>& out) {
