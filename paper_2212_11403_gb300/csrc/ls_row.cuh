@@ -72,21 +72,25 @@ struct RowQuads {
 // element by element; a table moved by one locus is all load and save, so this kernel takes calls of
 // few steps.  N = 10000, one locus forward / backward: 658 / 520 -> 158 / 186 us (0.8 GB moved, 75 / 63 % of
 // the measured copy rate); the two reductions between load and save are what keeps it from the rest.
+// 20 elements a thread get 64 registers, four CTAs of 256 threads an SM; with the 98 the compiler would take, two
+// (tables of N = 5001 moved by 1 / 8 loci: 109 / 244 against 87 / 193 us).
 template <int DIR, int E4, bool SHIFT>
-__global__ void __launch_bounds__(kRowMaxThreads) row_steps_kernel(const PropParams p) {
+__global__ void __launch_bounds__(kRowMaxThreads, E4 == 5 ? 2 : 0) row_steps_kernel(const PropParams p) {
   __shared__ float buf[2][32];
   const int N = p.N, i = p.t_begin + blockIdx.x, row = i - p.tab_t0;
   float* state = p.state + (size_t)row * N;
   const RowQuads<SHIFT> P(N, state);
   float x[E4][4];
   int ph = 0;
-  auto total = [&](float s) {
+  // four sums of a thread's elements: in one, forty additions round the same way in every thread of an even row
+  // (N = 10000, four single steps: relative error of alpha 1.8e-7 against 9.6e-8 of the register-tile kernel)
+  auto total = [&](const float (&s)[4]) {
     ph ^= 1;
-    return row_sum(s, buf[ph]);
+    return row_sum((s[0] + s[1]) + (s[2] + s[3]), buf[ph]);
   };
   float sig_prev = 1.0f;
   {
-    float s = 0.0f;
+    float s[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
     for (int e = 0; e < E4; ++e) {
       const int pos = P.at(e);
@@ -94,7 +98,7 @@ __global__ void __launch_bounds__(kRowMaxThreads) row_steps_kernel(const PropPar
       for (int k = 0; k < 4; ++k) x[e][k] = 0.0f;
       if (p.load_state && pos < N) P.load(state, pos, x[e]);
 #pragma unroll
-      for (int k = 0; k < 4; ++k) s += x[e][k];
+      for (int k = 0; k < 4; ++k) s[k] += x[e][k];
     }
     if (p.load_state && DIR == 0) sig_prev = total(s);
   }
@@ -123,7 +127,7 @@ __global__ void __launch_bounds__(kRowMaxThreads) row_steps_kernel(const PropPar
     const uint32_t* bits = p.bits2 + (size_t)l * p.rw2;
     const uint32_t inv = (bits[i >> 5] >> (i & 31)) & 1u ? 0u : 0xffffffffu;  // match = bit ^ inv
     const float tm = p.thm[l], tx = p.thx[l];
-    float s = 0.0f;
+    float s[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
     for (int e = 0; e < E4; ++e) {
       const int pos = P.at(e);
@@ -134,7 +138,7 @@ __global__ void __launch_bounds__(kRowMaxThreads) row_steps_kernel(const PropPar
         for (int k = 0; k < 4; ++k) {
           b[k] = pos + k == i || !P.in(pos + k) ? 0.0f : fmaf(c, x[e][k], r);  // alpha before its emission, or beta
           x[e][k] = ((w >> k) & 1u ? tm : tx) * b[k];
-          s += x[e][k];
+          s[k] += x[e][k];
         }
         const float(&v)[4] = DIR == 0 ? x[e] : b;
         if (out && SHIFT) {  // a stored row need not lie on the boundaries of the table's
