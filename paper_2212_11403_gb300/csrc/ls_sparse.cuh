@@ -41,6 +41,12 @@
 // at a time for that).  N = 20003, L = 2000, K = 3 x 512: forward / backward 32.3 / 30.2 -> 14.5 / 14.7 ms
 // (before: one word and one bit test, select and count per slot and locus, set ids in registers, two warps a
 // scheduler; with three warps, transposing 32 slots at a time, 17.4 / 17.5).
+//
+// Short windows are bound by the window changes.  The lookups of eight slots run side by side in a fixed number of
+// steps, only the part of a block that the window reaches is worked out, and variants of few slots take five or
+// six CTAs per SM (72 to 96 registers): N = 10000, L = 1024, K = 256, windows of 4 / 16 / 64 / 256 loci 29.3 / 9.8 /
+// 4.5 / 3.6 -> 14.3 / 5.2 / 3.2 / 3.0 ms with sets as they are (before the blocks of 64 loci 15.7 / 6.8 / 4.9 / 4.5),
+// 92 / 23.8 / 8.7 / 5.6 -> 49 / 13.3 / 6.5 / 5.3 ms widened; the run of N = 20003 above 32.2 -> 29.3 ms in all.
 #pragma once
 
 #include <cstdint>
@@ -49,7 +55,7 @@
 
 namespace lsk {
 
-constexpr int kSparseWarps = 4;   // targets per CTA (four CTAs per SM)
+constexpr int kSparseWarps = 4;   // targets per CTA (four to six CTAs per SM)
 constexpr int kSparseChunk = 64;  // loci per block: two 32-bit haplotype-major words per donor
 constexpr int kSparseScal = 4;    // per-locus constants staged per block: 1-rho, rho, n1, emission ratio
 
@@ -126,7 +132,7 @@ __device__ __forceinline__ void transpose16x2(uint32_t (&m)[16]) {
 }
 
 template <int DIR, int KS>
-__global__ void __launch_bounds__(kSparseWarps * 32, 4) ls_sparse_kernel(const __grid_constant__ SparseParams p) {
+__global__ void __launch_bounds__(kSparseWarps * 32, KS == 8 ? 6 : KS == 4 ? 5 : 4) ls_sparse_kernel(const __grid_constant__ SparseParams p) {
   static_assert(KS % 2 == 0, "slots come in pairs");
   constexpr float eps = 2.220446049250313e-16f;
   constexpr int INF_ID = 0x7fffffff;
@@ -163,8 +169,10 @@ __global__ void __launch_bounds__(kSparseWarps * 32, 4) ls_sparse_kernel(const _
     return q < K ? p.idx[((size_t)i * p.Wn + w) * K + q] : -1;
   };
   // the words of block b (loci 64 b .. 64 b + 63) for the current set, and the outside donors' emissions
-  // (sc: the block's constants)
+  // (sc: the block's constants), where the window reaches: 32 loci at a time transposed, eight stored, the emissions
+  // of each
   auto gather = [&](int b, const float* sc) {
+    const int first = max(cur_w * p.WS - CH * b, 0), last = min(p.WS - (CH * b - cur_w * p.WS), CH);  // [first, last)
     __syncwarp();
     const uint32_t* hwb = p.hw + (size_t)(b >> 2) * N * 8 + 2 * (b & 3);
     const uint2 tw = *reinterpret_cast<const uint2*>(hwb + (size_t)i * 8);
@@ -188,25 +196,28 @@ __global__ void __launch_bounds__(kSparseWarps * 32, 4) ls_sparse_kernel(const _
       auto put = [&](uint32_t (&m)[16], int k0) {
         transpose16x2(m);
 #pragma unroll
-        for (int k = 0; k < 16; ++k) {
-          dst[(k0 + k) * step] = (uint16_t)m[k];
-          dst[(k0 + 16 + k) * step] = (uint16_t)(m[k] >> 16);
-        }
-        if (KS <= 16) {
+        for (int q = 0; q < 32; q += 8) {  // eight loci at a time
+          if (k0 + q + 8 <= first || k0 + q >= last) continue;
 #pragma unroll
-          for (int k = 0; k < 32; ++k) dst[(k0 + k) * step + 1] = 0;
+          for (int k = q; k < q + 8; ++k) {
+            const uint32_t v = k < 16 ? m[k & 15] & 0xffffu : m[k & 15] >> 16;
+            if (KS <= 16) words[32 * (k0 + k)] = v;
+            else dst[(k0 + k) * step] = (uint16_t)v;
+          }
         }
       };
-      put(lo, 0);
-      put(hi, 32);
+      if (first < 32) put(lo, 0);
+      if (last > 32) put(hi, 32);
     }
     if (p.pool) {
       const int nout = N - 1 - nset;
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
+        const int k0 = max(first - 32 * h, 0), k1 = min(last - 32 * h, 32);
+        if (k0 >= k1) continue;
         int mis = 0;  // slots (padding included) that differ from the target at locus 32 h + lane
 #pragma unroll 8
-        for (int k = 0; k < 32; ++k) {
+        for (int k = k0; k < k1; ++k) {
           int n = 0;
 #pragma unroll
           for (int g = 0; g < NG; ++g) n += __popc(word_at(32 * h + k, g));
@@ -247,27 +258,37 @@ __global__ void __launch_bounds__(kSparseWarps * 32, 4) ls_sparse_kernel(const _
     }
     float mapped = 0.0f;
     int ne = 0, nv = 0;
+    constexpr int SB = KS < 8 ? KS : 8;  // slots looked up side by side
 #pragma unroll
-    for (int s = 0; s < KS; ++s) {
-      const int id = set_entry(w, s);
-      float v = 0.0f;
-      if (map && id >= 0) {
-        int lo = 0, hi = 32 * KS;  // first position with sid >= id
-        while (lo < hi) {
-          const int mid = (lo + hi) >> 1;
-          if (sid[mid] < id) lo = mid + 1;
-          else hi = mid;
-        }
-        if (lo < 32 * KS && sid[lo] == id) {
-          v = sval[lo];
-          mapped += v;
-        } else {
-          v = fill;
-          ++ne;
-        }
+    for (int s0 = 0; s0 < KS; s0 += SB) {
+      int id[SB], pos[SB];  // pos: entries of the old set below id (at most 32 KS - 1 counted)
+#pragma unroll
+      for (int q = 0; q < SB; ++q) {
+        id[q] = set_entry(w, s0 + q);
+        pos[q] = 0;
       }
-      nv += id >= 0;
-      X(s) = v;
+      if (map) {
+#pragma unroll 1
+        for (int step = KS == 48 ? 1024 : 16 * KS; step > 0; step >>= 1)
+#pragma unroll
+          for (int q = 0; q < SB; ++q)
+            if ((KS != 48 || pos[q] + step < 32 * KS) && sid[pos[q] + step - 1] < id[q]) pos[q] += step;
+      }
+#pragma unroll
+      for (int q = 0; q < SB; ++q) {
+        float v = 0.0f;
+        if (map && id[q] >= 0) {
+          if (sid[pos[q]] == id[q]) {
+            v = sval[pos[q]];
+            mapped += v;
+          } else {
+            v = fill;
+            ++ne;
+          }
+        }
+        nv += id[q] >= 0;
+        X(s0 + q) = v;
+      }
     }
     __syncwarp();
     cur_w = w;
