@@ -235,9 +235,9 @@ void keep_faster(const lsk::PropParams& p, Cand* cs, int* nc) {
   if (n) *nc = n;
 }
 
-// Launch plan of p (null: any call up to N = 20480) for targets [t_begin, t_begin + t_count): full waves of the best variant, then the
-// remainder with the variant best for it when that is cheaper.  At most two launches; no heap use
-// (the allocation-free pipeline plans with it too).
+// Launch plan of p (null: any call up to N = 20480) for targets [t_begin, t_begin + t_count): full waves of the
+// best variant, then the remainder with the variant best for it when that is cheaper.  At most two launches; no
+// heap use (the allocation-free pipeline plans with it too).
 int plan(ls_ctx* c, const lsk::PropParams* p, int t_begin, int t_count, Launch* out, int* nout) {
   *nout = 0;
   Cand cs[kMaxCand];
@@ -1135,7 +1135,7 @@ int ls_distance(ls_ctx* ctx, const ls_table* fwd, const ls_table* bck, float* d_
 
 // Small data sets leave most of the GPU idle and are bound by the latency of a locus, so ls_run_all runs
 // their two directions side by side: where each is one launch and all CTAs of both are resident at once
-// (one-warp and 8-target CTAs: N up to 1216).  The backward then leaves t 2^100 at the decode loci in
+// (one-warp and 8-target CTAs: N up to 1216 on 152 SMs).  The backward then leaves t 2^100 at the decode loci in
 // scratch of the call (at most kPairBytes) and the decode forms the product alpha (t 2^100) that it otherwise
 // finds.  Not while profiling (the phases are timed one after the other), with LS_TAIL_OVERLAP=0, in a
 // captured call, or where the scratch cannot be had.  Calls in flight at the same time on other streams follow
@@ -1220,6 +1220,14 @@ int ls_run_all(ls_ctx* ctx, const int32_t* decode_loci, int32_t D, float* d_out,
   CUDA_TRY(cudaMemsetAsync(stat, 0, sizeof(uint32_t) * N, s));
   if ((rc = pair.prepare(D))) return rc;
   const bool both = pair.both;  // the directions side by side
+  if (both && D > 0) {
+    // the backward multiplies what it finds at the decode loci by t 2^100.  Ahead of both directions, whose CTAs
+    // would otherwise go where this kernel leaves room (L = 600, N = 600 / 912
+    // with 16 decode loci: 440 / 472 us behind the fork, 352 / 483 behind the forward's launch, 345 / 436 here)
+    const long long n = (long long)D * N * N;
+    lsk::fill_kernel<<<(unsigned)std::min<long long>((n + 1023) / 1024, 4096), 256, 0, s>>>(pair.t, n, 1.0f);
+    CUDA_TRY(cudaGetLastError());
+  }
   if (both && (rc = pair.fork())) return rc;
   cudaStream_t sb = both ? ctx->side : s;  // the backward's stream
   if (prof) CUDA_TRY(cudaEventRecord(ctx->ev[0], s));
@@ -1241,13 +1249,6 @@ int ls_run_all(ls_ctx* ctx, const int32_t* decode_loci, int32_t D, float* d_out,
   p.store = dd;
   if ((rc = run_launches(ctx, p, 0, N, s, &ctx->launches[0]))) return rc;
   if (prof) CUDA_TRY(cudaEventRecord(ctx->ev[1], s));
-  if (both && D > 0) {
-    // the backward multiplies what it finds at the decode loci by t 2^100.  Behind the forward's launch, whose CTAs
-    // would otherwise go where this kernel leaves room (N = 500, L = 500, 64 decode loci: 600 against 480 us)
-    const long long n = (long long)D * N * N;
-    lsk::fill_kernel<<<(unsigned)std::min<long long>((n + 1023) / 1024, 4096), 256, 0, sb>>>(pair.t, n, 1.0f);
-    CUDA_TRY(cudaGetLastError());
-  }
   // backward over all loci: alpha * beta overwrites alpha at the decode loci
   base_params(ctx, p, 1);
   p.l_first = L - 1;
