@@ -380,10 +380,11 @@ int run_row_steps(lsk::PropParams p, int t_begin, int t_count, cudaStream_t s) {
 }
 
 // Posterior rows: DEC 0 grid (rows), DEC 1 grid (N, D).  The row kernel takes buffers on 16-byte boundaries:
-// posteriors up to 64 elements a thread (N = 5000 / 10000 / 20000 / 26000: 100 / 442 / 893 / 1170 -> 64 / 249 /
-// 637 / 902 us), the decode in place up to 20 (N = 2500 / 5000: 25 / 74 -> 16 / 49 us; at N = 10000 both take
-// 0.31 ms, bound by the logarithms), on or off the quad grid (N = 10001: 443 -> 258 us).  The two-pass kernels
-// take the others.
+// posteriors up to 64 elements a thread (N = 5000 / 10000 / 20000 / 26000: 100 / 442 / 893 / 1170 -> 64 / 204 /
+// 637 / 902 us; 20 elements and up to 512 threads as long as they hold a row, against 40 and 256: all targets at
+// N = 5121 / 7000 / 10000 73 / 113 / 204 against 84 / 138 / 257 us), the decode in place up to N = 5120 (N = 2500 /
+// 5000: 25 / 74 -> 16 / 49 us; at N = 10000 both take 0.31 ms, bound by the logarithms), on or off the quad grid.
+// The two-pass kernels take the others.
 template <int DEC, int E4>
 void launch_posterior(const lsk::PostArgs& a, dim3 grid, cudaStream_t s) {
   const int nt = row_threads(a.N, E4);
@@ -395,6 +396,7 @@ int launch_posterior(const lsk::PostArgs& a, dim3 grid, cudaStream_t s) {
   const bool quads = on_quads(a.out, a.alpha, a.beta);
   if (quads && a.N <= 2048) launch_posterior<DEC, 2>(a, grid, s);
   else if (quads && a.N <= 5120) launch_posterior<DEC, 5>(a, grid, s);
+  else if (!DEC && quads && (a.N <= lsk::kRowMidPostN || a.N == lsk::kRowMidPostN + 3)) launch_posterior<0, 5>(a, grid, s);
   else if (DEC) lsk::decode_kernel<<<grid, 256, 0, s>>>(a.out, a.beta, a.N, a.bits, a.row_words, a.thm, a.thx, a.dl);
   else if (quads && (a.N <= lsk::kRowMaxN || a.N == lsk::kRowMaxN + 3)) launch_posterior<0, 10>(a, grid, s);
   else if (quads && (a.N <= lsk::kRowMaxPostN || a.N == lsk::kRowMaxPostN + 3)) launch_posterior<0, 16>(a, grid, s);

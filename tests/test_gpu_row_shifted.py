@@ -1,5 +1,5 @@
 """Rows that start off a 16-byte boundary (N not a multiple of four) at the limits of every row kernel that takes
-them: posteriors of caller-held rows against float64, decoded distances against the FP64 oracle."""
+them (and next to them): posteriors of caller-held rows against float64, decoded distances against the FP64 oracle."""
 import numpy as np
 import pytest
 
@@ -15,7 +15,7 @@ def ls():
     return m
 
 
-@pytest.mark.parametrize("N", [2045, 2047, 2049, 5118, 5119, 5121, 20477, 20478, 20481, 32765, 32766, 32769])
+@pytest.mark.parametrize("N", [2045, 2047, 2049, 5118, 5119, 5121, 10236, 10237, 10238, 10239, 10240, 10241, 20477, 20478, 20481, 32765, 32766, 32769])
 def test_posterior_rows(ls, N):
     import torch
     T, t0 = 5, N - 5
