@@ -148,8 +148,9 @@ int ls_table_info(const ls_table* t, int32_t* kind, int32_t* locus, int32_t* t_f
 int ls_table_read(const ls_table* t, float* state, double* logscale, ls_stream_t stream);
 
 /* Sizes the propagation calls (ls_forward, ls_backward, ls_checkpoints, ls_run_all and their
- * callers) serve: the uniform prior for N up to 114688 (register-tile kernels to N = 40960, one
- * CTA per target to 57344, two-CTA clusters beyond); a prior matrix up to N = 20480 in either
+ * callers) serve: the uniform prior for N up to 114688 (register-tile kernels to N = 40960;
+ * from 20481 on, and alone beyond 40960, the large-N kernel of one CTA per target to 57344, two-CTA clusters
+ * beyond); a prior matrix up to N = 20480 in either
  * prior format and up to N = 106496 in the BF16 format.  Beyond these the launch planner returns
  * LS_ERR_UNSUPPORTED before anything is enqueued. */
 
@@ -237,12 +238,13 @@ int ls_run_all(ls_ctx* ctx, const int32_t* decode_loci, int32_t D, float* d_out,
  * with respect to a common log-scale of the rho_m of group k.  The paper defines no gradient;
  * this one is the score by the Fisher identity (posterior expectation of the complete-data score
  * of Eq. transition and App. A.3's emission), computed by two forward statistic passes and one
- * backward pass in FP32 with FP64 sums.  Outputs are host doubles (any may be NULL); dlogrho has
- * K entries, 0 for groups without intervals.  Device memory: (3 * (number of nonempty groups) + 2)
- * floats per target and donor, held for the call only (the scratch of this and the other calls
- * that need some comes from a pool per device, which keeps at most 4 GB between calls until the
- * device's last context and network is destroyed); the targets
- * are processed in blocks whose scratch stays within 16 GiB (the environment variable
+ * backward pass in FP32; the expectations' sums over donors are pairs of floats, those over targets and
+ * groups FP64.  Outputs are host doubles (any may be NULL); dlogrho has K entries, 0 for groups without
+ * intervals.  Device memory: (3 * (number of nonempty groups) + 2) floats per target and donor, held for
+ * the call only (up to 4 GB of the scratch of this and the other calls that need some comes from a pool
+ * per device, which keeps at most 4 GB between calls until the device's last context and network is
+ * destroyed, and gives it back where an allocation would fail; the rest is allocated and freed by the
+ * call); the targets are processed in blocks whose scratch stays within 16 GiB (the environment variable
  * LS_GRAD_BUDGET_MB, a positive number of MiB, sets another ceiling; one target is the minimum).
  * Synchronous.  Requires the uniform prior (LS_ERR_UNSUPPORTED otherwise), rho < 1 and mu < 1.
  * Returns LS_WARN_* like ls_run_all. */
@@ -360,7 +362,8 @@ int ls_sparse_run_all(ls_ctx* ctx, const int32_t* idx, int32_t K, int32_t WS, in
  * at zero, and calls whose GPU work overlaps (different streams, or different contexts on one
  * device running at once) race on it.  It launches the propagation kernels that ls_run_all launches (the
  * same planner), one after the other on the caller's stream only; ls_run_all runs the two
- * directions of small data sets (N up to 1216) side by side, with bit-identical results.  N > LS_NOALLOC_MAX_N gives LS_ERR_UNSUPPORTED; D is
+ * directions of small data sets (those whose CTAs for both fit the GPU at once: N up to 1216 on 152 SMs) side by
+ * side, with bit-identical results.  N > LS_NOALLOC_MAX_N gives LS_ERR_UNSUPPORTED; D is
  * limited to 64 as for ls_run_all.  Synchronous when pac_out is given (it waits for the PAC sum and
  * returns LS_WARN_* like ls_run_all), asynchronous otherwise.  A device wait that ran out of time
  * is recorded in the scratch area and reported as LS_ERR_DEVICE by the next call that passes

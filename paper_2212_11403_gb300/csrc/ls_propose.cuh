@@ -47,8 +47,9 @@ __global__ void hapmajor_kernel(const uint32_t* __restrict__ bits, int row_words
 // Mismatch counts of one window, min(popcount, 255) as bytes: M[i*Np + j] (columns up to Np are written).
 // 64 x 64 pairs per block of 256 threads, 4 x 4 per thread with both sides' words in registers; the counts
 // are symmetric, so a block off the diagonal also writes the tile's mirror image and half the blocks have
-// nothing to do.  Bound by the population counts (16 a cycle and SM, eight a pair).  N = 12345: 305 -> 162 us
-// a window (before, every pair counted twice with one 4-byte shared load per word).
+// nothing to do.  Bound by the shared memory (94 % busy: a warp's lanes read rows of B 128 bytes apart, on the same
+// banks), then by the population counts (16 a cycle and SM, eight a pair).  N = 12345: 305 -> 162 us a window
+// (before, every pair counted twice with one 4-byte shared load per word).
 __global__ void __launch_bounds__(256) mismatch_kernel(const uint32_t* __restrict__ hw, int N, int Np, uint8_t* __restrict__ M) {
   if (blockIdx.y > blockIdx.x) return;
   __shared__ __align__(16) uint32_t A[64][8], B[64][8];
@@ -395,7 +396,7 @@ __global__ void __launch_bounds__(256) stage1_hist_kernel(Stage1Args a, int N, i
 // is id order and nothing has to be sorted: the K-th largest score is found by bisection over the 32
 // bits of an order-preserving integer key held in registers (V keys a lane, key v of lane q is
 // candidate 32 v + q), and the selected candidates are compacted in position order by ballots.  It is
-// bound by the compares' integer pipe; no barrier.  12345 targets, C = 1024, K = 512: 988 -> 173 us a
+// bound by the latency of its loads with few warps in flight, then by the compares; no barrier.  12345 targets, C = 1024, K = 512: 988 -> 173 us a
 // window (before: two bitonic sorts in shared memory per target; 246 us without the shared leading
 // bits and the early end).
 template <int V>
