@@ -1140,11 +1140,14 @@ int ls_distance(ls_ctx* ctx, const ls_table* fwd, const ls_table* bck, float* d_
 // (one-warp and 8-target CTAs: N up to 1216 on 152 SMs).  The backward then leaves t 2^100 at the decode loci in
 // scratch of the call (at most kPairBytes) and the decode forms the product alpha (t 2^100) that it otherwise
 // finds.  Not while profiling (the phases are timed one after the other), with LS_TAIL_OVERLAP=0, in a
-// captured call, or where the scratch cannot be had.  Calls in flight at the same time on other streams follow
-// one another on the side stream.
+// captured call, with few loci, or where the scratch cannot be had.  Calls in flight at the same time on other
+// streams follow one another on the side stream.
 // N = 200 / 500 / 1003 / 1200, L = 4000: 2087 / 2175 / 2897 / 3445 -> 1107 / 1262 / 1931 / 2469 us with
 // scratch kept in the context; the call's own costs about 10 us more (N = 200, L = 1000: 371 -> 380).
+// Fewer loci than kPairMinL hide less than the fork, the join and the scratch cost (N = 200, one decode locus, L = 2 /
+// 8 / 24: 49.5 / 52.3 / 55.1 us against 46.6 / 51.4 / 58.5 in turn; N = 33: 48.3 / 49.2 / 53.2 against 45.3 / 49.0 / 56.9).
 static constexpr size_t kPairBytes = (size_t)256 << 20;
+static constexpr int kPairMinL = 8;
 
 struct Pair {  // one call's side-by-side run; the side stream is joined before the scratch goes back
   ls_ctx* c;
@@ -1156,7 +1159,7 @@ struct Pair {  // one call's side-by-side run; the side stream is joined before 
   int prepare(int D) {
     const char* ov = getenv("LS_TAIL_OVERLAP");
     const size_t n = (size_t)D * c->N * c->N;
-    if (c->profile || (ov && ov[0] == '0') || sizeof(float) * n > kPairBytes) return LS_OK;
+    if (c->L < kPairMinL || c->profile || (ov && ov[0] == '0') || sizeof(float) * n > kPairBytes) return LS_OK;
     Launch lp[2];
     int nlp = 0, rc = plan(c, nullptr, 0, c->N, lp, &nlp);
     if (rc) return rc;
