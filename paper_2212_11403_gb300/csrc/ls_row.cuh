@@ -173,7 +173,8 @@ __global__ void __launch_bounds__(kRowMaxThreads, E4 == 5 ? 2 : 0) row_steps_ker
 // pass left in out at D decode loci ([D][N][N], row i = recipient i), t = theta beta, are divided by their
 // emission theta^l (1 - mu where the donor carries the target's allele at l, mu elsewhere; a zero theta
 // means alpha = 0 too, and the entry is 0) and replaced by half distances.  A zero normaliser gives p =
-// eps for every donor (Sec. 2.2); the target's own entry is 0.  Bound by memory (posteriors at N = 10000: 204 us, 5.9 TB/s; before, with the
+// eps for every donor (Sec. 2.2); the target's own entry is 0.  Bound by memory (posteriors at N = 10000: 204 us,
+// 5.9 TB/s; before, with the
 // rows read twice, 442 us) and, with distances, by the logarithms too.
 struct PostArgs {
   const float *alpha, *beta;  // DEC 0; DEC 1: null and, where out holds alpha alone, the backward's t 2^100
