@@ -73,25 +73,26 @@ struct RowQuads {
 // element by element; a table moved by one locus is all load and save, so this kernel takes calls of
 // few steps.  N = 10000, one locus forward / backward: 658 / 520 -> 158 / 186 us (0.8 GB moved, 75 / 63 % of
 // the measured copy rate); the two reductions between load and save are what keeps it from the rest.
-// 20 elements a thread get 64 registers, four CTAs of 256 threads an SM; with the 98 the compiler would take, two
-// (tables of N = 5001 moved by 1 / 8 loci: 109 / 244 against 87 / 193 us).
 template <int DIR, int E4, bool SHIFT>
-__global__ void __launch_bounds__(kRowMaxThreads, E4 == 5 ? 2 : 0) row_steps_kernel(const PropParams p) {
+__global__ void __launch_bounds__(kRowMaxThreads) row_steps_kernel(const PropParams p) {
   __shared__ float buf[2][32];
   const int N = p.N, i = p.t_begin + blockIdx.x, row = i - p.tab_t0;
   float* state = p.state + (size_t)row * N;
   const RowQuads<SHIFT> P(N, state);
   float x[E4][4];
   int ph = 0;
-  // four sums of a thread's elements: in one, forty additions round the same way in every thread of an even row
-  // (N = 10000, four single steps: relative error of alpha 1.8e-7 against 9.6e-8 of the register-tile kernel)
-  auto total = [&](const float (&s)[4]) {
+  // forty elements of a thread are summed in four parts: in one, the additions round the same way in every thread of an
+  // even row (N = 10000, four single steps: relative error of alpha 1.8e-7 against 9.6e-8 of the register-tile kernel;
+  // now 6.9e-8).  Up to twenty, one sum is no further off than that kernel's (N = 2100 to 5117: 1.1e-7 against 1.3e-7)
+  constexpr int PARTS = E4 <= 5 ? 1 : 4;
+  auto total = [&](const float (&s)[PARTS]) {
     ph ^= 1;
-    return row_sum((s[0] + s[1]) + (s[2] + s[3]), buf[ph]);
+    if constexpr (PARTS == 4) return row_sum((s[0] + s[1]) + (s[2] + s[3]), buf[ph]);
+    else return row_sum(s[0], buf[ph]);
   };
   float sig_prev = 1.0f;
   {
-    float s[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    float s[PARTS] = {};
 #pragma unroll
     for (int e = 0; e < E4; ++e) {
       const int pos = P.at(e);
@@ -99,7 +100,7 @@ __global__ void __launch_bounds__(kRowMaxThreads, E4 == 5 ? 2 : 0) row_steps_ker
       for (int k = 0; k < 4; ++k) x[e][k] = 0.0f;
       if (p.load_state && pos < N) P.load(state, pos, x[e]);
 #pragma unroll
-      for (int k = 0; k < 4; ++k) s[k] += x[e][k];
+      for (int k = 0; k < 4; ++k) s[k % PARTS] += x[e][k];
     }
     if (p.load_state && DIR == 0) sig_prev = total(s);
   }
@@ -128,7 +129,7 @@ __global__ void __launch_bounds__(kRowMaxThreads, E4 == 5 ? 2 : 0) row_steps_ker
     const uint32_t* bits = p.bits2 + (size_t)l * p.rw2;
     const uint32_t inv = (bits[i >> 5] >> (i & 31)) & 1u ? 0u : 0xffffffffu;  // match = bit ^ inv
     const float tm = p.thm[l], tx = p.thx[l];
-    float s[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    float s[PARTS] = {};
 #pragma unroll
     for (int e = 0; e < E4; ++e) {
       const int pos = P.at(e);
@@ -139,7 +140,7 @@ __global__ void __launch_bounds__(kRowMaxThreads, E4 == 5 ? 2 : 0) row_steps_ker
         for (int k = 0; k < 4; ++k) {
           b[k] = pos + k == i || !P.in(pos + k) ? 0.0f : fmaf(c, x[e][k], r);  // alpha before its emission, or beta
           x[e][k] = ((w >> k) & 1u ? tm : tx) * b[k];
-          s[k] += x[e][k];
+          s[k % PARTS] += x[e][k];
         }
         const float(&v)[4] = DIR == 0 ? x[e] : b;
         if (out && SHIFT) {  // a stored row need not lie on the boundaries of the table's
@@ -174,8 +175,7 @@ __global__ void __launch_bounds__(kRowMaxThreads, E4 == 5 ? 2 : 0) row_steps_ker
 // emission theta^l (1 - mu where the donor carries the target's allele at l, mu elsewhere; a zero theta
 // means alpha = 0 too, and the entry is 0) and replaced by half distances.  A zero normaliser gives p =
 // eps for every donor (Sec. 2.2); the target's own entry is 0.  Bound by memory (posteriors at N = 10000: 204 us,
-// 5.9 TB/s; before, with the
-// rows read twice, 442 us) and, with distances, by the logarithms too.
+// 5.9 TB/s; before, with the rows read twice, 442 us) and, with distances, by the logarithms too.
 struct PostArgs {
   const float *alpha, *beta;  // DEC 0; DEC 1: null and, where out holds alpha alone, the backward's t 2^100
   float* out;
